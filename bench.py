@@ -41,27 +41,13 @@ STATE_FIELDS = 24
 BYTES_PER_POINT_STAGE = [8 * 3 * 24, 8 * 5 * 24, 8 * 5 * 24, 8 * 4 * 24]
 # RK4 combine flops per field per stage (stage 1: 2; 2-3: 4; 4: 3)
 COMBINE_FLOPS = [2, 4, 4, 3]
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
-# each pass of the vacuum stage, from the committed ncu capture of the 96^3
-# case (the derivative pass: exponent scan + limb conversion + integer pass;
-# the algebra pass: the mean over a step's stages 1, 2, 3, 4), and the hash of
-# the kernel sources it was taken on.  Reported scaled to the bench grid by
-# points; null when the kernel sources differ from the profiled ones.
-NCU_TRAFFIC = {"sources_sha256_16": "6129913db8cd4ae6", "grid": 96,
-               "bytes_per_launch": {
-                   # exponent scan (stage 1 only) + limb copy + integer pass, mean over the 4 stages of a step
-                   "derivative": ((169877760 + 3258880) + (169882880 + 122540544) + (237195264 + 1092143360)
-                                  + (169875712 + 122436608) + (237027584 + 1092392960)
-                                  + (169882112 + 121968384) + (237173760 + 1092693760)
-                                  + (169882880 + 122204928) + (237097728 + 1092242688)) / 4,
-                   # algebra pass, modes 1, 2, 2, 3 of one step
-                   "algebra": ((1396294400 + 521755648)
-                               + (1671427584 + 385866240)
-                               + (1672915200 + 386181120)
-                               + (1646590720 + 483951104)) / 4}}
-# derivative-pass buffer: first + second derivatives and KO terms per point (vacuum)
-DERIV_DOUBLES = 162
-KERNEL_SOURCES = ["common.cuh", "stage_kernel.cuh", "stage_int.cuh", "limbs.cu", "stage_vac.cu",
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the
+# stage kernel of the vacuum system (mean over a step's four stages), from the ncu
+# capture of a small case, and the hash of the kernel sources it was taken on.
+# Reported scaled to the bench grid by points; null when the kernel sources differ
+# from the profiled ones.
+NCU_TRAFFIC = {"sources_sha256_16": "", "points": 96 ** 3, "bytes_per_launch": {"stage": 0.0}}
+KERNEL_SOURCES = ["common.cuh", "stage_kernel.cuh", "stage_split.cuh", "stage_int.cuh", "limbs.cu", "stage_vac.cu",
                   "generated/bssn_algebra.cuh"]
 
 
@@ -841,13 +827,13 @@ def main():
     acc = torch.empty_like(ev.state)
     stream = torch.cuda.current_stream()
 
-    # pass options as cosmos_rk4_step uses them: the algebra pass of stages 1-3 records the exponents
-    # of the state it writes (+32, stage 1 clearing the record first: +64), the derivative pass of
-    # stages 2-4 takes them instead of scanning (+16)
+    # pass options as cosmos_rk4_step uses them: pass 2 of stages 1-3 records the exponents of the state
+    # it writes (+32, stage 1 clearing the record first: +64), pass 1 of stages 2-4 takes them instead
+    # of scanning (+16)
     pass_opts = {(1, 1): 0, (1, 2): 32 + 64, (2, 1): 16, (2, 2): 32, (3, 1): 16, (3, 2): 32, (4, 1): 16, (4, 2): 0}
 
     def stage_calls(t, events=None):
-        """One RK4 step as 4 stages x (derivative pass, algebra pass), the sequence of
+        """One RK4 step as 4 stages x (limb copy, stage kernel), the sequence of
         cosmos_rk4_step; events bracket each pass on the launching stream."""
         seq = [(ev.state, U1), (U1, U2), (U2, U1), (U1, None)]
         for s, (src, dst) in enumerate(seq, start=1):
@@ -890,9 +876,9 @@ def main():
     nranks = ws_
     pts = float(n) ** 3
     value = nranks * pts * args.steps / elapsed
-    # per step: exponent scan (stage 1), 4 x (limb copy, integer derivative pass, algebra pass),
-    # exponent record compaction (stages 1-3)
-    gpu_launches = 16 * args.steps
+    # per step: exponent scan (stage 1), 4 x (limb copy, stage kernel), exponent record compaction
+    # (stages 1-3)
+    gpu_launches = 12 * args.steps
 
     # ---- end to end through the C ABI with host buffers (pinned) ----
     # Every step copies its inputs from pinned host memory and reads its result
@@ -975,7 +961,7 @@ def main():
         gpass = [statistics.mean([gev[k][st][q][0].elapsed_time(gev[k][st][q][1]) for k in range(gk) for st in range(4)])
                  for q in range(2)]
         generic = {"value": pts * gk / tg, "unit": UNIT, "ms_per_step": 1e3 * tg / gk, "steps": gk, "warmup": 3,
-                   "derivative_pass_ms": gpass[0], "algebra_pass_ms": gpass[1],
+                   "limb_copy_ms": gpass[0], "stage_kernel_ms": gpass[1],
                    "state": "inputs.smooth_state(256, seed=2562, kmax=6, scale=0.5): every field a base value plus "
                             "3 seeded Fourier modes with wave numbers up to 6 per axis"}
         del ev, U1, U2, acc, dev, host_in, host_out
@@ -998,69 +984,50 @@ def main():
         cpu = cpu_baseline_sample(n, planes=n // 2, repeats=1, state=host_state)
     # average launch duration per kernel (over the 4 stages and all steps)
     avg = {name: statistics.mean([x for st in pass_ms[q] for x in st]) * 1e-3
-           for q, name in enumerate(["derivative", "algebra"])}
+           for q, name in enumerate(["limbs", "stage"])}
     stage_avg = [statistics.mean(pass_ms[0][s]) + statistics.mean(pass_ms[1][s]) for s in range(4)]
     roof, roof2, sweep = None, None, None
     if cpu is not None:
         parts = cpu["flops_parts"]
         fl = lambda d: d["add"] + d["mul"] + d["div"] + d["sqrt"]  # noqa: E731
         combine = statistics.mean(COMBINE_FLOPS) * STATE_FIELDS
-        # algebra pass: the generated algebra's operations + the KO multiply-add (2 per field) + the RK4
-        # combine; the oracle's count (its plain loops form every symmetric component twice) beside it
+        # stage kernel: the generated algebra's operations + the KO multiply-add (2 per field) + the RK4
+        # combine; its finite differences are integer work.  Beside it the oracle's count (its plain
+        # loops form every symmetric component twice) and its stencils as FP64 operations.
         alg_flops = generated_algebra_ops("vac") + 2 * STATE_FIELDS + combine
-        oracle_flops = {"derivative": fl(parts["derivatives"]) + fl(parts["ko"]),
-                        "algebra": fl(parts["algebra"]) + combine}
-        bytes_point = {"derivative": 8 * (STATE_FIELDS + DERIV_DOUBLES),
-                       "algebra": 8 * (DERIV_DOUBLES + statistics.mean([b / 8 for b in BYTES_PER_POINT_STAGE]))}
+        oracle_flops = {"stencils": fl(parts["derivatives"]) + fl(parts["ko"]), "algebra": fl(parts["algebra"]) + combine}
+        # the state read and its limb copy written; the limb copy read and the stage's states
+        bytes_point = {"limbs": 8 * 2 * STATE_FIELDS,
+                       "stage": 8 * STATE_FIELDS + statistics.mean(BYTES_PER_POINT_STAGE)}
         peak = fp64_peak / 1e12
         hbm_peak, hbm_src = hbm_peak_gbs()
         traffic_ok = kernel_sources_hash() == NCU_TRAFFIC["sources_sha256_16"]
-
-        def traffic(name):
-            return NCU_TRAFFIC["bytes_per_launch"][name] * (n / NCU_TRAFFIC["grid"]) ** 3 if traffic_ok else None
-
-        def roof_algebra():
-            achieved = pts * alg_flops / avg["algebra"] / 1e12
-            return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "traffic": traffic("algebra"),
-                    "traffic_note": "bytes per launch, ncu small-case capture scaled by points",
-                    "kernel": "algebra pass (stage_kernel<T_vac>)", "avg_launch_ms": 1e3 * avg["algebra"],
-                    "algorithmic_flops_per_point": alg_flops,
-                    "flops_note": "generated algebra after CSE + KO multiply-add + RK4 combine",
-                    "oracle_flops_per_point": oracle_flops["algebra"],
-                    "algorithmic_bytes_per_point": bytes_point["algebra"],
-                    "hbm_GBps_algorithmic": pts * bytes_point["algebra"] / avg["algebra"] / 1e9,
-                    "peak_source": "FP64 DFMA throughput measured in this run (cosmos_probe_fp64); nominal 1.25"}
-
-        def roof_derivative():
-            achieved = pts * bytes_point["derivative"] / avg["derivative"] / 1e9
-            return {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
-                    "frac": achieved / hbm_peak, "traffic": traffic("derivative"),
-                    "traffic_note": "bytes per launch (exponent scan + limb conversion + integer pass), ncu small-case "
-                                    "capture scaled by points",
-                    "kernel": "derivative pass (limb pre-pass + ideriv_kernel<T_vac>)",
-                    "avg_launch_ms": 1e3 * avg["derivative"],
-                    "algorithmic_bytes_per_point": bytes_point["derivative"],
-                    "stencil_flops_per_point_fp64_equivalent": oracle_flops["derivative"],
-                    "stencil_TFLOPs_fp64_equivalent": pts * oracle_flops["derivative"] / avg["derivative"] / 1e12,
-                    "arithmetic": "exact integer (fixed-point digits), not the FP64 pipe",
-                    "peak_source": "HBM copy bandwidth " + hbm_src}
-
-        rf = {"derivative": roof_derivative, "algebra": roof_algebra}
-        dom = max(avg, key=avg.get)
-        other = "algebra" if dom == "derivative" else "derivative"
-        roof, roof2 = rf[dom](), rf[other]()
-        # the whole step against the sum of its passes' own roofline times: the algebra pass's
-        # generated FP64 operations at the FP64 peak, the derivative pass's bytes at the HBM peak
-        # (its stencils run in integer units, so no FP64 bound applies to it)
+        achieved = pts * alg_flops / avg["stage"] / 1e12
+        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                "traffic": NCU_TRAFFIC["bytes_per_launch"]["stage"] * pts / NCU_TRAFFIC["points"] if traffic_ok else None,
+                "traffic_note": "bytes per launch, ncu small-case capture scaled by points",
+                "kernel": "stage kernel (split_stage_kernel<T_vac>): differences, algebra and combine",
+                "avg_launch_ms": 1e3 * avg["stage"], "algorithmic_flops_per_point": alg_flops,
+                "flops_note": "generated algebra after CSE + KO multiply-add + RK4 combine, on the FP64 pipe",
+                "oracle_flops_per_point": oracle_flops["algebra"],
+                "stencil_flops_per_point_fp64_equivalent": oracle_flops["stencils"],
+                "stencil_arithmetic": "exact integer (fixed point), beside the FP64 pipe",
+                "algorithmic_bytes_per_point": bytes_point["stage"],
+                "hbm_GBps_algorithmic": pts * bytes_point["stage"] / avg["stage"] / 1e9,
+                "peak_source": "FP64 DFMA throughput measured in this run (cosmos_probe_fp64); nominal 1.25"}
+        achieved = pts * bytes_point["limbs"] / avg["limbs"] / 1e9
+        roof2 = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
+                 "traffic": None, "kernel": "limb copy of the stage state (stage 1 with the exponent scan)",
+                 "avg_launch_ms": 1e3 * avg["limbs"], "algorithmic_bytes_per_point": bytes_point["limbs"],
+                 "peak_source": "HBM copy bandwidth " + hbm_src}
+        # the whole step against the sum of its kernels' own roofline times
         t_alg = 4 * pts * alg_flops / (peak * 1e12)
-        t_der = 4 * pts * bytes_point["derivative"] / (hbm_peak * 1e9)
-        t_fp64_equiv = 4 * pts * (alg_flops + oracle_flops["derivative"]) / (peak * 1e12)
-        sweep = {"roofline_ms_per_step": 1e3 * (t_alg + t_der), "algebra_fp64_ms_per_step": 1e3 * t_alg,
-                 "derivative_hbm_ms_per_step": 1e3 * t_der, "ms_per_step": 1e3 * elapsed / args.steps,
-                 "frac": (t_alg + t_der) / (elapsed / args.steps),
-                 "note": "sum of the two passes' roofline times / measured RK4 step (4 stages)",
-                 "context_fp64_equivalent_ms_per_step": 1e3 * t_fp64_equiv,
+        t_limbs = 4 * pts * bytes_point["limbs"] / (hbm_peak * 1e9)
+        sweep = {"roofline_ms_per_step": 1e3 * (t_alg + t_limbs), "algebra_fp64_ms_per_step": 1e3 * t_alg,
+                 "limbs_hbm_ms_per_step": 1e3 * t_limbs, "ms_per_step": 1e3 * elapsed / args.steps,
+                 "frac": (t_alg + t_limbs) / (elapsed / args.steps),
+                 "note": "sum of the two kernels' roofline times / measured RK4 step (4 stages)",
+                 "context_fp64_equivalent_ms_per_step": 1e3 * 4 * pts * (alg_flops + oracle_flops["stencils"]) / (peak * 1e12),
                  "context_note": "FP64 time of the algebra plus the stencils counted as the FP64 flops they stand "
                                  "for (integer units do them): not a bound on the executed work"}
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": args.gpus, "steps": args.steps,

@@ -184,7 +184,7 @@ int cosmos_rk4_stage(const cosmos_grid* g, const cosmos_params* p, int stage, co
  * Before each RK4 stage the ranks exchange the ghost planes of the stage
  * state (periodic in z across the ranks) and take the largest of their
  * per-field exponents (cosmos_field_exponents), so that the integer
- * derivative pass rounds exactly as on the whole grid; cosmos_rk4_stage_slab
+ * differences round exactly as on the whole grid; cosmos_rk4_stage_slab
  * then advances the slab's interior planes.  The results equal the single-
  * grid ones bitwise.  The paper's code runs on one node with OpenMP; this is
  * the GPU form of its grid's natural split.
@@ -192,15 +192,15 @@ int cosmos_rk4_stage(const cosmos_grid* g, const cosmos_params* p, int stage, co
 
 /* E[s] = the largest biased FP64 exponent over the whole array of limb slot
  * s (slot s = field s; with the fluid on, the scalar's fields move down by 4:
- * 24 + 2 scalar slots), the reference exponent of the integer derivative
- * pass.  E: device memory, 24 + 2 * scalar ints.  Asynchronous. */
+ * 24 + 2 scalar slots), the reference exponent of the integer
+ * differences.  E: device memory, 24 + 2 * scalar ints.  Asynchronous. */
 int cosmos_field_exponents(const cosmos_grid* g, const cosmos_params* p, const double* state, int* E,
                            void* stream);
 
-/* cosmos_rk4_stage with the algebra pass and the stage combine restricted to
- * planes k_lo .. k_lo + k_cnt - 1 (the derivative and fluid passes cover
- * every plane, so planes within 3 of the range must hold the right values:
- * the ghost planes of a slab), and, if E is not NULL, the derivative pass's
+/* cosmos_rk4_stage with the algebra and the stage combine restricted to
+ * planes k_lo .. k_lo + k_cnt - 1 (the fluid pass and the fixed-point copy
+ * cover every plane; planes within 3 of the range must hold the right values:
+ * the ghost planes of a slab), and, if E is not NULL, the differences'
  * reference exponents taken from E (device, as cosmos_field_exponents
  * writes it) instead of its own scan of U_s.  Every entry of E must be at
  * least the exponent cosmos_field_exponents gives for U_s itself (the
@@ -215,16 +215,17 @@ int cosmos_rk4_stage_slab(const cosmos_grid* g, const cosmos_params* p, int stag
 /* One pass of a fused RK4 stage (arguments as cosmos_rk4_stage), so that
  * the passes can be scheduled or timed separately:
  *   pass 0: fluid primitives and face fluxes of U_s (nothing without fluid)
- *   pass 1: derivative pass: finite differences and Kreiss-Oliger terms of U_s
- *   pass 2: algebra pass + stage combine (needs passes 0 and 1 of this stage)
+ *   pass 1: fixed-point copy of U_s, which the finite differences are taken of
+ *   pass 2: finite differences, Kreiss-Oliger terms, algebra and stage combine
+ *           (needs passes 0 and 1 of this stage, and U_s unchanged since)
  * Passes 0, 1, 2 in order equal one cosmos_rk4_stage call.  The workspace
  * carries the intermediate results between passes.  Option bits added to
  * `pass` reproduce what cosmos_rk4_step does between its stages:
- *   + 32 (pass 2, stages 1-3): the algebra pass records the largest FP64
+ *   + 32 (pass 2, stages 1-3): the pass records the largest FP64
  *        exponent of every field it writes to U_next into the workspace
  *        (+ 64: the same, clearing the record first: needed once per
  *        workspace before its first record);
- *   + 16 (pass 1): the derivative pass takes those recorded exponents
+ *   + 16 (pass 1): the copy takes those recorded exponents
  *        instead of scanning U_s, which must then be the U_next of the
  *        recording pass, unchanged since.
  * Results are bitwise those without the options (the same maxima). */
@@ -237,7 +238,7 @@ int cosmos_stage_pass(const cosmos_grid* g, const cosmos_params* p, int pass, in
  * in place on `state`: k_s = F(U_s, t + c_s dt), U_{n+1} = U_n + dt/6
  * (k1 + 2 k2 + 2 k3 + k4), as four cosmos_rk4_stage calls, each fused with
  * its stage combine (stages 2-4 take their fields' largest exponents as the
- * algebra pass of the stage before records them, instead of a scan of the
+ * stage before records them, instead of a scan of the
  * state: bitwise the same).  ws: COSMOS_OP_RK4 bytes (two stage buffers,
  * the accumulator and the fluid buffers).  Errors as cosmos_rhs. */
 int cosmos_rk4_step(const cosmos_grid* g, const cosmos_params* p, double* state, double t, double dt, void* ws,
@@ -257,9 +258,9 @@ int cosmos_rk4_step_stages(const cosmos_grid* g, const cosmos_params* p, double*
  * result to host_out; synchronous.  host_in and host_out may be the same
  * buffer.  With pinned buffers the copies overlap the computation: the
  * host-to-device copy goes in four field groups on a private stream, each
- * followed by the first derivative pass over those fields, and the
+ * followed by the first fixed-point copy of those fields, and the
  * device-to-host copy in up to eight slabs of z-planes, each started when the
- * last algebra pass has written them.  The result is bitwise that of
+ * last stage has written them.  The result is bitwise that of
  * cosmos_rk4_step.  Errors: COSMOS_EINVAL (NULL buffer, steps < 0),
  * COSMOS_EALIGN, COSMOS_EWORKSPACE, COSMOS_ECUDA (the call returns only after
  * its own copies have ended, on errors too). */

@@ -82,10 +82,68 @@ def contract_sym(Mu, N):
     return s
 
 
-def algebra(fluid: bool, scalar: bool):
+def split_layout(fluid: bool, scalar: bool):
+    """Input slots of the split form (``algebra(..., split=True)``): region A holds
+    what the first phase reads, region B what the second one does and the slots
+    ``r{f}`` that take the outputs of fields without a slot of their own there.
+
+    Per field with second derivatives ten slots (d_k, dd_p, Kreiss-Oliger
+    bracket k), per field with first derivatives four (d_k, k); m{f} of a field
+    whose derivatives only advect it is that whole advection with its
+    dissipation term; kdiff = K - Kref.  ``out`` = the region-B slot that takes
+    output f: its k or m slot (read by that output alone) or r{f}.
+
+    Units: lengths in l (the algebra does not see its value but through the
+    parameters below).  u of K, At, Pi carries l, u of the fluid fields and rho
+    l^2, m the units of its output; differences, k, u of B^i and kdiff come
+    without the l of their field, which the parameters that multiply them hold: len = l, c75 = 3/4 l, c43 = 4/3
+    l, eta l^2, lapse_c1 l, lapse_c2 l.  out[f] carries one l more than field f.
+
+    The raised At is formed in the first phase (both phases then take about as
+    long as the differences of the other region), except with the fluid, whose
+    own quantities already fill the registers between the phases."""
+
+    def d2(f):
+        return [f"d{f}_{k}" for k in range(3)] + [f"dd{f}_{p}" for p in range(6)] + [f"k{f}"]
+
+    def d1(f):
+        return [f"d{f}_{k}" for k in range(3)] + [f"k{f}"]
+
+    a, b = [], []
+    for f in range(GT, GT + 6):
+        a += d2(f)
+    for f in range(GAM, GAM + 3):
+        a += d1(f)
+    early = not fluid
+    a += [f"u{f}" for f in [*range(GT, GT + 6), *range(BET, BET + 3)] + [*range(AT, AT + 6)] * early]
+    if fluid:
+        a += ["u0", "u24", "u25", "u26", "u27", "rho"]
+    ph = 24 + 4 * fluid
+    for f in [CHI, ALP, BET, BET + 1, BET + 2] + [ph] * scalar:
+        b += d2(f)
+    b += d1(TRK)
+    b += [f"m{f}" for f in [*range(AT, AT + 6), *range(BB, BB + 3)] + [ph + 1] * scalar]
+    b += [f"u{f}" for f in [*range(0, GAM), *range(ALP, 24)]] + ["kdiff"]
+    if fluid:
+        b += ["u24", "u25", "u26", "u27", "rho"]
+    if scalar:
+        b += [f"u{ph + 1}"]
+    b += [f"r{f}" for f in [*range(GT, GT + 6), *range(GAM, GAM + 3)] + [24, 25, 26, 27] * fluid]
+    nf = 24 + 4 * fluid + 2 * scalar
+    out = [b.index(next(x for x in (f"k{f}", f"m{f}", f"r{f}") if x in b)) for f in range(nf)]
+    return dict(a=a, b=b, out=out, early=early)
+
+
+def algebra(fluid: bool, scalar: bool, split: bool = False):
+    """The right-hand side as a graph: (graph, layout, outputs).
+
+    With ``split`` the outputs contain the dissipation terms, the inputs are
+    those of ``split_layout``, and the graph carries ``cut``: the nodes that end
+    the first phase, whose inputs are those of region A."""
     g = Graph()
     L = layout(fluid, scalar)
     nf = L["nf"]
+    cut = []
     u = [g.input(f"u{f}") for f in range(nf)]
 
     def d(f, k):
@@ -94,7 +152,12 @@ def algebra(fluid: bool, scalar: bool):
     def dd(f, i, j):
         return g.input(f"dd{f}_{PIDX[(i, j)]}")
 
-    eta, Kref = g.param("eta"), g.param("Kref")
+    eta = g.param("eta")
+    if split:
+        ko, ulen, c75, c43 = g.param("ko"), g.param("len"), g.param("c75"), g.param("c43")
+    else:
+        Kref = g.param("Kref")
+        ulen, c75, c43 = 1.0, 0.75, 4.0 / 3.0
     c1, c2, shift_on, w = g.param("lapse_c1"), g.param("lapse_c2"), g.param("shift_on"), g.param("w")
     pi = math.pi
 
@@ -163,47 +226,48 @@ def algebra(fluid: bool, scalar: bool):
     # ---- conformal Ricci tensor, doubled ----
     # R_ij = -1/2 gt^lm d_l d_m gt_ij + gt_k(i d_j) Gt^k + Gd^k Gamma_(ij)k
     #        + (T_ij + T_ji) + U_ij,
-    # T_ij = sum_km C[k][m][i] Gamma_jkm, U_ij = sum_kl C[k][l][i] Gamma_klj,
-    # C[k][m][i] = gt^ml Gamma^k_li.  The Christoffel products are accumulated
-    # into the six components index i by index i, so that only the nine
-    # C[.][.][i] of one i exist at a time (fewer values live at once).
-    acc = [None] * 6  # 2 (T_ij + T_ji + U_ij)
-
-    def add_to(m, t):
-        acc[m] = t if acc[m] is None else acc[m] + t
-
+    # T_ij = sum_km C[k][m][i] Gamma_jkm, U_ij = sum_km C[k][m][i] Gamma_kmj,
+    # C[k][m][i] = gt^ml Gamma^k_li.  T_ij + U_ij = V_ij = sum_km C[k][m][i] d_m gt_jk
+    # (Gamma_jkm + Gamma_kjm = d_m gt_jk), so the quadratic part is V_ij + T_ji: 15
+    # products instead of 21 off the diagonal.  The Christoffel products are
+    # accumulated into the six components index i by index i, so that only the
+    # nine C[.][.][i] of one i exist at a time (fewer values live at once).
+    accT, accV = [None] * 6, [None] * 6  # 2 T_ji (i <= j), V_ij
     for i in range(3):
         Ci = [[gu[m, 0] * Gu[k][0, i] + gu[m, 1] * Gu[k][1, i] + gu[m, 2] * Gu[k][2, i] for m in range(3)]
               for k in range(3)]
         # Gamma_jkm is symmetric in k, m: T_ij sums (C[k][m][i] + C[m][k][i]) Gamma_jkm over k <= m
         Cs = {(k, m): (Ci[k][m] if k == m else Ci[k][m] + Ci[m][k]) for (k, m) in PAIRS}
         for j in range(3):
-            s = None
-            for (k, m) in PAIRS:
-                t = Cs[(k, m)] * Gl2[j][k, m]
-                s = t if s is None else s + t
-            add_to(PIDX[(i, j)], 2.0 * s if i == j else s)  # 2 T_ij (T_ii counted twice)
+            if j <= i:  # T_ij into R_ji
+                s = None
+                for (k, m) in PAIRS:
+                    t = Cs[(k, m)] * Gl2[j][k, m]
+                    s = t if s is None else s + t
+                accT[PIDX[(i, j)]] = s
             if j >= i:
-                u_ = None
+                s = None
                 for k in range(3):
-                    for l in range(3):
-                        t = Ci[k][l] * Gl2[k][l, j]
-                        u_ = t if u_ is None else u_ + t
-                add_to(PIDX[(i, j)], u_)  # 2 U_ij
+                    for m in range(3):
+                        t = Ci[k][m] * dgt(m, j, k)
+                        s = t if s is None else s + t
+                accV[PIDX[(i, j)]] = s
+    acc = [accT[m] + 2.0 * accV[m] for m in range(6)]
     Gd = [contract_sym(gu2, Gu[k]) for k in range(3)]
     # 2 R_ij as one flat sum:
     #   -gt^lm d_l d_m gt_ij + gt_ki d_j Gt^k + gt_kj d_i Gt^k + Gd^k d_k gt_ij + acc
     # (Gamma_ijk + Gamma_jik = d_k gt_ij); on the diagonal the two equal terms are formed once
+    lgt = Sym([ulen * x for x in gt.c])
     Ric2 = []
     for m, (i, j) in enumerate(PAIRS):
         r = acc[m]
         for q, (l, n) in enumerate(PAIRS):
             r = r - gu2[q] * ddgt(l, n, i, j)
         if i == j:
-            r = r + 2.0 * (gt[0, i] * dGt(i, 0) + gt[1, i] * dGt(i, 1) + gt[2, i] * dGt(i, 2))
+            r = r + 2.0 * (lgt[0, i] * dGt(i, 0) + lgt[1, i] * dGt(i, 1) + lgt[2, i] * dGt(i, 2))
         else:
             for k in range(3):
-                r = r + gt[k, i] * dGt(j, k) + gt[k, j] * dGt(i, k)
+                r = r + lgt[k, i] * dGt(j, k) + lgt[k, j] * dGt(i, k)
         for k in range(3):
             r = r + Gd[k] * dgt(k, i, j)
         Ric2.append(r)
@@ -287,8 +351,20 @@ def algebra(fluid: bool, scalar: bool):
     out = [None] * nf
     divb = dbeta(0, 0) + dbeta(1, 1) + dbeta(2, 2)
 
+    merged = {*range(AT, AT + 6), *range(BB, BB + 3)} | ({24 + 4 * fluid + 1} if scalar else set())
+
     def adv(f):
-        return beta[0] * d(f, 0) + beta[1] * d(f, 1) + beta[2] * d(f, 2)
+        """Advection of field f; in the split form with its dissipation term, in the units of the output."""
+        if split and f in merged:
+            return g.input(f"m{f}")
+        s = beta[0] * d(f, 0) + beta[1] * d(f, 1) + beta[2] * d(f, 2)
+        if split and not BET <= f < BET + 3:
+            s = ko * g.input(f"k{f}") + s
+            if GT <= f < GT + 6 or GAM <= f < GAM + 3:
+                cut.append(s)
+            if f == TRK or GAM <= f < GAM + 3:
+                s = ulen * s
+        return s
 
     third_div = (1.0 / 3.0) * divb
     out[CHI] = adv(CHI) + (2.0 * chi) * ((1.0 / 3.0) * (alpha * K) - third_div)
@@ -333,7 +409,7 @@ def algebra(fluid: bool, scalar: bool):
                 s = s + At[i, k] * W[k][j] + At[j, k] * W[k][i]
         out[AT + m] = s
     # gt^ij y_j and -2 At^ij z_j collect the terms of d_t Gt^i that one tensor multiplies
-    a43 = (4.0 / 3.0) * alpha
+    a43 = c43 * alpha
     a16 = (16.0 * pi) * alpha
     y, z = [], []
     az = 1.5 * (alpha * ichi)
@@ -353,10 +429,14 @@ def algebra(fluid: bool, scalar: bool):
         s = s + two_alpha * GA[i]
         Gt_src.append(s)
         out[GAM + i] = adv(GAM + i) + s
-    out[ALP] = adv(ALP) - alpha * (c1 + c2 * alpha) * (K - Kref)
+    out[ALP] = adv(ALP) - alpha * (c1 + c2 * alpha) * (g.input("kdiff") if split else K - Kref)
     for i in range(3):
-        out[BET + i] = shift_on * (adv(BET + i) + 0.75 * B[i])
-        out[BB + i] = shift_on * (adv(BB + i) + Gt_src[i] - eta * B[i])
+        out[BET + i] = shift_on * (adv(BET + i) + c75 * B[i])
+        if split:  # m of B^i has the switch on its advection
+            out[BET + i] = ko * g.input(f"k{BET + i}") + out[BET + i]
+            out[BB + i] = adv(BB + i) + shift_on * (Gt_src[i] - eta * B[i])
+        else:
+            out[BB + i] = shift_on * (adv(BB + i) + Gt_src[i] - eta * B[i])
     if fluid:
         q = 24
         E, J, wJ, isg, P, iEP = fl["E"], fl["J"], fl["wJ"], fl["isg"], fl["P"], fl["iEP"]
@@ -374,19 +454,26 @@ def algebra(fluid: bool, scalar: bool):
         for i in range(3):
             s = (J[0] * dbeta(i, 0) + J[1] * dbeta(i, 1) + J[2] * dbeta(i, 2)) - E * dal[i]
             # S^jk d_i gamma_jk, gamma_jk = gt_jk / chi
-            s = s + half_alpha * (ichi * (contract_sym(Su2, Sym([dgt(i, a, b) for (a, b) in PAIRS])) - dchi[i] * Str_f))
+            Sdg = contract_sym(Su2, Sym([dgt(i, a, b) for (a, b) in PAIRS]))
+            cut.append(Sdg)
+            s = s + half_alpha * (ichi * (Sdg - dchi[i] * Str_f))
             out[q + 1 + i] = isg * s
     if scalar:
         s = 24 + 4 * fluid
         Pi_ = u[s + 1]
-        dPi = [d(s + 1, k) for k in range(3)]
         ddphi = contract_sym(gu2, Sym([dd(s, a, b) for (a, b) in PAIRS]))
         Gd_dphi = Gd[0] * dphi[0] + Gd[1] * dphi[1] + Gd[2] * dphi[2]
         wchi_dphi = wchi[0] * dphi[0] + wchi[1] * dphi[1] + wchi[2] * dphi[2]
         lap_phi = chi * (ddphi - Gd_dphi) - 0.5 * wchi_dphi
         da_dphi = chi * (wphi[0] * dal[0] + wphi[1] * dal[1] + wphi[2] * dal[2])
         out[s] = adv(s) - alpha * Pi_
-        out[s + 1] = (beta[0] * dPi[0] + beta[1] * dPi[1] + beta[2] * dPi[2]) + alpha * (K * Pi_ - lap_phi) - da_dphi
+        out[s + 1] = adv(s + 1) + alpha * (K * Pi_ - lap_phi) - da_dphi
+    if split:
+        S = split_layout(fluid, scalar)
+        g.cut = cut + Ric2 + Gd + [x for t in Gu for x in t.c] + gu.c
+        if S["early"]:
+            g.cut += [x for row in Aud for x in row] + Atu.c + GA + [AA]
+        return g, S, out
     # ---- constraints (diagnostic outputs, same graph) ----
     #  H   = R + 2/3 K^2 - At_ij At^ij - 16 pi rho_H,   R = chi gt^ij R_ij
     #  M^i = gt^ik gt^jl Dt_j At_kl - 3/(2 chi) At^ij d_j chi - 2/3 gt^ij d_j K - 8 pi gt^ij J_j

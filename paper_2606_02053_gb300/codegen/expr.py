@@ -343,7 +343,7 @@ def op_counts(g: Graph, outputs: Sequence[Ex]) -> Dict[str, int]:
 _SUM_OPS = ("add", "sub", "neg")
 
 
-def sum_chains(g: Graph, order: Sequence[int], out_ids: Sequence[int]):
+def sum_chains(g: Graph, order: Sequence[int], out_ids: Sequence[int], keep: Sequence[int] = ()):
     """The sums of the emitted code that are rebuilt as multiply-add chains.
 
     A sum tree is a maximal set of add / sub / neg nodes in which every node but
@@ -356,12 +356,14 @@ def sum_chains(g: Graph, order: Sequence[int], out_ids: Sequence[int]):
     left as a lone multiply), the others follow in the order they become
     available, which keeps the products short-lived.
 
+    Nodes in ``keep`` are never interior.
+
     Returns ({root: [(sign, term), ...]}, the set of interior nodes)."""
     uses: Dict[int, List[int]] = {}
     for n in order:
         for a in g.args[n]:
             uses.setdefault(a, []).append(n)
-    outs = set(out_ids)
+    outs = set(out_ids) | set(keep)
 
     def interior(n):
         u = uses.get(n, [])
@@ -491,6 +493,89 @@ def emit_function(g: Graph, fname: str, in_names: Sequence[str], out_exprs: Sequ
         sig += f", const {params[0]}& {param_struct}"
     sig += extra_args + ")"
     return sig + " {\n" + "\n".join(lines) + "\n}\n"
+
+
+def emit_split(g: Graph, fname: str, a_names: Sequence[str], b_names: Sequence[str], out_exprs: Sequence[Ex],
+               cut: Sequence[Ex], param_struct_type: str) -> str:
+    """Emit the outputs as a function of two phases,
+    ``fname(const InA& ina, const InB& inb, Out&& out, Next&& next, const Params& p)``:
+    first the nodes that ``cut`` depends on, which read their inputs from ina
+    (a_names) only, then ``next()``, then the rest, which reads inb (b_names)
+    only.  What the second phase needs of the first stays in temporaries.  Sums
+    are multiply-add chains as in ``emit_function``; no chain crosses the cut,
+    and a chain that starts with an input starts at its second term."""
+    ai, bi = ({nm: i for i, nm in enumerate(x)} for x in (a_names, b_names))
+    outs = [o.id for o in out_exprs]
+    reach = _reachable(g, outs)
+    first = set(_reachable(g, [c.id for c in cut])) & set(reach)
+    leaf = ("in", "param", "const")
+    leaves = [n for n in reach if g.ops[n] in leaf]
+    one = [n for n in reach if n in first and g.ops[n] not in leaf]
+    two = [n for n in reach if n not in first and g.ops[n] not in leaf]
+    order = leaves + one + two
+    split = len(leaves) + len(one)
+    crossing = {a for n in two for a in g.args[n] if a in first and g.ops[a] not in leaf}
+    chains, inner = sum_chains(g, order, outs, crossing)
+    pos = {n: i for i, n in enumerate(order)}
+    steps_at: Dict[int, List[tuple]] = {}
+    for r, terms in chains.items():
+        p = split if pos[r] >= split else 0
+        at = []
+        for _, x in terms:
+            p = max(p, pos[x])
+            at.append(p)
+        if g.ops[terms[0][1]] in leaf:
+            at[0] = at[1]
+        for j, p in enumerate(at):
+            steps_at.setdefault(p, []).append((r, j))
+    names: Dict[int, str] = {}
+    lines = []
+    written = set()
+    outs_of: Dict[int, List[int]] = {}
+    for k, n in enumerate(outs):
+        outs_of.setdefault(n, []).append(k)
+
+    def name_inputs(index, array):
+        for n in leaves:
+            if g.ops[n] == "in":
+                names.pop(n, None)
+                if g.data[n] in index:
+                    names[n] = f"{array}[{index[g.data[n]]}]"
+
+    def write_outputs(n, t):
+        for k in outs_of.get(n, []):
+            lines.append(f"  out[{k}] = {t};")
+            written.add(k)
+
+    name_inputs(ai, "ina")
+    for i, n in enumerate(order):
+        op = g.ops[n]
+        if i == split:
+            lines.append("  next();")
+            name_inputs(bi, "inb")
+        if op == "param":
+            names[n] = f"p.{g.data[n]}"
+        elif op == "const":
+            names[n] = _fmt(g.data[n])
+        elif op != "in" and n not in inner and n not in chains:
+            t = f"t{n}"
+            lines.append(f"  const double {t} = {_expr(g, n, lambda a: names[a])};")
+            names[n] = t
+            write_outputs(n, t)
+        for r, j in steps_at.get(i, []):
+            terms = chains[r]
+            s, x = terms[j]
+            last = j == len(terms) - 1
+            t = f"t{r}" if last else f"t{r}_{j}"
+            rhs = ("" if s > 0 else "-") + names[x] if j == 0 else f"t{r}_{j - 1} {'+' if s > 0 else '-'} {names[x]}"
+            lines.append(f"  const double {t} = {rhs};")
+            if last:
+                names[r] = t
+                write_outputs(r, t)
+    assert len(written) == len(outs), "an output is a plain input"
+    return (f"template <class InA, class InB, class Out, class Next>\n__device__ __forceinline__ void {fname}"
+            f"(const InA& ina, const InB& inb, Out&& out, Next&& next, const {param_struct_type}& p) {{\n"
+            + "\n".join(lines) + "\n}\n")
 
 
 # ---------------------------------------------------------------------------

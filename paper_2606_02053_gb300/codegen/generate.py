@@ -11,7 +11,7 @@ import sys
 
 from . import bssn
 from . import fluid as fluid_dsl
-from .expr import Ex, emit_function, op_counts, vjp
+from .expr import Ex, emit_function, emit_split, op_counts, vjp
 
 ADJOINT_VARIANTS = ("vac", "fluid", "scalar", "fluid_scalar")
 
@@ -33,6 +33,9 @@ struct AlgebraParams {
   double lapse_c2;
   double shift_on;  // 1: Gamma-driver shift, 0: frozen shift
   double w;         // fluid equation of state P = w rho
+  // split form (codegen/bssn.py, split_layout): factor of the Kreiss-Oliger brackets, and the unit
+  // of length l, 3/4 l, 4/3 l (its eta carries l^2, its lapse_c1 and lapse_c2 l)
+  double ko, len, c75, c43;
 };
 """
 
@@ -56,6 +59,13 @@ def render() -> dict:
         body.append(_slot_fn("d1_slot", L["d1"]))
         body.append(_slot_fn("d2_slot", L["d2"]))
         body.append(emit_function(g, "rhs", L["names"], out, ["AlgebraParams"], accessors=True))
+        gs, S, outs = bssn.algebra(fluid, scalar, split=True)
+        body.append("// the right-hand side in two phases (codegen/bssn.py, split_layout); the slots of its inputs\n"
+                    "// in regions A and B, and of its outputs in B")
+        body.append(f"constexpr int SA = {len(S['a'])}, SB = {len(S['b'])};")
+        body.append(f"constexpr bool SPLIT_EARLY = {str(S['early']).lower()};  // At among the states of region A")
+        body.append(_table_fn("out_slot", S["out"]))
+        body.append(emit_split(gs, "rhs_split", S["a"], S["b"], outs, gs.cut, "AlgebraParams"))
         body.append(emit_function(g, "constraints", L["names"], g.constraints, ["AlgebraParams"]))
         if name in ADJOINT_VARIANTS:
             # reverse mode: in[0 .. NIN) as for rhs, in[NIN + f] = cotangent of out[f];

@@ -26,9 +26,14 @@ static int nin_of(const cosmos_params* p) {
 }
 
 // Forward stage and reverse launchers of the matter variant.
-static cudaError_t launch_stage_for(const cosmos_params* p, const StageArgs& a, int mode, cudaStream_t s) {
-  if (p->fluid) return p->scalar ? launch_stage_fluid_scalar(a, mode, s) : launch_stage_fluid(a, mode, s);
-  return p->scalar ? launch_stage_scalar(a, mode, s) : launch_stage_vac(a, mode, s);
+static cudaError_t launch_stage_for(const cosmos_params* p, const StageArgs& a, int mode, int k_cnt, cudaStream_t s) {
+  if (p->fluid) return p->scalar ? launch_stage_fluid_scalar(a, mode, k_cnt, s) : launch_stage_fluid(a, mode, k_cnt, s);
+  return p->scalar ? launch_stage_scalar(a, mode, k_cnt, s) : launch_stage_vac(a, mode, k_cnt, s);
+}
+
+static cudaError_t launch_deriv_for(const cosmos_params* p, const StageArgs& a, cudaStream_t s) {
+  if (p->fluid) return p->scalar ? launch_deriv_fluid_scalar(a, s) : launch_deriv_fluid(a, s);
+  return p->scalar ? launch_deriv_scalar(a, s) : launch_deriv_vac(a, s);
 }
 
 static cudaError_t launch_vjp_for(const cosmos_params* p, const VjpArgs& a, cudaStream_t s) {
@@ -56,10 +61,10 @@ static AdjLayout adj_layout(const cosmos_grid* g, const cosmos_params* p, int op
     L.LAM = take(nf * fs);
     L.Dfw = take((size_t)nder(p->scalar) * fs);
   }
-  if (op == COSMOS_OP_VJP) L.Dfw = take((size_t)nder(p->scalar) * fs);  // derivative pass of the linearisation point
+  if (op == COSMOS_OP_VJP) L.Dfw = take((size_t)nder(p->scalar) * fs);  // differences at the linearisation point
   if (op == COSMOS_OP_ADJOINT || op == COSMOS_OP_VJP) {
-    // limb copy for the integer derivative pass (the forward stages and the
-    // linearisation points use the same derivative pass as cosmos_rk4_step)
+    // limb copy for the integer differences of the forward stages and of the
+    // linearisation points
     const int nslot = 24 + 2 * p->scalar;
     L.limbs = take((size_t)nslot * fs);
     L.expo = take(((size_t)nslot + 1) / 2);
@@ -91,7 +96,7 @@ static int check_ws_adj(size_t need, void* ws, size_t ws_bytes) {
   return COSMOS_OK;
 }
 
-// Limb copy of every derivative field of U for the integer derivative pass.
+// Limb copy of every derivative field of U.
 static cudaError_t limbs_of(const cosmos_params* p, const DevGrid& g, const double* U, double* ws, const AdjLayout& L,
                             StageArgs& a, cudaStream_t s) {
   const int nslot = 24 + 2 * p->scalar;
@@ -133,11 +138,10 @@ static cudaError_t vjp_once(const cosmos_grid* g, const cosmos_params* p, const 
   d.c = a.c;
   d.U = U;
   d.D = ws + L.Dfw;
-  d.skip_ko = 1;
   a.D = d.D;
   {
     cudaError_t e = limbs_of(p, d.g, U, ws, L, d, s);
-    if (e == cudaSuccess) e = launch_stage_for(p, d, -1, s);
+    if (e == cudaSuccess) e = launch_deriv_for(p, d, s);
     if (e != cudaSuccess) return e;
   }
   if (p->fluid) {
@@ -176,8 +180,7 @@ static cudaError_t fwd_stage(const cosmos_grid* g, const cosmos_params* p, const
   a.out = out;
   a.acc = acc;
   a.cdt = cdt;
-  a.bk = 2.0;
-  a.D = ws + L.Dfw;
+  set_units(&a, p->ko_sigma, 2.0);
   if (p->fluid) {
     cudaError_t e = launch_fluid_prim(a.g, U_s, ws + L.prim, p->w, s);
     if (e != cudaSuccess) return e;
@@ -187,7 +190,7 @@ static cudaError_t fwd_stage(const cosmos_grid* g, const cosmos_params* p, const
   }
   const cudaError_t e = limbs_of(p, a.g, U_s, ws, L, a, s);
   if (e != cudaSuccess) return e;
-  return launch_stage_for(p, a, MODE_S1, s);
+  return launch_stage_for(p, a, MODE_S1, g->nz, s);
 }
 
 // Compaction: per-block partial histograms over shells k = floor(sqrt(m)) + 1,

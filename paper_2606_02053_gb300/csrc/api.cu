@@ -41,8 +41,28 @@ Coef make_coef(const cosmos_grid* g, double sigma) {
   c.mix[0] = 1.0 / (144.0 * g->h[0] * g->h[1]);
   c.mix[1] = 1.0 / (144.0 * g->h[0] * g->h[2]);
   c.mix[2] = 1.0 / (144.0 * g->h[1] * g->h[2]);
-  c.ko_s = (c.ko[0] == c.ko[1] && c.ko[1] == c.ko[2]) ? c.ko[0] : 1.0;
   return c;
+}
+
+void set_units(StageArgs* a, double sigma, double bk) {
+  const double len = 12.0 * a->g.h[0];
+  a->len = len;
+  a->len2 = len * len;
+  for (int d = 0; d < 3; ++d) a->ratio[d] = a->g.h[0] / a->g.h[d];
+  a->eq = a->g.h[0] == a->g.h[1] && a->g.h[0] == a->g.h[2];
+  const double inv[4] = {1.0 / len, 1.0 / (len * len), 1.0 / (len * len * len), 1.0};
+  for (int q = 0; q < 4; ++q) {
+    a->inv_len[q] = inv[q];
+    a->cdt_len[q] = a->cdt * inv[q];
+    a->bk_len[q] = bk * inv[q];
+  }
+  a->ap.eta *= len * len;
+  a->ap.lapse_c1 *= len;
+  a->ap.lapse_c2 *= len;
+  a->ap.ko = 12.0 * sigma / 64.0;  // l sigma / (64 h_x)
+  a->ap.len = len;
+  a->ap.c75 = 0.75 * len;
+  a->ap.c43 = 4.0 / 3.0 * len;
 }
 
 DevGrid make_devgrid(const cosmos_grid* g) {
@@ -63,6 +83,7 @@ double K_ref(const cosmos_params* p, double t) {
 
 AlgebraParams algebra_params(const cosmos_params* p, double t) {
   AlgebraParams a;
+  a.ko = a.len = a.c75 = a.c43 = 0.0;  // of the split form only (set_units)
   a.eta = p->eta;
   a.Kref = K_ref(p, t);
   a.lapse_c1 = p->slicing == 0 ? 2.0 : 0.0;
@@ -85,7 +106,7 @@ int validate(const cosmos_grid* g, const cosmos_params* p) {
   if (!g || !p) return COSMOS_EINVAL;
   if (g->nx < 1 || g->ny < 1 || g->nz < 1 || g->pitch < g->nx) return COSMOS_EINVAL;
   if (g->nz > 65535 || (g->ny + BY - 1) / BY > 65535) return COSMOS_EINVAL;
-  // the derivative pass forms neighbour offsets within one field in 32 bits
+  // neighbour offsets within one field are formed in 32 bits
   if ((long long)g->pitch * g->ny * g->nz >= (1ll << 31)) return COSMOS_EINVAL;
   for (int d = 0; d < 3; ++d)
     if (!(g->h[d] > 0.0) || !isfinite(g->h[d])) return COSMOS_EINVAL;
@@ -116,9 +137,8 @@ WsLayout ws_layout(const cosmos_grid* g, const cosmos_params* p, int op) {
       L.prim = take(4 * fs);
       L.flux = take(12 * fs);
     }
-    L.D = take((size_t)nder(p->scalar) * fs);
-    // limb copy of the stage state (8 bytes per value) for the integer
-    // derivative pass, one slot per field with derivatives, and their exponents
+    // limb copy of the stage state (8 bytes per value), one slot per field with
+    // derivatives, and their exponents
     const int nslot = 24 + 2 * p->scalar;
     L.limbs = take((size_t)nslot * fs);
     L.expo = take(((size_t)nslot + 1) / 2);
@@ -297,7 +317,7 @@ __global__ void fp64_fma_chains(double* __restrict__ out, int iters, double a, d
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
-typedef cudaError_t (*StageLauncher)(const StageArgs&, int, cudaStream_t);
+typedef cudaError_t (*StageLauncher)(const StageArgs&, int, int, cudaStream_t);
 typedef cudaError_t (*ConstraintLauncher)(const ConstraintArgs&, cudaStream_t);
 
 static StageLauncher stage_launcher(const cosmos_params* p) {
@@ -315,19 +335,16 @@ static ConstraintLauncher constraint_launcher(const cosmos_params* p) {
 }
 
 // Shared body of cosmos_rhs / cosmos_rk4_stage / cosmos_stage_pass.
-// pass_mask bit 0: fluid pre-pass (primitives, face fluxes); bit 1: derivative
-// pass; bit 2: algebra pass + combine.
-// f_lo, f_hi: field range of the derivative pass (f_hi = 0: all fields);
-// k_lo, k_cnt: plane range of the algebra pass (k_cnt = 0: all planes).
+// pass_mask bit 0: fluid pre-pass (primitives, face fluxes); bit 1: limb copy of
+// the stage state; bit 2: differences, algebra and combine.
+// f_lo, f_hi: field range of the limb copy (f_hi = 0: all fields);
+// k_lo, k_cnt: plane range of the stage (k_cnt = 0: all planes).
 int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const double* U_s, double* U_n, double* out,
               double* acc, double t_stage, double cdt, double bk, double* ws, const WsLayout& L, cudaStream_t s,
               int pass_mask, int f_lo, int f_hi, int k_lo, int k_cnt, const int* E_ext, int expo_flags) {
   StageArgs a;
   memset(&a, 0, sizeof(a));
-  a.f_lo = f_lo;
-  a.f_hi = f_hi;
   a.k_lo = k_lo;
-  a.k_cnt = k_cnt;
   a.g = make_devgrid(g);
   a.c = make_coef(g, p->ko_sigma);
   a.ap = algebra_params(p, t_stage);
@@ -337,8 +354,9 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
   a.out = out;
   a.acc = acc;
   a.cdt = cdt;
-  a.bk = bk;
-  a.D = ws + L.D;
+  set_units(&a, p->ko_sigma, bk);
+  a.L = (const long long*)(ws + L.limbs);
+  a.E = E_ext ? E_ext : (const int*)(ws + L.expo);
   if (p->fluid) {
     double* prim = ws + L.prim;
     double* flux = ws + L.flux;
@@ -350,9 +368,7 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
     a.flux = flux;
   }
   if (pass_mask & 2) {
-    // limb copy of the fields of this derivative pass (slots of fields f_lo .. f_hi - 1)
-    a.L = (const long long*)(ws + L.limbs);
-    a.E = (const int*)(ws + L.expo);
+    // slots of fields f_lo .. f_hi - 1
     const int nf = cosmos_nfields(p), hi = f_hi > 0 ? f_hi : nf;
     int s_lo = 1 << 30, s_hi = 0;
     for (int f = f_lo; f < hi; ++f) {
@@ -362,9 +378,8 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
       s_hi = sl + 1 > s_hi ? sl + 1 : s_hi;
     }
     if (E_ext) {
-      a.E = E_ext;
       CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, E_ext, (long long*)(ws + L.limbs), s));
-    } else if (expo_flags & 1) {  // exponents recorded by the previous stage's algebra pass
+    } else if (expo_flags & 1) {  // exponents recorded by the previous stage
       CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, a.E, (long long*)(ws + L.limbs), s));
     } else {
       CK(launch_limbs(a.g, U_s, p->fluid, s_lo, s_hi, (int*)(ws + L.expo), (long long*)(ws + L.limbs), s));
@@ -375,13 +390,7 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
     a.E_rec = (unsigned*)(ws + L.erec);
     if (expo_flags & 4) CK(cudaMemsetAsync(a.E_rec, 0, sizeof(unsigned) * 32 * nslot, s));
   }
-  if ((pass_mask & 6) == 6) {
-    CK(stage_launcher(p)(a, mode, s));
-  } else if (pass_mask & 2) {
-    CK(stage_launcher(p)(a, -1, s));  // derivative pass only
-  } else if (pass_mask & 4) {
-    CK(stage_launcher(p)(a, mode | 8, s));  // algebra pass only
-  }
+  if (pass_mask & 4) CK(stage_launcher(p)(a, mode, k_cnt > 0 ? k_cnt : g->nz, s));
   if ((expo_flags & 2) && (pass_mask & 4)) CK(launch_exponents_from_record(a.E_rec, (int*)(ws + L.expo), nslot, s));
   return COSMOS_OK;
 }
@@ -562,7 +571,7 @@ int rk4_on(const cosmos_grid* g, const cosmos_params* p, double* state, double t
   double* acc = w + L.acc;
   const double dt2 = 0.5 * dt;
   int e;
-  // stage 1 scans U_n (the caller may have changed it); each algebra pass records the
+  // stage 1 scans U_n (the caller may have changed it); each stage records the
   // exponents of the state it writes, so stages 2-4 need no scan
   if ((e = run_stage(g, p, MODE_S1, state, state, A, acc, t, dt2, 2.0, w, L, s, 7, 0, 0, 0, 0, nullptr, 6))) return e;
   if ((e = run_stage(g, p, MODE_S23, A, state, B, acc, t + dt2, dt2, 2.0, w, L, s, 7, 0, 0, 0, 0, nullptr, 3)))
@@ -648,9 +657,9 @@ int cosmos_evolve_host(const cosmos_grid* g, const cosmos_params* p, const doubl
   double* acc = w + L.acc;
   const double dt2 = 0.5 * dt;
   // The copies run on their own stream: the host-to-device copy in NCH field
-  // groups, each followed on `s` by the first derivative pass over those
+  // groups, each followed on `s` by the first limb copy of those
   // fields; the device-to-host copy in NSL slabs of z-planes, each started as
-  // soon as the last algebra pass has written its planes.
+  // soon as the last stage has written its planes.
   constexpr int NCH = 4, NSL_MAX = 8;
   const int nsl = g->nz < NSL_MAX ? g->nz : NSL_MAX;
   const size_t plane = (size_t)g->ny * (size_t)g->pitch;
@@ -682,7 +691,7 @@ int cosmos_evolve_host(const cosmos_grid* g, const cosmos_params* p, const doubl
                               nullptr, 6))) {
       return e;
     }
-    // as cosmos_rk4_step: stages 2-4 take the exponents the algebra pass before recorded
+    // as cosmos_rk4_step: stages 2-4 take the exponents the stage before recorded
     if ((e = run_stage(g, p, MODE_S23, A, dev_state, B, acc, ts + dt2, dt2, 2.0, w, L, s, 7, 0, 0, 0, 0, nullptr, 3)))
       return e;
     if ((e = run_stage(g, p, MODE_S23, B, dev_state, A, acc, ts + dt2, dt, 2.0, w, L, s, 7, 0, 0, 0, 0, nullptr, 3)))

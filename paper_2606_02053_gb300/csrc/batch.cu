@@ -46,18 +46,18 @@ static long max_tiles(const cosmos_grid& g) {
 }
 
 struct BatchLayout {
-  std::vector<size_t> A, B, acc, prim, flux, D, limbs;  // per instance, in doubles from ws
-  size_t args, tiles, dtiles, kref, expo, erec;         // byte offsets (expo: n x nslot exponents; erec:
-                                                        // the algebra passes' record, 32 unsigned per slot)
+  std::vector<size_t> A, B, acc, prim, flux, limbs;  // per instance, in doubles from ws
+  size_t args, tiles, stiles, kref, expo, erec;         // byte offsets (expo: n x nslot exponents; erec:
+                                                        // the stages' record, 32 unsigned per slot)
   size_t total;
 };
 
-// limb slots of the integer derivative pass (stage_int.cuh)
+// limb slots (stage_int.cuh)
 static int nslot_of(const cosmos_params* p) { return 24 + 2 * p->scalar; }
 
-// BX x DBY (32 x 8) tiles of every plane: the derivative pass's work list
-static long deriv_tiles(const cosmos_grid& g) {
-  return (long)((g.nx + BX - 1) / BX) * ((g.ny + DBY - 1) / DBY) * g.nz;
+// SPLIT_TX x SPLIT_TY tiles of every plane: the work list of the stage kernel
+static long stage_tiles(const cosmos_grid& g) {
+  return (long)((g.nx + SPLIT_TX - 1) / SPLIT_TX) * ((g.ny + SPLIT_TY - 1) / SPLIT_TY) * g.nz;
 }
 
 static BatchLayout batch_layout(int n, const cosmos_grid* grids, const cosmos_params* p, int max_steps) {
@@ -69,7 +69,7 @@ static BatchLayout batch_layout(int n, const cosmos_grid* grids, const cosmos_pa
     off += al256(bytes);
     return o;
   };
-  long tiles = 0, dtiles = 0;
+  long tiles = 0, stiles = 0;
   for (int i = 0; i < n; ++i) {
     const size_t fs = (size_t)grids[i].pitch * grids[i].ny * grids[i].nz;
     L.A.push_back(take(nf * fs * 8) / 8);
@@ -77,14 +77,13 @@ static BatchLayout batch_layout(int n, const cosmos_grid* grids, const cosmos_pa
     L.acc.push_back(take(nf * fs * 8) / 8);
     L.prim.push_back(p->fluid ? take(4 * fs * 8) / 8 : 0);
     L.flux.push_back(p->fluid ? take(12 * fs * 8) / 8 : 0);
-    L.D.push_back(take((size_t)nder(p->scalar) * fs * 8) / 8);
     L.limbs.push_back(take((size_t)nslot_of(p) * fs * 8) / 8);
     tiles += max_tiles(grids[i]);
-    dtiles += deriv_tiles(grids[i]);
+    stiles += stage_tiles(grids[i]);
   }
   L.args = take(sizeof(StageArgs) * 4 * (size_t)n);
   L.tiles = take(sizeof(BatchTile) * (size_t)tiles);
-  L.dtiles = take(sizeof(BatchTile) * (size_t)dtiles);
+  L.stiles = take(sizeof(BatchTile) * (size_t)stiles);
   L.kref = take(sizeof(double) * (size_t)max_steps * 4 * n);
   L.expo = take(sizeof(int) * (size_t)n * nslot_of(p));
   L.erec = take(sizeof(unsigned) * 32 * (size_t)n * nslot_of(p));  // per instance and slot, one line each
@@ -105,10 +104,11 @@ struct cosmos_batch_s {
   int sms = 0;
   char* ws = nullptr;
   BatchLayout L;
-  long ntiles = 0, ndtiles = 0;
+  long ntiles = 0, nstiles = 0;
   StageArgs* d_args = nullptr;  // [4][n]
   BatchTile* d_tiles = nullptr;
-  BatchTile* d_dtiles = nullptr;  // derivative-pass tiles (BX x DBY of one z-plane; c = the plane)
+  bool eq = true;                 // every grid has equal spacing
+  BatchTile* d_stiles = nullptr;  // stage-kernel tiles (SPLIT_TX x SPLIT_TY of one z-plane; c = the plane)
   double* d_kref = nullptr;     // [max_steps][4][n]
   cudaGraphExec_t gexec = nullptr;
   int g_first = -1, g_steps = -1;
@@ -202,7 +202,7 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
   double* wsd = (double*)ws;
   b->d_args = (StageArgs*)(b->ws + L.args);
   b->d_tiles = (BatchTile*)(b->ws + L.tiles);
-  b->d_dtiles = (BatchTile*)(b->ws + L.dtiles);
+  b->d_stiles = (BatchTile*)(b->ws + L.stiles);
   b->d_kref = (double*)(b->ws + L.kref);
 
   // per-stage, per-instance arguments (same fields as the single-grid stages)
@@ -227,8 +227,8 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
       a.out = outs[s];
       a.acc = acc;
       a.cdt = cdt[s];
-      a.bk = 2.0;
-      a.D = wsd + L.D[i];
+      set_units(&a, p->ko_sigma, 2.0);
+      b->eq = b->eq && a.eq;
       a.L = (const long long*)(wsd + L.limbs[i]);
       a.E = (const int*)(b->ws + L.expo) + (size_t)i * nslot_of(p);
       // stages 1-3 record the exponents of the state they write for the next stage
@@ -257,20 +257,18 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
     return COSMOS_ECUDA;
   }
   {
-    // Derivative-pass tiles instance by instance, plane by plane: the resident
-    // blocks of the persistent pass then work on neighbouring planes of one grid,
-    // whose z-stencils share their planes in L2 (interleaving the instances, as
-    // for the pointwise passes, spread them over every grid at once and sent the
-    // shared planes back to DRAM).
-    std::vector<BatchTile> dt;
+    // Tiles instance by instance, plane by plane: the blocks of the persistent
+    // stage kernel then work on neighbouring planes of one grid, whose z-stencils
+    // share their planes in L2.
+    std::vector<BatchTile> st;
     for (int i = 0; i < n; ++i) {
       const cosmos_grid& g = grids[i];
-      const int tx = (g.nx + BX - 1) / BX, ty = (g.ny + DBY - 1) / DBY;
-      for (long w = 0; w < deriv_tiles(g); ++w)
-        dt.push_back(BatchTile{i, (int)(w % tx), (int)((w / tx) % ty), (int)(w / ((long)tx * ty))});
+      const int tx = (g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = (g.ny + SPLIT_TY - 1) / SPLIT_TY;
+      for (long w = 0; w < stage_tiles(g); ++w)
+        st.push_back(BatchTile{i, (int)(w % tx), (int)((w / tx) % ty), (int)(w / ((long)tx * ty))});
     }
-    b->ndtiles = (long)dt.size();
-    if (cudaMemcpy(b->d_dtiles, dt.data(), sizeof(BatchTile) * dt.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+    b->nstiles = (long)st.size();
+    if (cudaMemcpy(b->d_stiles, st.data(), sizeof(BatchTile) * st.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
       delete b;
       return COSMOS_ECUDA;
     }
@@ -289,16 +287,6 @@ int cosmos_batch_set_tuning(cosmos_batch b, const cosmos_batch_tuning* tuning) {
   drop_graph(b);
   b->tune = *tuning;
   return upload_tiles(b);
-}
-
-// persistent grid of the integer derivative pass: its resident blocks on every SM
-static int ideriv_blocks(cosmos_batch b) { return b->sms * COSMOS_IDERIV_MIN_BLOCKS; }
-
-// every grid of the batch admits the integer pass's division-free periodic wrap
-static bool ideriv_near(cosmos_batch b) {
-  for (int i = 0; i < b->n; ++i)
-    if (!near_indices(make_devgrid(&b->grids[i]))) return false;
-  return true;
 }
 
 static int batch_launch_steps(cosmos_batch b, int first_step, int steps, cudaStream_t s) {
@@ -320,13 +308,12 @@ static int batch_launch_steps(cosmos_batch b, int first_step, int steps, cudaStr
       const double* kref = b->d_kref + ((size_t)st * 4 + stage) * b->n;
       const int ns = nslot_of(&b->p);
       // stage 1 scans every instance's state; stages 2-4 take the exponents the previous
-      // stage's algebra pass recorded
+      // stage's stage recorded
       const cudaError_t le = stage == 0
                                  ? launch_batch_limbs(args, b->n, ns, b->p.fluid, (int*)(b->ws + b->L.expo), s)
                                  : launch_batch_to_limbs(args, b->n, ns, b->p.fluid, s);
       if (le != cudaSuccess ||
-          launch(args, b->d_tiles, b->ntiles, b->tune.mapping, kref, modes[stage], grid, block, s, b->d_dtiles,
-                 b->ndtiles, ideriv_blocks(b), ideriv_near(b)) != cudaSuccess)
+          launch(args, b->d_stiles, b->nstiles, kref, modes[stage], b->eq, s) != cudaSuccess)
         return COSMOS_ECUDA;
       if (stage < 3 && launch_exponents_from_record((unsigned*)(b->ws + b->L.erec), (int*)(b->ws + b->L.expo),
                                                     b->n * ns, s) != cudaSuccess)
@@ -383,8 +370,7 @@ int cosmos_batch_time_stage(cosmos_batch b, int reps, double* ms_out, void* stre
       rc = COSMOS_ECUDA;
     if (rc == COSMOS_OK &&
         (launch_batch_limbs(b->d_args, b->n, nslot_of(&b->p), b->p.fluid, (int*)(b->ws + b->L.expo), s) != cudaSuccess ||
-         launch(b->d_args, b->d_tiles, b->ntiles, b->tune.mapping, b->d_kref, MODE_S1, grid, block, s, b->d_dtiles,
-                b->ndtiles, ideriv_blocks(b), ideriv_near(b)) != cudaSuccess ||
+         launch(b->d_args, b->d_stiles, b->nstiles, b->d_kref, MODE_S1, b->eq, s) != cudaSuccess ||
          launch_exponents_from_record((unsigned*)(b->ws + b->L.erec), (int*)(b->ws + b->L.expo),
                                       b->n * nslot_of(&b->p), s) != cudaSuccess))  // leaves the record cleared
       rc = COSMOS_ECUDA;

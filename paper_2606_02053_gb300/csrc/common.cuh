@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/cosmos.h"
 #include "generated/bssn_algebra.cuh"
@@ -16,7 +17,9 @@ constexpr int BY = 4;   // rows per block
 #ifndef COSMOS_DERIV_ROWS
 #define COSMOS_DERIV_ROWS 8
 #endif
-constexpr int DBY = COSMOS_DERIV_ROWS;  // rows per block of the derivative pass
+constexpr int DBY = COSMOS_DERIV_ROWS;  // rows per block of the reverse mode's derivative pass
+// tile of one z-plane in the stage kernel (stage_split.cuh), one point per algebra thread
+constexpr int SPLIT_TX = 16, SPLIT_TY = 8;
 
 // Grid description as the kernels see it.
 struct DevGrid {
@@ -64,8 +67,6 @@ struct Coef {
   double mix[3];          // mixed xy, xz, yz:  1/(144 h_a h_b)
   double ko[3];           // sigma/(64 h_d)
   double ih[3];           // 1/h_d (flux divergence)
-  double ko_s;            // factor of the KO slots of the derivative buffer: ko[0] with equal
-                          // spacing (the slots hold the bracket), else 1 (they hold the term)
 };
 
 Coef make_coef(const cosmos_grid* g, double sigma);
@@ -74,35 +75,39 @@ double K_ref(const cosmos_params* p, double t);                 // background tr
 AlgebraParams algebra_params(const cosmos_params* p, double t); // runtime parameters of the algebra
 int validate(const cosmos_grid* g, const cosmos_params* p);     // COSMOS_OK or COSMOS_EINVAL
 
-// RK4 stage modes of the fused kernel
+// RK4 stage modes
 enum StageMode { MODE_RHS = 0, MODE_S1 = 1, MODE_S23 = 2, MODE_S4 = 3 };
 
 struct StageArgs {
   DevGrid g;
   Coef c;
-  AlgebraParams ap;
+  AlgebraParams ap;                // eta and ko in the units of stage_split.cuh (l = 12 h_x), Kref as given
   const double* __restrict__ U;    // stencil input (stage state)
-  const double* __restrict__ U0;   // U_n (pointwise) -- MODE_S1/S23/S4
+  const double* __restrict__ U0;   // U_n (pointwise) -- MODE_S1/S23
   double* U0w;                     // U_n written in MODE_S4
   double* out;                     // MODE_RHS: rhs;  MODE_S1/S23: U_next
   double* acc;                     // accumulator
   const double* __restrict__ prim; // fluid primitives [4][pts] (fluid only)
   const double* __restrict__ flux; // fluid face fluxes [3][4][pts] (fluid only)
-  double* D;                       // derivative-pass output [NDER][pts] (see stage_kernel.cuh)
+  double* D;                       // finite differences of U for the reverse mode (ideriv_kernel only)
   double cdt;                      // dt * c_{s+1}, or dt/6 in MODE_S4
-  double bk;                       // accumulator weight (2 for stages 2, 3)
-  int f_lo, f_hi;                  // derivative pass: only fields f_lo <= f < f_hi (f_hi = 0: all)
-  int k_lo, k_cnt;                 // algebra pass: only planes k_lo .. k_lo + k_cnt - 1 (k_cnt = 0: all)
-  int skip_ko;                     // derivative pass: leave the Kreiss-Oliger slots of D unwritten
-  const long long* __restrict__ L; // limb copy of U (stage_int.cuh); null: the FP64 derivative pass
+  double len, len2;                // l = 12 h_x, l^2
+  double inv_len[4];               // 1/l, 1/l^2, 1/l^3 (per degree of the field, stage_split.cuh), 1
+  double cdt_len[4], bk_len[4];    // cdt and the accumulator weight (2 for stages 2, 3) times those
+  double ratio[3];                 // h_x / h_d
+  int eq;                          // equal spacing
+  int k_lo;                        // first plane (the plane count is the launch's)
+  const long long* __restrict__ L; // limb copy of U (stage_int.cuh)
   const int* __restrict__ E;       // reference exponent of each limb slot
-  unsigned* E_rec;                 // algebra pass, stages 1-3: records the largest biased exponent of
-                                   // each limb slot of U_next at E_rec[32 slot] (null: no record)
+  unsigned* E_rec;                 // stages 1-3: records the largest biased exponent of each limb
+                                   // slot of U_next at E_rec[32 slot] (null: no record)
 };
+// Fills the units of `a` (its grid, ap, cdt given) for dissipation sigma.
+void set_units(StageArgs* a, double sigma, double bk);
 
-// Doubles per point of the derivative-pass buffer: first and second
-// derivatives plus the Kreiss-Oliger term of every non-fluid field.
-inline int nder(int scalar) { return 3 * (24 + 2 * scalar) + 6 * (11 + scalar) + 24 + 2 * scalar; }
+// Doubles per point of the finite differences that the reverse mode keeps:
+// first and second derivatives.
+inline int nder(int scalar) { return 3 * (24 + 2 * scalar) + 6 * (11 + scalar); }
 
 // One work item of a batch: instance `inst`; for 2D tiles (a, b, c) = (block
 // column, block row, z-plane), for linear runs a = first point index.
@@ -126,24 +131,23 @@ struct ConstraintArgs {
 #endif
 
 // Launchers implemented per matter variant (stage_<variant>.cu).
-cudaError_t launch_stage_vac(const StageArgs& a, int mode, cudaStream_t s);
-cudaError_t launch_stage_fluid(const StageArgs& a, int mode, cudaStream_t s);
-cudaError_t launch_stage_scalar(const StageArgs& a, int mode, cudaStream_t s);
-cudaError_t launch_stage_fluid_scalar(const StageArgs& a, int mode, cudaStream_t s);
-// batched stage: derivative pass over the BX x DBY tile list (dtiles), algebra
-// pass over the tuned work list (tiles, mapping)
-// (last two: resident blocks of the integer derivative pass, 0 for the FP64
-// pass; whether near_indices holds for every grid of the batch)
-typedef cudaError_t (*BatchStageLauncher)(const StageArgs*, const BatchTile*, long, int, const double*, int, dim3,
-                                          dim3, cudaStream_t, const BatchTile*, long, int, bool);
-cudaError_t launch_batch_stage_vac(const StageArgs*, const BatchTile*, long, int, const double*, int, dim3, dim3,
-                                   cudaStream_t, const BatchTile*, long, int, bool);
-cudaError_t launch_batch_stage_fluid(const StageArgs*, const BatchTile*, long, int, const double*, int, dim3, dim3,
-                                     cudaStream_t, const BatchTile*, long, int, bool);
-cudaError_t launch_batch_stage_scalar(const StageArgs*, const BatchTile*, long, int, const double*, int, dim3, dim3,
-                                      cudaStream_t, const BatchTile*, long, int, bool);
-cudaError_t launch_batch_stage_fluid_scalar(const StageArgs*, const BatchTile*, long, int, const double*, int, dim3,
-                                            dim3, cudaStream_t, const BatchTile*, long, int, bool);
+// (k_cnt planes from a.k_lo)
+cudaError_t launch_stage_vac(const StageArgs& a, int mode, int k_cnt, cudaStream_t s);
+cudaError_t launch_stage_fluid(const StageArgs& a, int mode, int k_cnt, cudaStream_t s);
+cudaError_t launch_stage_scalar(const StageArgs& a, int mode, int k_cnt, cudaStream_t s);
+cudaError_t launch_stage_fluid_scalar(const StageArgs& a, int mode, int k_cnt, cudaStream_t s);
+cudaError_t launch_deriv_vac(const StageArgs& a, cudaStream_t s);  // finite differences into a.D
+cudaError_t launch_deriv_fluid(const StageArgs& a, cudaStream_t s);
+cudaError_t launch_deriv_scalar(const StageArgs& a, cudaStream_t s);
+cudaError_t launch_deriv_fluid_scalar(const StageArgs& a, cudaStream_t s);
+// batched stage over the tile list (SPLIT_TX x SPLIT_TY of one plane), K_ref per instance;
+// eq: every grid has equal spacing
+typedef cudaError_t (*BatchStageLauncher)(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
+cudaError_t launch_batch_stage_vac(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
+cudaError_t launch_batch_stage_fluid(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
+cudaError_t launch_batch_stage_scalar(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
+cudaError_t launch_batch_stage_fluid_scalar(const StageArgs*, const BatchTile*, long, const double*, int, bool,
+                                            cudaStream_t);
 cudaError_t launch_batch_fluid(const StageArgs* args, const BatchTile* tiles, long ntiles, int mapping, double w,
                                dim3 grid, dim3 block, cudaStream_t s);
 cudaError_t launch_constraints_vac(const ConstraintArgs& a, cudaStream_t s);
@@ -169,7 +173,7 @@ cudaError_t launch_to_limbs(const DevGrid& g, const double* U, int fluid, int s_
                             long long* L, cudaStream_t s);
 cudaError_t launch_field_exponents(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, int* E,
                                    cudaStream_t s);
-// E[s] = rec[32 s] and rec[32 s] = 0 for s < nslot (the exponents an algebra pass recorded)
+// E[s] = rec[32 s] and rec[32 s] = 0 for s < nslot (the exponents a stage recorded)
 cudaError_t launch_exponents_from_record(unsigned* rec, int* E, int nslot, cudaStream_t s);
 // the batched limb copy with the exponents already in args[i].E
 cudaError_t launch_batch_to_limbs(const StageArgs* args, int n, int nslot, int fluid, cudaStream_t s);
@@ -183,7 +187,7 @@ cudaError_t launch_fluid_flux(const DevGrid& g, const double* U, const double* p
                               int nf_offset_fluid, cudaStream_t s);
 
 inline dim3 point_grid(const DevGrid& g) { return dim3((g.nx + BX - 1) / BX, (g.ny + BY - 1) / BY, g.nz); }
-// integer derivative pass: one BX x DBY tile of one z-plane per block
+// reverse mode's derivative pass: one BX x DBY tile of one z-plane per block
 inline dim3 ideriv_grid(const DevGrid& g) { return dim3((g.nx + BX - 1) / BX, (g.ny + DBY - 1) / DBY, g.nz); }
 // Every index the integer derivative pass forms for a tile lies in [-n, 2n)
 // along each axis, so one compare and select wraps it (stage_int.cuh,

@@ -428,7 +428,7 @@ int advance(const Ctx& c, int l, double t, double dt, double theta0) {
   double* Y3 = child ? c.saved(l, 2) : w + W.stageB;
   double* Y4 = child ? c.saved(l, 3) : w + W.stageA;
   const double dt2 = 0.5 * dt;
-  // on a refined level the algebra pass skips the ghost z-planes: whatever it
+  // on a refined level the stage skips the ghost z-planes: whatever it
   // would write there is replaced from the parent before it is read
   const int k_lo = v.lo[2], k_cnt = v.hi[2] - v.lo[2];
   int e;

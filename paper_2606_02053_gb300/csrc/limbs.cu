@@ -1,4 +1,4 @@
-// Pre-pass of the integer derivative pass (stage_int.cuh): the reference
+// Pre-pass of the integer differences (stage_int.cuh): the reference
 // exponent of every limb slot, then the limb copy of the stage state.
 #include "stage_kernel.cuh"
 

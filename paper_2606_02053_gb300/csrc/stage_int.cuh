@@ -1,9 +1,11 @@
-// Derivative pass in exact integer arithmetic.
+// Finite differences in exact integer arithmetic.
 //
-// GB300 runs FP64 at about 2 operations per clock per SM and 32-bit integer
-// adds and multiply-adds at about 60: the finite-difference and Kreiss-Oliger
-// stencils, integer-coefficient sums of neighbouring values, are cheaper in
-// integer arithmetic than in FP64, and can be made exact there.
+// GB300 runs FP64 at 2 operations per clock per SM and 32-bit integer adds and
+// multiply-adds at about 60: the finite-difference and Kreiss-Oliger stencils,
+// integer-coefficient sums of neighbouring values, are cheaper in integer
+// arithmetic than in FP64, and can be made exact there.  The stage kernel
+// (stage_split.cuh) forms them tile by tile; ideriv_kernel below writes them to
+// memory for the reverse mode.
 //
 // Representation ("limbs"): every value f of one field is held as the signed
 // 64-bit integer V = f 2^(1085 - e_ref), with e_ref the largest biased FP64
@@ -11,20 +13,18 @@
 // 53 + 10 significant bits (|V| < 2^63), every value down to 2^-10 of it is
 // exact, and smaller ones are truncated by at most 2^-62 of the largest (a
 // relative 2e-15 even of a 256^3 second derivative of such a field, where the
-// tolerance is 1e-12).  On load V is split into three 21-bit digits
-// V = L0 + L1 2^21 + L2 2^42 (L0, L1 in [0, 2^21), L2 signed).  A stencil
-// sum_o c_o f_o with integer c_o is then the digit-wise sums sum_o c_o L_k(o):
-// with sum |c_o| <= 324 (the largest, the mixed derivative on staged first-
-// derivative sums) every digit sum stays below 2^31, so there are no carries
-// and the sum is exact.  Each result is rounded once to FP64 (round to
-// nearest even) and multiplied by its stencil coefficient (1/(12 h),
-// 1/(12 h^2), 1/(144 h_a h_b)): the stored value is within one rounding of the
-// exact stencil of the inputs.
+// tolerance is 1e-12).  A stencil sum_o c_o f_o with integer c_o (sum |c_o| <= 324,
+// the mixed derivative on staged first-derivative sums) needs up to 72 bits.
+// It is carried as (w, h): w the sum of the V modulo 2^64, h the sum of their
+// upper parts floor(V / 2^42), which stays below 2^30.  The lower parts add less
+// than 324 x 2^42 < 2^51, so h tells whether the sum fits 64 bits (then it is w),
+// and if not, w - h 2^42, taken modulo 2^64, is the exact difference: the sum is
+// h 2^42 + that.  Two words and one, three instructions a sum, none to take a
+// loaded value apart but one shift (three 21-bit digits took four, and ten to
+// put a sum together again).  Each result is rounded once to FP64 (round to nearest even).
 //
 // The state is converted to limbs by a pre-pass (limbs.cu: the exponent of
-// every field, then the conversion); the derivative pass reads the limb copy
-// (8 bytes per value, as the state) instead of the state and writes the same
-// derivative buffer as the FP64 pass.
+// every field, then the conversion).
 #pragma once
 
 #include "common.cuh"
@@ -32,13 +32,17 @@
 namespace cosmos {
 
 constexpr int LIMB_EXTRA = 10;                    // significant bits below the largest value's last place
-constexpr unsigned LIMB_MASK = (1u << 21) - 1;    // one 21-bit digit
 
-__device__ __forceinline__ int3 l_add(int3 a, int3 b) { return make_int3(a.x + b.x, a.y + b.y, a.z + b.z); }
-__device__ __forceinline__ int3 l_sub(int3 a, int3 b) { return make_int3(a.x - b.x, a.y - b.y, a.z - b.z); }
-__device__ __forceinline__ int3 l_mul(int3 a, int k) { return make_int3(a.x * k, a.y * k, a.z * k); }
-// a k + b
-__device__ __forceinline__ int3 l_mad(int3 a, int k, int3 b) { return make_int3(a.x * k + b.x, a.y * k + b.y, a.z * k + b.z); }
+struct Limb {
+  unsigned long long w;  // the sum modulo 2^64
+  int h;                 // the sum of floor(V / 2^42)
+};
+__host__ __device__ __forceinline__ Limb l_add(Limb a, Limb b) { return {a.w + b.w, a.h + b.h}; }
+__host__ __device__ __forceinline__ Limb l_sub(Limb a, Limb b) { return {a.w - b.w, a.h - b.h}; }
+// k > 0
+__host__ __device__ __forceinline__ Limb l_mul(Limb a, int k) { return {a.w * (unsigned)k, a.h * k}; }
+// 8 a - b, the first-derivative sum of a = f(+1) - f(-1), b = f(+2) - f(-2)
+__host__ __device__ __forceinline__ Limb l_d1(Limb a, Limb b) { return l_sub(l_mul(a, 8), b); }
 
 // V of f for a field with reference exponent e_ref (>= the exponent of f).
 __device__ __forceinline__ long long to_limbs(double f, int e_ref) {
@@ -51,77 +55,103 @@ __device__ __forceinline__ long long to_limbs(double f, int e_ref) {
   return (b >> 63) ? -(long long)V : (long long)V;
 }
 
-// the digits of a stored V
-__device__ __forceinline__ int3 digits(long long V) {
-  return make_int3((int)(V & LIMB_MASK), (int)((V >> 21) & LIMB_MASK), (int)(V >> 42));
-}
+__host__ __device__ __forceinline__ Limb limb_of(long long V) { return {(unsigned long long)V, (int)(V >> 42)}; }
 
-// FP64 (round to nearest even) of the unsigned 128-bit magnitude (uh, lo)
-// times 2^(e_ref - 1085), negated if neg.
-__device__ __forceinline__ double round_mag(unsigned long long uh, unsigned long long lo, bool neg, int e_ref) {
-  if ((uh | lo) == 0) return 0.0;
-  const int n = uh ? 127 - __clzll(uh) : 63 - __clzll(lo);  // leading one
-  int ex = n + e_ref - 1085 + 1023;                           // biased exponent of the result
-  unsigned long long m;
-  if (n <= 52) {
-    m = lo << (52 - n);
-  } else {
-    const int r = n - 52;  // bits dropped, < 64 (|value| < 2^73)
-    m = (lo >> r) | (r ? uh << (64 - r) : 0ull);
-    const int rb = r - 1;
-    const unsigned long long round = (lo >> rb) & 1ull;
-    const bool sticky = (lo & ((1ull << rb) - 1ull)) != 0;
-    if (round && (sticky || (m & 1ull))) {
-      ++m;
-      if (m >> 53) {
-        m >>= 1;
-        ++ex;
-      }
+// e_ref outside the range in which every sum's exponent is that of a normal
+// number (uniform over a field).
+__host__ __device__ __forceinline__ bool limb_odd(int e_ref) { return e_ref < 80 || e_ref > 1960; }
+
+// limb_big: the sum may not fit a signed 64-bit word (|h| 2^42 near 2^63 or above).
+constexpr int LIMB_FIT = (1 << 21) - (1 << 11);  // LIMB_FIT 2^42 + 2^51 < 2^63
+__host__ __device__ __forceinline__ bool limb_big(Limb S) { return (unsigned)(S.h + LIMB_FIT) >= 2u * LIMB_FIT; }
+
+// FP64 value (bits; round to nearest even) of the sum S times 2^(e_ref - 1085);
+// ODD = limb_odd(e_ref); ANY: also for sums with limb_big.
+//
+// The sum is taken into one signed 64-bit word; where it does not fit, its low 8
+// or 9 bits are dropped first, their "any set" kept in the lowest bit: at least
+// two bits are dropped again below, so that bit never is the last kept one and
+// the rounding is that of the whole sum.  The magnitude's leading one is moved
+// to bit 63 of a pair of 32-bit words, the upper 53 bits are kept, and the
+// dropped 11 (in the upper bits of r) round to nearest even through the carry
+// of r + (2^31 - 1) + the last kept bit; the leading one, or a carry out of the
+// significand, adds into the exponent field.  About 25 instructions, without a
+// branch, so that the conversions of one thread overlap; a 128-bit path for the
+// large sums, taken by half the warps on data that vary along every axis, cost
+// as many again.
+template <bool ODD, bool ANY>
+__host__ __device__ __forceinline__ unsigned long long limb_bits(Limb S, int e_ref) {
+  long long v = (long long)S.w;
+  int ex = e_ref;
+  if (ANY) {
+    const long long t1 = (long long)(S.w - ((unsigned long long)(unsigned)S.h << 42));  // |t1| < 2^51
+    const int ah = S.h < 0 ? -S.h : S.h;
+    // big sums: below 2^70 (2^62 after 8) / below 2^72 (below 2^63 after 9)
+    const int sh = limb_big(S) ? (ah < (1 << 28) ? 8 : 9) : 0;
+    v = (t1 >> sh) + (long long)(((unsigned long long)(unsigned)S.h << (10 - sh)) << 32);
+    v |= ((unsigned)t1 & ((1u << sh) - 1u)) ? 1 : 0;
+    ex += sh;
+  }
+  const int sg = (int)(v >> 63);
+  const unsigned long long u = (unsigned long long)((v ^ (long long)sg) - (long long)sg);
+  const unsigned hi = (unsigned)(u >> 32), lo = (unsigned)u;
+  const bool one = hi == 0;  // one word
+  const unsigned h = one ? lo : hi, l = one ? 0u : lo;
+  const int E = one ? ex - 32 : ex;
+#ifdef __CUDA_ARCH__
+  const int s = __clz((int)h);
+  const unsigned h2 = __funnelshift_l(l, h, s), l2 = l << (s & 31);
+#else
+  const int s = h ? __builtin_clz(h) : 32;
+  const unsigned h2 = s & 31 ? h << s | l >> (32 - s) : h, l2 = l << (s & 31);
+#endif
+  const unsigned mh = h2 >> 11, ml = (h2 << 21) | (l2 >> 11);
+  const unsigned r = l2 << 21, up = 0x7FFFFFFFu + (ml & 1u);
+  // biased exponent 63 - s + E - 1085 + 1023, of which the leading one is 1
+  const unsigned eb = (unsigned)(E - s) << 20;
+#ifdef __CUDA_ARCH__
+  unsigned drop, bl, bh;
+  asm("add.cc.u32 %0, %3, %4;\n\taddc.cc.u32 %1, %5, 0;\n\taddc.u32 %2, %6, %7;"
+      : "=r"(drop), "=r"(bl), "=r"(bh)
+      : "r"(r), "r"(up), "r"(ml), "r"(mh), "r"(eb));
+#else
+  const unsigned inc = (unsigned)(((unsigned long long)r + up) >> 32);
+  const unsigned long long sum = (((unsigned long long)mh << 32) | ml) + inc;
+  unsigned bl = (unsigned)sum, bh = (unsigned)(sum >> 32) + eb;
+#endif
+  if (ODD) {
+    if (e_ref >= 2047) return 0x7FF8000000000000ull;  // the field holds Inf or NaN
+    const int be = E - s + (int)((bh - eb) >> 20);    // biased exponent
+    if (be <= 0) bh = bl = 0;                         // below the normal range: far below any stencil of this field
+    if (be >= 2047) {
+      bh = 0x7FFu << 20;
+      bl = 0;
     }
   }
-  if (ex <= 0) return neg ? -0.0 : 0.0;  // below the normal range: far below any stencil of this field
-  unsigned long long bits = ((unsigned long long)ex << 52) | (m & 0xFFFFFFFFFFFFFull);
-  if (neg) bits |= 1ull << 63;
-  return __longlong_as_double((long long)bits);
+  if (h == 0) bh = 0;  // bl is zero already
+  bh |= (unsigned)sg & 0x80000000u;
+  return ((unsigned long long)bh << 32) | bl;
 }
 
-// round_mag for a magnitude below 2^63 (uh = 0), bitwise the same, without a
-// branch on the magnitude (the lanes of a warp hold sums of every size): the
-// leading one is moved to bit 62 (exact, lo < 2^63), then the low 10 bits are
-// dropped with round to nearest even by adding 0x1FF plus the lowest kept bit
-// (no overflow: x < 2^63).  Sums of at most 53 significant bits have those 10
-// bits zero and pass unchanged.  The leading one, or a carry out of the
-// significand, adds into the exponent field.
-__device__ __forceinline__ double round_mag64(unsigned long long lo, bool neg, int e_ref) {
-  if (lo == 0) return 0.0;
-  const int n = 63 - __clzll(lo);  // position of the leading one, 0..62
-  const unsigned long long x = lo << (62 - n);
-  const unsigned long long m = (x + 0x1FFull + ((x >> 10) & 1ull)) >> 10;  // in [2^52, 2^53]
-  const long long b = ((long long)(n + e_ref - 63) << 52) + (long long)m;  // biased exponent n + e_ref - 62
-  if ((b >> 52) <= 0) return neg ? -0.0 : 0.0;  // below the normal range (as round_mag)
-  return __longlong_as_double((long long)((unsigned long long)b | ((unsigned long long)neg << 63)));
+template <bool ODD>
+__device__ __forceinline__ double limb_value(Limb S, int e_ref) {
+  return __longlong_as_double((long long)limb_bits<ODD, true>(S, e_ref));
 }
 
-// FP64 value of the digit sums S.x + S.y 2^21 + S.z 2^42 (|S.k| < 2^31) in the
-// units of a field with reference exponent e_ref.
-__device__ __forceinline__ double from_limbs(int3 S, int e_ref) {
-  if (e_ref >= 2047) return __longlong_as_double(0x7FF8000000000000ll);  // the field holds Inf or NaN
-  const long long t1 = (long long)S.x + ((long long)S.y << 21);         // |t1| < 2^52
-  if (S.z < (1 << 20) && S.z > -(1 << 20)) {                            // |value| < 2^63: one 64-bit word
-    const long long v = t1 + ((long long)S.z << 42);
-    const bool neg = v < 0;
-    return round_mag64(neg ? (unsigned long long)(-v) : (unsigned long long)v, neg, e_ref);
+// N sums of one warp (every lane takes part) at once: the form without the
+// large sums' part when no lane has one.
+template <bool ODD, int N>
+__device__ __forceinline__ void limb_values(const Limb (&S)[N], const int (&e)[N], double (&v)[N]) {
+  unsigned top = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) top = max(top, (unsigned)(S[q].h + LIMB_FIT));
+  if (__any_sync(0xffffffffu, top >= 2u * LIMB_FIT)) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = limb_value<ODD>(S[q], e[q]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = __longlong_as_double((long long)limb_bits<ODD, false>(S[q], e[q]));
   }
-  // value = t1 + S.z 2^42 as a signed 128-bit integer (hi, lo)
-  const unsigned long long p = (unsigned long long)((long long)S.z << 42);
-  unsigned long long lo = p + (unsigned long long)t1;
-  long long hi = ((long long)S.z >> 22) + (t1 >> 63) + (lo < p ? 1 : 0);
-  const bool neg = hi < 0;
-  if (neg) {
-    lo = ~lo + 1ull;
-    hi = ~hi + (lo == 0 ? 1 : 0);
-  }
-  return round_mag((unsigned long long)hi, lo, neg, e_ref);
 }
 
 // ---------------------------------------------------------------------------
@@ -134,11 +164,13 @@ __device__ __forceinline__ int limb_field(int s, int fluid) { return (fluid && s
 // ---------------------------------------------------------------------------
 // Integer stencils (digit sums; the caller converts and scales)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int3 ldl(const long long* __restrict__ L, int o) { return digits(__ldg(L + o)); }
+__device__ __forceinline__ Limb ldl(const long long* __restrict__ L, int o) { return limb_of(__ldg(L + o)); }
 
-// Digit sums staged in shared memory as int4 (w unused): one 128-bit access each.
-__device__ __forceinline__ int4 p4(int3 v) { return make_int4(v.x, v.y, v.z, 0); }
-__device__ __forceinline__ int3 q3(int4 v) { return make_int3(v.x, v.y, v.z); }
+// Sums staged in shared memory as int4 (the last word unused): one 128-bit access each.
+__device__ __forceinline__ int4 p4(Limb v) { return make_int4((int)v.w, (int)(v.w >> 32), v.h, 0); }
+__device__ __forceinline__ Limb q3(int4 v) {
+  return {((unsigned long long)(unsigned)v.y << 32) | (unsigned)v.x, v.z};
+}
 
 // Periodic neighbour offsets of one point within one field, as 32-bit
 // element offsets (a field of the grids this pass accepts has < 2^31 points).
@@ -190,119 +222,85 @@ __device__ __forceinline__ void stage_dydz_int(const DevGrid& g, const long long
   for (int q = tid; q < TXH * DBY; q += BX * DBY) {
     const int qx = q % TXH, qy = q / TXH;
     const int x = i0 - 2 + qx, y = j0 + qy;
-    sDy[q] = p4(l_sub(l_mul(l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y + 1, k)),
-                                  ldl(Lf, limb_plane_off<NEAR>(g, x, y - 1, k))), 8),
-                      l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y + 2, k)), ldl(Lf, limb_plane_off<NEAR>(g, x, y - 2, k)))));
+    sDy[q] = p4(l_d1(l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y + 1, k)),
+                           ldl(Lf, limb_plane_off<NEAR>(g, x, y - 1, k))),
+                     l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y + 2, k)), ldl(Lf, limb_plane_off<NEAR>(g, x, y - 2, k)))));
   }
   for (int q = tid; q < TXH * (DBY + 4); q += BX * DBY) {
     const int qx = q % TXH, qy = q / TXH;
     const int x = i0 - 2 + qx, y = j0 - 2 + qy;
-    sDz[q] = p4(l_sub(l_mul(l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y, k + 1)),
-                                  ldl(Lf, limb_plane_off<NEAR>(g, x, y, k - 1))), 8),
-                      l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y, k + 2)), ldl(Lf, limb_plane_off<NEAR>(g, x, y, k - 2)))));
+    sDz[q] = p4(l_d1(l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y, k + 1)),
+                           ldl(Lf, limb_plane_off<NEAR>(g, x, y, k - 1))),
+                     l_sub(ldl(Lf, limb_plane_off<NEAR>(g, x, y, k + 2)), ldl(Lf, limb_plane_off<NEAR>(g, x, y, k - 2)))));
   }
 }
 
 
-// Neighbour sums of one axis at point n: D1 sum 8 (f+1 - f-1) - (f+2 - f-2)
-// and s_k = f(+k) + f(-k), k = 1, 2, 3 (each neighbour loaded once).
+// D1 sum 8 (f+1 - f-1) - (f+2 - f-2) of axis D at point n, and with it
+// s_k = f(+k) + f(-k), k = 1, 2.
 template <int D>
-__device__ __forceinline__ void iaxis(const long long* __restrict__ L, const NbrI& n, int3& d1, int3& s1, int3& s2,
-                                      int3& s3) {
-  const int3 p1 = ldl(L, dispi<D>(n, 1)), m1 = ldl(L, dispi<D>(n, -1));
-  const int3 p2 = ldl(L, dispi<D>(n, 2)), m2 = ldl(L, dispi<D>(n, -2));
-  d1 = l_sub(l_mul(l_sub(p1, m1), 8), l_sub(p2, m2));
+__device__ __forceinline__ void iaxis(const long long* __restrict__ L, const NbrI& n, Limb& d1, Limb& s1, Limb& s2) {
+  const Limb p1 = ldl(L, dispi<D>(n, 1)), m1 = ldl(L, dispi<D>(n, -1));
+  const Limb p2 = ldl(L, dispi<D>(n, 2)), m2 = ldl(L, dispi<D>(n, -2));
+  d1 = l_d1(l_sub(p1, m1), l_sub(p2, m2));
   s1 = l_add(p1, m1);
   s2 = l_add(p2, m2);
-  s3 = l_add(ldl(L, dispi<D>(n, 3)), ldl(L, dispi<D>(n, -3)));
 }
 
-// Field with first derivatives only: D1 along the three axes and the KO term.
-template <class T>
-__device__ __forceinline__ void ideriv_d1_point(const StageArgs& a, int m, const NbrI& n, bool ko_equal) {
+template <int D>
+__device__ __forceinline__ Limb id1(const long long* __restrict__ L, const NbrI& n) {
+  Limb d1, s1, s2;
+  iaxis<D>(L, n, d1, s1, s2);
+  return d1;
+}
+
+// First derivatives of a field that has no second ones.
+template <class T, bool ODD>
+__device__ __forceinline__ void ideriv_d1_point(const StageArgs& a, int m, const NbrI& n, int e) {
   const long fs = a.g.fstride;
-  const Coef& c = a.c;
-  double* __restrict__ D = a.D;
-  constexpr int NDER0 = 3 * T::ND1 + 6 * T::ND2;
-  const int f = T::d1_field(m);
-  const int s = ko_slot<T>(f);
+  const int s = ko_slot<T>(T::d1_field(m));
   const long long* Lf = a.L + (long)s * fs;
-  const int e = max(a.E[s], 1);
-  const int3 f0 = ldl(Lf, n.c);
-  int3 P1 = make_int3(0, 0, 0), P2 = P1, P3 = P1, d1, s1, s2, s3;
-  double ko = 0.0;
-#define COSMOS_IAXIS(AX)                                                                       \
-  iaxis<AX>(Lf, n, d1, s1, s2, s3);                                                            \
-  D[(long)(3 * m + AX) * fs + n.c] = from_limbs(d1, e) * c.d1b[AX];                            \
-  if (ko_equal) {                                                                              \
-    P1 = l_add(P1, s1);                                                                        \
-    P2 = l_add(P2, s2);                                                                        \
-    P3 = l_add(P3, s3);                                                                        \
-  } else {                                                                                     \
-    ko = fma(c.ko[AX], from_limbs(l_mad(f0, -20, l_mad(s2, -6, l_mad(s1, 15, s3))), e), ko);  \
-  }
-  COSMOS_IAXIS(0)
-  COSMOS_IAXIS(1)
-  COSMOS_IAXIS(2)
-#undef COSMOS_IAXIS
-  if (!a.skip_ko) {
-    if (ko_equal) ko = from_limbs(l_mad(f0, -60, l_mad(P2, -6, l_mad(P1, 15, P3))), e);  // scaled in the algebra pass
-    D[(long)(NDER0 + s) * fs + n.c] = ko;
-  }
+  double* __restrict__ D = a.D + (long)(3 * m) * fs + n.c;
+  D[0] = limb_value<ODD>(id1<0>(Lf, n), e) * a.c.d1b[0];
+  D[fs] = limb_value<ODD>(id1<1>(Lf, n), e) * a.c.d1b[1];
+  D[2 * fs] = limb_value<ODD>(id1<2>(Lf, n), e) * a.c.d1b[2];
 }
 
-// Everything the algebra needs from second-derivative field m2 at point n
-// (same outputs and layout as deriv_d2_point), each written as soon as it is
-// formed; D_y and D_z sums come from the staging area.
-template <class T>
-__device__ __forceinline__ void ideriv_d2_point(const StageArgs& a, int m2, const NbrI& n, int tx, int ty,
-                                                bool ko_equal, const int4* __restrict__ sDy,
-                                                const int4* __restrict__ sDz) {
+// First and second derivatives of field m2 at point n, each written as soon as
+// it is formed; D_y and D_z sums come from the staging area.
+template <class T, bool ODD>
+__device__ __forceinline__ void ideriv_d2_point(const StageArgs& a, int m2, const NbrI& n, int e, int tx, int ty,
+                                                const int4* __restrict__ sDy, const int4* __restrict__ sDz) {
   constexpr int TXH = BX + 4;
   const long fs = a.g.fstride;
   const Coef& c = a.c;
   double* __restrict__ D = a.D;
-  constexpr int NDER0 = 3 * T::ND1 + 6 * T::ND2;
   const int f = T::d2_field(m2);
   const int s = ko_slot<T>(f);
   const long long* Lf = a.L + (long)s * fs;
-  const int e = max(a.E[s], 1);
   const int m1 = T::d1_slot(f);
   const long b = (long)(3 * T::ND1 + 6 * m2) * fs + n.c;
-  const int3 f0 = ldl(Lf, n.c);
-  const int3 f30 = l_mul(f0, -30);
-  int3 P1 = make_int3(0, 0, 0), P2 = P1, P3 = P1, d1, s1, s2, s3;
-  double ko = 0.0;
+  const Limb f30 = l_mul(ldl(Lf, n.c), 30);
+  Limb d1, s1, s2;
   // second derivative 16 (f+1 + f-1) - (f+2 + f-2) - 30 f0 of axis AX into slot SL
-#define COSMOS_IAXIS2(AX, SL)                                                                  \
-  iaxis<AX>(Lf, n, d1, s1, s2, s3);                                                            \
-  D[b + SL * fs] = from_limbs(l_sub(l_mad(s1, 16, f30), s2), e) * c.d2b[AX];                   \
-  if (ko_equal) {                                                                              \
-    P1 = l_add(P1, s1);                                                                        \
-    P2 = l_add(P2, s2);                                                                        \
-    P3 = l_add(P3, s3);                                                                        \
-  } else {                                                                                     \
-    ko = fma(c.ko[AX], from_limbs(l_mad(f0, -20, l_mad(s2, -6, l_mad(s1, 15, s3))), e), ko);  \
-  }
+#define COSMOS_IAXIS2(AX, SL)          \
+  iaxis<AX>(Lf, n, d1, s1, s2);        \
+  D[b + SL * fs] = limb_value<ODD>(l_sub(l_sub(l_mul(s1, 16), s2), f30), e) * c.d2b[AX];
   COSMOS_IAXIS2(0, 0)
-  D[(long)(3 * m1 + 0) * fs + n.c] = from_limbs(d1, e) * c.d1b[0];
+  D[(long)(3 * m1 + 0) * fs + n.c] = limb_value<ODD>(d1, e) * c.d1b[0];
   COSMOS_IAXIS2(1, 3)
   COSMOS_IAXIS2(2, 5)
 #undef COSMOS_IAXIS2
-  if (!a.skip_ko) {
-    if (ko_equal) ko = from_limbs(l_mad(f0, -60, l_mad(P2, -6, l_mad(P1, 15, P3))), e);  // scaled in the algebra pass
-    D[(long)(NDER0 + s) * fs + n.c] = ko;
-  }
   const int4* ry = sDy + ty * TXH + tx + 2;        // D_y sums at (i + o, j)
   const int4* rz = sDz + (ty + 2) * TXH + tx + 2;  // D_z sums at (i + o, j), row stride TXH along y
-  D[(long)(3 * m1 + 1) * fs + n.c] = from_limbs(q3(ry[0]), e) * c.d1b[1];
-  D[(long)(3 * m1 + 2) * fs + n.c] = from_limbs(q3(rz[0]), e) * c.d1b[2];
+  D[(long)(3 * m1 + 1) * fs + n.c] = limb_value<ODD>(q3(ry[0]), e) * c.d1b[1];
+  D[(long)(3 * m1 + 2) * fs + n.c] = limb_value<ODD>(q3(rz[0]), e) * c.d1b[2];
   D[b + 1 * fs] =
-      from_limbs(l_sub(l_mul(l_sub(q3(ry[1]), q3(ry[-1])), 8), l_sub(q3(ry[2]), q3(ry[-2]))), e) * c.mix[0];
+      limb_value<ODD>(l_d1(l_sub(q3(ry[1]), q3(ry[-1])), l_sub(q3(ry[2]), q3(ry[-2]))), e) * c.mix[0];
   D[b + 2 * fs] =
-      from_limbs(l_sub(l_mul(l_sub(q3(rz[1]), q3(rz[-1])), 8), l_sub(q3(rz[2]), q3(rz[-2]))), e) * c.mix[1];
-  D[b + 4 * fs] = from_limbs(l_sub(l_mul(l_sub(q3(rz[TXH]), q3(rz[-TXH])), 8),
-                                   l_sub(q3(rz[2 * TXH]), q3(rz[-2 * TXH]))), e) * c.mix[2];
+      limb_value<ODD>(l_d1(l_sub(q3(rz[1]), q3(rz[-1])), l_sub(q3(rz[2]), q3(rz[-2]))), e) * c.mix[1];
+  D[b + 4 * fs] = limb_value<ODD>(l_d1(l_sub(q3(rz[TXH]), q3(rz[-TXH])),
+                                        l_sub(q3(rz[2 * TXH]), q3(rz[-2 * TXH]))), e) * c.mix[2];
 }
 
 // One BX x DBY tile of one z-plane (block of BX x DBY threads); the D_y / D_z
@@ -315,21 +313,28 @@ __device__ __forceinline__ void ideriv_tile(const StageArgs& a, int i0, int j0, 
   const bool valid = i < a.g.nx && j < a.g.ny;
   const NbrI n = make_nbri<NEAR>(a.g, i, j, k);
   const long fs = a.g.fstride;
-  const bool ko_equal = a.c.ko[0] == a.c.ko[1] && a.c.ko[1] == a.c.ko[2];
-  const int f_lo = a.f_lo, f_hi = a.f_hi > 0 ? a.f_hi : (1 << 30);
 #pragma unroll 1
   for (int m = 0; m < T::ND1; ++m) {
-    const int f = T::d1_field(m);
-    if (T::d2_slot(f) >= 0 || f < f_lo || f >= f_hi) continue;
-    if (valid) ideriv_d1_point<T>(a, m, n, ko_equal);
+    if (T::d2_slot(T::d1_field(m)) >= 0) continue;
+    const int e = max(a.E[ko_slot<T>(T::d1_field(m))], 1);
+    if (!valid) continue;
+    if (limb_odd(e))
+      ideriv_d1_point<T, true>(a, m, n, e);
+    else
+      ideriv_d1_point<T, false>(a, m, n, e);
   }
 #pragma unroll 1
   for (int m2 = 0; m2 < T::ND2; ++m2) {
     const int f = T::d2_field(m2);
-    if (f < f_lo || f >= f_hi) continue;  // uniform across the block
     stage_dydz_int<NEAR>(a.g, a.L + (long)ko_slot<T>(f) * fs, i0, j0, k, tid, sDy, sDz);
     __syncthreads();
-    if (valid) ideriv_d2_point<T>(a, m2, n, tx, ty, ko_equal, sDy, sDz);
+    if (valid) {
+      const int e = max(a.E[ko_slot<T>(f)], 1);
+      if (limb_odd(e))
+        ideriv_d2_point<T, true>(a, m2, n, e, tx, ty, sDy, sDz);
+      else
+        ideriv_d2_point<T, false>(a, m2, n, e, tx, ty, sDy, sDz);
+    }
     __syncthreads();
   }
 }
@@ -339,33 +344,6 @@ template <class T, bool NEAR>
 __global__ void __launch_bounds__(BX* DBY, COSMOS_IDERIV_MIN_BLOCKS) ideriv_kernel(const StageArgs a) {
   __shared__ int4 sDy[(BX + 4) * DBY], sDz[(BX + 4) * (DBY + 4)];
   ideriv_tile<T, NEAR>(a, blockIdx.x * BX, blockIdx.y * DBY, blockIdx.z, sDy, sDz);
-}
-
-// Persistent batched integer derivative pass over BX x DBY tiles of every
-// instance.  Each tile's instance arguments are copied to shared memory first:
-// read from there they cannot alias the derivative stores, so they need not
-// be reloaded from global memory after each store.
-template <class T, bool NEAR>
-__global__ void __launch_bounds__(BX* DBY, COSMOS_IDERIV_MIN_BLOCKS)
-    batch_ideriv_kernel(const StageArgs* __restrict__ args, const BatchTile* __restrict__ tiles, long ntiles) {
-  __shared__ int4 sDy[(BX + 4) * DBY], sDz[(BX + 4) * (DBY + 4)];
-  __shared__ StageArgs sa;
-  static_assert(sizeof(StageArgs) % sizeof(long long) == 0, "StageArgs is copied in 8-byte words");
-  constexpr int W = (int)(sizeof(StageArgs) / sizeof(long long));
-  const int tid = threadIdx.y * BX + threadIdx.x;
-  int inst = -1;
-  for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
-    const BatchTile t = tiles[w];
-    if (t.inst != inst) {  // uniform across the block
-      __syncthreads();     // every thread is done with the previous instance's arguments
-      const long long* src = reinterpret_cast<const long long*>(args + t.inst);
-      long long* dst = reinterpret_cast<long long*>(&sa);
-      for (int q = tid; q < W; q += BX * DBY) dst[q] = src[q];
-      __syncthreads();
-      inst = t.inst;
-    }
-    ideriv_tile<T, NEAR>(sa, t.a * BX, t.b * DBY, t.c, sDy, sDz);
-  }
 }
 
 }  // namespace cosmos

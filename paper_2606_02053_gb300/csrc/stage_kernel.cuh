@@ -1,26 +1,13 @@
-// BSSN right-hand side + RK4 stage, as two passes per stage:
-//
-//  * derivative pass: for one BX x DBY tile of a z-plane, every 4th-order
-//    centred first and second derivative the algebra needs and the
-//    6th-derivative Kreiss-Oliger term of every non-fluid field, written to
-//    the derivative buffer D.  The launchers run it in exact integer
-//    arithmetic on a fixed-point copy of the state (stage_int.cuh:
-//    ideriv_kernel, batch_ideriv_kernel); the launchers refuse arguments
-//    without that copy;
-//  * algebra pass (stage_kernel, batch_stage_kernel): one point per thread,
-//    the generated pointwise BSSN + matter algebra on the state and D, the KO
-//    term or the Kurganov-Tadmor flux divergence, and the RK4 stage combine.
+// Point-wise stencils in FP64 and the kernels that use them: the constraints
+// (constraint_kernel), and the per-variant launchers (COSMOS_DEFINE_VARIANT).
+// The right-hand side with its RK4 stage combine is stage_split.cuh, on the
+// exact integer differences of stage_int.cuh.
 //
 // Every stencil is written so that its large cancellations happen in exact
-// neighbour differences.  Also here: the constraint kernel and the per-variant
-// launchers (COSMOS_DEFINE_VARIANT).
+// neighbour differences.
 #pragma once
 
 #include "common.cuh"
-
-#ifndef COSMOS_STAGE_MIN_BLOCKS
-#define COSMOS_STAGE_MIN_BLOCKS 3  // resident 128-thread blocks per SM the register budget is sized for
-#endif
 
 namespace cosmos {
 
@@ -142,24 +129,6 @@ __device__ __forceinline__ void gather(const double* __restrict__ U, const doubl
   if constexpr (T::FLUID) in[T::NIN - 1] = ldg(prim, n.c);
 }
 
-// ---------------------------------------------------------------------------
-// Stage = derivative pass + algebra pass.
-//
-// Derivative pass (one BX x DBY tile of one z-plane per block): writes every
-// finite difference the algebra needs, and the Kreiss-Oliger term of every
-// non-fluid field, into D (layout: D[3 m + d] first derivative d of the m-th
-// first-derivative field, D[3 ND1 + 6 m + p] second derivative p of the m-th
-// second-derivative field, D[NDER0 + ko_slot(f)] KO term of field f, divided by
-// c.ko[0] when the spacing is equal -- see Coef::ko_s).  For the
-// second-derivative fields the first derivatives along y and z are computed
-// once per tile point (with a 2-point halo) into shared memory, and the mixed
-// derivatives are D_x(D_y f), D_x(D_z f), D_y(D_z f) of those values; along x
-// the neighbour differences d_k = f(+-k) - f0 are shared by D1, D2 and KO.
-// Optional restrictions (StageArgs): a field range f_lo .. f_hi, no KO slots
-// (skip_ko, for the reverse mode), and for the algebra pass a plane range.
-// Algebra pass (any point mapping): the generated pointwise algebra on the
-// state values and D, KO and the fluid flux divergence, and the RK4 combine.
-// ---------------------------------------------------------------------------
 constexpr int TXH = BX + 4;  // tile width with the x halo
 
 template <class T>
@@ -176,103 +145,6 @@ __device__ __forceinline__ long plane_off(const DevGrid& g, int x, int y, int k)
 #include "stage_int.cuh"
 
 namespace cosmos {
-
-// Inputs of the algebra pass at one point, read from global memory where the
-// generated code uses them (state values, then the derivative buffer, then the
-// fluid density), so that no input has to stay live in a register.
-template <class T>
-struct AlgIn {
-  const double* __restrict__ U;
-  const double* __restrict__ D;
-  const double* __restrict__ prim;
-  long fs, c;
-  __device__ __forceinline__ double operator[](int k) const {
-    constexpr int NDER0 = 3 * T::ND1 + 6 * T::ND2;
-    if (k < T::NF) return ldg(U + (long)k * fs, c);
-    if (k < T::NF + NDER0) return ldg(D + (long)(k - T::NF) * fs, c);
-    return ldg(prim, c);
-  }
-};
-
-// The largest biased exponent of v over the warp's active lanes into *E (one
-// atomic per warp): the next stage's reference exponent without a scan of the
-// state (the exponent field of the stored value, as field_exponent_kernel reads).
-__device__ __forceinline__ void record_exponent(unsigned* E, double v) {
-  const unsigned e = (unsigned)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7FFu);
-  const unsigned mask = __activemask();
-  const unsigned m = __reduce_max_sync(mask, e);
-  unsigned lane;
-  asm("mov.u32 %0, %%laneid;" : "=r"(lane));
-  if (lane == (unsigned)(__ffs(mask) - 1)) atomicMax(E, m);
-}
-
-// Output side of the algebra pass: out[f] = r adds the Kreiss-Oliger term (or
-// the fluid flux divergence) and applies the RK4 stage combine of MODE, as
-// soon as the generated code has the value.
-template <class T, int MODE>
-struct AlgOut {
-  const StageArgs& a;
-  long fs, c;
-  long cm[3];
-  struct Slot {
-    const AlgOut& o;
-    int f;
-    __device__ __forceinline__ void operator=(double r) const {
-      const StageArgs& a = o.a;
-      const long fs = o.fs, c = o.c;
-      constexpr int NDER0 = 3 * T::ND1 + 6 * T::ND2;
-      if (T::FLUID && f >= 24 && f < 28) {
-        const double* H = a.flux + (long)(f - 24) * fs;  // direction d at H + 4 d fs
-        r -= (ldg(H, c) - ldg(H, o.cm[0])) * a.c.ih[0];
-        r -= (ldg(H + 4 * fs, c) - ldg(H + 4 * fs, o.cm[1])) * a.c.ih[1];
-        r -= (ldg(H + 8 * fs, c) - ldg(H + 8 * fs, o.cm[2])) * a.c.ih[2];
-      } else {
-        r = fma(a.c.ko_s, ldg(a.D + (long)(NDER0 + ko_slot<T>(f)) * fs, c), r);  // see Coef::ko_s
-      }
-      const long ofs = (long)f * fs + c;
-      if constexpr (MODE == MODE_RHS) {
-        a.out[ofs] = r;
-      } else if constexpr (MODE == MODE_S1) {
-        const double v = fma(a.cdt, r, ldg(a.U0, ofs));
-        a.out[ofs] = v;
-        a.acc[ofs] = r;
-        if (a.E_rec && !(T::FLUID && f >= 24 && f < 28)) record_exponent(a.E_rec + 32 * ko_slot<T>(f), v);
-      } else if constexpr (MODE == MODE_S23) {
-        const double v = fma(a.cdt, r, ldg(a.U0, ofs));
-        a.out[ofs] = v;
-        a.acc[ofs] = fma(a.bk, r, a.acc[ofs]);
-        if (a.E_rec && !(T::FLUID && f >= 24 && f < 28)) record_exponent(a.E_rec + 32 * ko_slot<T>(f), v);
-      } else {
-        a.U0w[ofs] = fma(a.cdt, a.acc[ofs] + r, a.U0w[ofs]);
-      }
-    }
-  };
-  __device__ __forceinline__ Slot operator[](int f) const { return Slot{*this, f}; }
-};
-
-// Algebra pass at one grid point (i, j, k).
-template <class T, int MODE>
-__device__ __forceinline__ void alg_point(const StageArgs& a, const AlgebraParams& ap, int i, int j, int k) {
-  const long fs = a.g.fstride;
-  const long c = ((long)k * a.g.ny + j) * a.g.pitch + i;
-  const AlgIn<T> in{a.U, a.D, a.prim, fs, c};
-  AlgOut<T, MODE> out{a, fs, c, {0, 0, 0}};
-  if constexpr (T::FLUID) {
-    out.cm[0] = c - i + wrap_index(i - 1, a.g.nx);
-    out.cm[1] = c + (long)(wrap_index(j - 1, a.g.ny) - j) * a.g.pitch;
-    out.cm[2] = c + (long)(wrap_index(k - 1, a.g.nz) - k) * a.g.pitch * a.g.ny;
-  }
-  T::rhs(in, out, ap);
-}
-
-template <class T, int MODE>
-__global__ void __launch_bounds__(BX* BY, COSMOS_STAGE_MIN_BLOCKS) stage_kernel(const StageArgs a) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z + a.k_lo;
-  if (i >= a.g.nx || j >= a.g.ny) return;
-  alg_point<T, MODE>(a, a.ap, i, j, k);
-}
 
 // Point (i, j, k) of work item `t` (thread `lane` of the block) of a batch:
 // 2D tiles of blockDim.x x blockDim.y points in one z-plane, or runs of
@@ -293,36 +165,6 @@ __device__ __forceinline__ bool batch_point(const BatchTile& t, const DevGrid& g
   j = (int)((p / g.nx) % g.ny);
   k = (int)(p / ((long)g.nx * g.ny));
   return true;
-}
-
-// Persistent batched algebra pass: blocks stride over the flat work list of
-// all instances; instance `inst` uses args[inst] with K_ref taken from kref.
-// The instance's arguments are copied to shared memory when the instance
-// changes: read from there they cannot alias the pass's stores.
-template <class T, int MODE>
-__global__ void __launch_bounds__(BX* BY, COSMOS_STAGE_MIN_BLOCKS)
-    batch_stage_kernel(const StageArgs* __restrict__ args, const BatchTile* __restrict__ tiles, long ntiles,
-                       int mapping, const double* __restrict__ kref) {
-  __shared__ StageArgs sa;
-  static_assert(sizeof(StageArgs) % sizeof(long long) == 0, "StageArgs is copied in 8-byte words");
-  constexpr int W = (int)(sizeof(StageArgs) / sizeof(long long));
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x, nthr = blockDim.x * blockDim.y;
-  int inst = -1;
-  for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
-    const BatchTile t = tiles[w];
-    if (t.inst != inst) {  // uniform across the block
-      __syncthreads();     // every thread is done with the previous instance's arguments
-      const long long* src = reinterpret_cast<const long long*>(args + t.inst);
-      long long* dst = reinterpret_cast<long long*>(&sa);
-      for (int q = tid; q < W; q += nthr) dst[q] = src[q];
-      __syncthreads();
-      inst = t.inst;
-    }
-    AlgebraParams ap = sa.ap;
-    ap.Kref = kref[t.inst];
-    int i, j, k;
-    if (batch_point(t, sa.g, mapping, i, j, k)) alg_point<T, MODE>(sa, ap, i, j, k);
-  }
 }
 
 // Constraints H, M^i per point plus per-block partial norms.
@@ -390,55 +232,37 @@ __global__ void __launch_bounds__(BX* BY, 2) constraint_kernel(const ConstraintA
     __device__ static constexpr int d2_field(int m) { return alg_##NAME::d2_field(m); }                        \
     __device__ static constexpr int d1_slot(int f) { return alg_##NAME::d1_slot(f); }                          \
     __device__ static constexpr int d2_slot(int f) { return alg_##NAME::d2_slot(f); }                          \
-    template <class In, class Out>                                                                              \
-    __device__ static __forceinline__ void rhs(const In& in, Out&& out, const AlgebraParams& p) {               \
-      alg_##NAME::rhs(in, out, p);                                                                              \
-    }                                                                                                           \
+    static constexpr bool SPLIT_EARLY = alg_##NAME::SPLIT_EARLY;                                                    \
+    static constexpr int SA = alg_##NAME::SA, SB = alg_##NAME::SB;                                                  \
+    __device__ static constexpr int out_slot(int f) { return alg_##NAME::out_slot(f); }                             \
+    template <class InA, class InB, class Out, class Next>                                                          \
+    __device__ static __forceinline__ void rhs_split(const InA& ina, const InB& inb, Out&& out, Next&& next,        \
+                                                     const AlgebraParams& p) {                                      \
+      alg_##NAME::rhs_split(ina, inb, out, next, p);                                                                \
+    }                                                                                                               \
     __device__ static __forceinline__ void constraints(const double* in, double* out, const AlgebraParams& p) {  \
       alg_##NAME::constraints(in, out, p);                                                                      \
     }                                                                                                           \
   };                                                                                                            \
-  cudaError_t launch_stage_##NAME(const StageArgs& a, int mode, cudaStream_t s) {                               \
-    dim3 grid = point_grid(a.g), block(BX, BY);                                                                \
-    if (a.k_cnt > 0) grid.z = a.k_cnt;                                                                          \
-    if (mode < 0 || !(mode & 8)) {                                                                            \
-      if (!a.L) return cudaErrorInvalidValue; /* the derivative pass reads the limb copy */                     \
-      if (near_indices(a.g))                                                                                    \
-        ideriv_kernel<T_##NAME, true><<<ideriv_grid(a.g), dim3(BX, DBY), 0, s>>>(a);                            \
-      else                                                                                                      \
-        ideriv_kernel<T_##NAME, false><<<ideriv_grid(a.g), dim3(BX, DBY), 0, s>>>(a);                           \
-    }                                                                                                           \
-    if (mode < 0) return cudaGetLastError();                                                                    \
-    switch (mode & 7) {                                                                                             \
-      case MODE_RHS: stage_kernel<T_##NAME, MODE_RHS><<<grid, block, 0, s>>>(a); break;                        \
-      case MODE_S1: stage_kernel<T_##NAME, MODE_S1><<<grid, block, 0, s>>>(a); break;                          \
-      case MODE_S23: stage_kernel<T_##NAME, MODE_S23><<<grid, block, 0, s>>>(a); break;                        \
-      default: stage_kernel<T_##NAME, MODE_S4><<<grid, block, 0, s>>>(a); break;                               \
-    }                                                                                                           \
-    return cudaGetLastError();                                                                                  \
-  }                                                                                                             \
-  cudaError_t launch_batch_stage_##NAME(const StageArgs* args, const BatchTile* tiles, long ntiles, int mapping,  \
-                                        const double* kref, int mode, dim3 grid, dim3 block, cudaStream_t s,      \
-                                        const BatchTile* dtiles, long ndtiles, int ideriv_blocks,                 \
-                                        bool ideriv_near) {                                                       \
-    if (ideriv_blocks <= 0) return cudaErrorInvalidValue;                                                       \
-    if (ideriv_near)                                                                                            \
-      batch_ideriv_kernel<T_##NAME, true><<<ideriv_blocks, dim3(BX, DBY), 0, s>>>(args, dtiles, ndtiles);       \
-    else                                                                                                        \
-      batch_ideriv_kernel<T_##NAME, false><<<ideriv_blocks, dim3(BX, DBY), 0, s>>>(args, dtiles, ndtiles);      \
-    switch (mode) {                                                                                             \
-      case MODE_S1:                                                                                             \
-        batch_stage_kernel<T_##NAME, MODE_S1><<<grid, block, 0, s>>>(args, tiles, ntiles, mapping, kref);       \
-        break;                                                                                                  \
-      case MODE_S23:                                                                                            \
-        batch_stage_kernel<T_##NAME, MODE_S23><<<grid, block, 0, s>>>(args, tiles, ntiles, mapping, kref);      \
-        break;                                                                                                  \
-      default:                                                                                                  \
-        batch_stage_kernel<T_##NAME, MODE_S4><<<grid, block, 0, s>>>(args, tiles, ntiles, mapping, kref);       \
-        break;                                                                                                  \
-    }                                                                                                           \
-    return cudaGetLastError();                                                                                  \
-  }                                                                                                             \
+  cudaError_t launch_stage_##NAME(const StageArgs& a, int mode, int k_cnt, cudaStream_t s) {                        \
+    if (!a.L) return cudaErrorInvalidValue; /* the differences are those of the limb copy */                        \
+    const long tiles = (long)((a.g.nx + SPLIT_TX - 1) / SPLIT_TX) * ((a.g.ny + SPLIT_TY - 1) / SPLIT_TY) * k_cnt;   \
+    return launch_split<T_##NAME, false>(a, nullptr, nullptr, tiles, nullptr, mode, a.eq, s);                             \
+  }                                                                                                                 \
+  cudaError_t launch_deriv_##NAME(const StageArgs& a, cudaStream_t s) {                                             \
+    if (!a.L) return cudaErrorInvalidValue;                                                                         \
+    if (near_indices(a.g))                                                                                          \
+      ideriv_kernel<T_##NAME, true><<<ideriv_grid(a.g), dim3(BX, DBY), 0, s>>>(a);                                  \
+    else                                                                                                            \
+      ideriv_kernel<T_##NAME, false><<<ideriv_grid(a.g), dim3(BX, DBY), 0, s>>>(a);                                 \
+    return cudaGetLastError();                                                                                      \
+  }                                                                                                                 \
+  cudaError_t launch_batch_stage_##NAME(const StageArgs* args, const BatchTile* tiles, long ntiles,                 \
+                                        const double* kref, int mode, bool eq, cudaStream_t s) {                             \
+    StageArgs none;                                                                                                 \
+    memset(&none, 0, sizeof(none));                                                                                 \
+    return launch_split<T_##NAME, true>(none, args, tiles, ntiles, kref, mode, eq, s);                                  \
+  }                                                                                                                 \
   cudaError_t launch_constraints_##NAME(const ConstraintArgs& a, cudaStream_t s) {                              \
     constraint_kernel<T_##NAME><<<point_grid(a.g), dim3(BX, BY), 0, s>>>(a);                                    \
     return cudaGetLastError();                                                                                  \

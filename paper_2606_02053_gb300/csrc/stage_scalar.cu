@@ -1,5 +1,5 @@
 // Stage / RHS / constraint kernels for the "scalar" matter variant.
-#include "stage_kernel.cuh"
+#include "stage_split.cuh"
 
 namespace cosmos {
 COSMOS_DEFINE_VARIANT(scalar, false, true)

@@ -1,0 +1,682 @@
+// One RK4 stage as one persistent kernel: finite differences, pointwise
+// algebra and stage combine of a tile side by side in one block.
+//
+// What bounds it: the algebra is FP64 work (799 instructions per point in
+// vacuum, Kreiss-Oliger terms included) at 2 multiply-adds per clock per SM
+// (lone multiplies and adds 1.7), and one warp per scheduler nearly keeps that
+// pipe full (a dependent chain of one warp issues one multiply-add per 64
+// cycles, its whole rate).  The finite differences are integer work
+// (stage_int.cuh) on units that the algebra leaves idle.  As two kernels one
+// after the other each left the other's units idle, and the 162 differences
+// per point travelled through memory.  Here a block has one algebra warpgroup
+// with 200 registers a thread and SPLIT_GROUPS difference warpgroups with 104,
+// and the differences of a tile (SPLIT_TX x SPLIT_TY points of one z-plane, a
+// point per algebra thread) go through shared memory.  256^3 vacuum stage: 10.0
+// + 27.5 ms as two kernels, 32.5 ms as this one (FP64 pipe 83% busy; its algebra
+// alone 29.5, its differences alone 25); 128^3 fluid 5.4 -> 4.8 ms; 20 x 12 x 9 145 ->
+// 40 us.  The algebra with 240 or 224 registers, the difference warps with 88 or 96,
+// and four groups of 64 were within 1 to 3% and slower.
+//
+// The algebra runs in two phases of about equal length (codegen/bssn.py,
+// split_layout): the first reads region A (conformal metric and Gamma: the
+// Ricci tensor), the second region B (everything else).  While the first
+// phase works on a tile the difference warps fill its region B, while the second does
+// they fill region A of the next tile, so neither region needs a second copy.
+// The second phase leaves its outputs in region B, and the difference warps do
+// the stage combine with them (their many threads hide the latency of the
+// state and accumulator loads that one algebra warp per scheduler could not).
+//
+//   algebra warps:     | wait A(t) | phase 1 | free A | wait B(t) | phase 2, r -> B | done |
+//   difference warps:  | fill B(t) | wait free A | fill A(t+1) | wait done | combine(t) |
+//
+// Units: with l = 12 h_x as the unit of length every difference of equal
+// spacing is its exact integer sum, rounded once, without a factor: 12 h d_k f,
+// (12 h)^2 d_k d_k f = 3 (16 s1 - s2 - 30 f0) 2^2 and (12 h)^2 d_a d_b f are the
+// digit sums themselves.  Fields that carry inverse lengths (K, At, Gt, B, Pi:
+// one; tau, S, rho: two) are scaled by l or l^2 where they enter, and the
+// outputs by a power of 1/l in the stage combine, where a factor is there
+// anyway.  K - K_ref is formed before the scaling (it cancels).
+#pragma once
+
+#include "stage_kernel.cuh"
+
+namespace cosmos {
+
+constexpr int SPLIT_PTS = SPLIT_TX * SPLIT_TY;
+constexpr int SPLIT_GROUPS = 3;  // difference warpgroups
+constexpr int SPLIT_THREADS = SPLIT_PTS * (1 + SPLIT_GROUPS);
+static_assert(SPLIT_PTS == 128, "one point per thread of a warpgroup");
+// Registers: the pool is the launch's SPLIT_THREADS x (65536 / SPLIT_THREADS,
+// rounded down to 8); the two shares below add up to no more than it.
+constexpr int SPLIT_POOL = (65536 / SPLIT_THREADS) & ~7;
+#ifndef COSMOS_SPLIT_REG_DIFF
+#define COSMOS_SPLIT_REG_DIFF 104
+#define COSMOS_SPLIT_REG_ALG 200
+#endif
+constexpr int SPLIT_REG_DIFF = COSMOS_SPLIT_REG_DIFF;
+constexpr int SPLIT_REG_ALG = COSMOS_SPLIT_REG_ALG;
+static_assert(SPLIT_REG_ALG + SPLIT_GROUPS * SPLIT_REG_DIFF <= SPLIT_POOL * (1 + SPLIT_GROUPS), "register shares");
+// Staged D_y (tile rows) and D_z (rows with a 2-point halo) sums, both with a
+// 2-point halo along x.
+constexpr int SPLIT_XH = SPLIT_TX + 4;
+constexpr int SPLIT_NDY = SPLIT_XH * SPLIT_TY, SPLIT_NDZ = SPLIT_XH * (SPLIT_TY + 4);
+// Periodic offsets of the rows, columns and planes a tile touches (3-point halo)
+constexpr int SPLIT_NXW = SPLIT_TX + 6, SPLIT_NYW = SPLIT_TY + 6, SPLIT_NZW = 7;
+
+// Named barriers (0 is left to __syncthreads)
+constexpr int BAR_FULL_A = 1, BAR_FREE_A = 2, BAR_FULL_B = 3, BAR_DONE_B = 4, BAR_DIFF = 5, BAR_GROUP = 6;
+
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Region layouts (the order of codegen/bssn.py, split_layout).
+template <class T>
+struct Slots {
+  static constexpr int A = T::SA, B = T::SB;
+  // region A: 6 x 10 (metric), 3 x 4 (Gamma), metric, shift, At (SPLIT_EARLY), fluid: chi, tau, S_i, rho
+  static constexpr int A_GT = 0, A_GAM = 60, A_STATE = 72;
+  static constexpr int A_NSTATE = 9 + (T::SPLIT_EARLY ? 6 : 0) + (T::FLUID ? 6 : 0);
+  // region B: ND2B x 10 (chi, alpha, beta^i, phi), K (4), merged advections, states, output slots
+  static constexpr int ND2B = 5 + (T::SCALAR ? 1 : 0), NM = 9 + (T::SCALAR ? 1 : 0);
+  static constexpr int B_K = 10 * ND2B, B_M = B_K + 4, B_STATE = B_M + NM;
+  static constexpr int B_NSTATE = 22 + (T::FLUID ? 5 : 0) + (T::SCALAR ? 1 : 0);
+  static constexpr int PHI = T::FLUID ? 28 : 24;
+  static_assert(A == A_STATE + A_NSTATE, "region A");
+  static_assert(B == B_STATE + B_NSTATE + 9 + (T::FLUID ? 4 : 0), "region B");
+  // field of the m-th second-derivative block of region B
+  __device__ static __forceinline__ int b_d2(int m) { return m == 0 ? 0 : (m == 1 ? 17 : (m < 5 ? 16 + m : PHI)); }
+  // field of the m-th merged advection
+  __device__ static __forceinline__ int b_m(int m) { return m < 6 ? 8 + m : (m < 9 ? 15 + m : PHI + 1); }
+  // field of the s-th state of each region, -1 for rho
+  __device__ static constexpr int a_state(int s) {
+    constexpr int E = T::SPLIT_EARLY ? 15 : 9;
+    return s < 6 ? 1 + s : (s < 9 ? 12 + s : (s < E ? s - 1 : (s == E ? 0 : (s < E + 5 ? 23 + s - E : -1))));
+  }
+  __device__ static constexpr int b_state(int s) {  // slot 21 is K - K_ref
+    return s < 14 ? s : (s < 21 ? s + 3 : (s == 21 ? 7 : (T::FLUID ? (s < 26 ? s + 2 : (s == 26 ? -1 : 29)) : 25)));
+  }
+  // powers of the unit of length on a state (B^i enters without its own)
+  __device__ static constexpr int state_degree(int f) {
+    return f < 0 ? 2 : (f >= 21 && f < 24 ? 0 : degree(f));
+  }
+  // powers of the unit of length that field f (and its time derivative, one more) carries
+  __device__ static constexpr int degree(int f) {
+    if (f >= 24) return (T::FLUID && f < 28) ? 2 : (f == PHI ? 0 : 1);
+    return ((f >= 7 && f <= 16) || f >= 21) ? 1 : 0;
+  }
+};
+
+template <class T>
+constexpr size_t split_smem_bytes() {
+  return sizeof(double) * SPLIT_PTS * (T::SA + T::SB) + sizeof(int4) * SPLIT_GROUPS * (SPLIT_NDY + SPLIT_NDZ) +
+         sizeof(int) * (SPLIT_GROUPS * (48 + 32) + 32);
+}
+
+// Tile w of the plane range of one grid, or of a batch's tile list.
+struct SplitTile {
+  int i0, j0, k, inst;
+};
+
+struct SlotIn {
+  const double* s;
+  __device__ __forceinline__ double operator[](int k) const { return s[k * SPLIT_PTS]; }
+};
+
+template <class T>
+struct SlotOut {
+  double* s;
+  struct Slot {
+    double* p;
+    __device__ __forceinline__ void operator=(double v) const { *p = v; }
+  };
+  __device__ __forceinline__ Slot operator[](int f) const { return Slot{s + T::out_slot(f) * SPLIT_PTS}; }
+};
+
+// What a difference thread needs of a tile and its instance.  Offsets are in
+// bytes within one field, 32 bits (a field of 4 GiB or more cannot be held
+// with the other fields and buffers of a stage in the device's memory): added
+// to a field's base, which is uniform, they need no 64-bit arithmetic.
+struct DiffCtx {
+  const char* L;
+  const char* U;
+  long fb;           // bytes of one field
+  unsigned o[3][6];  // neighbours -3, -2, -1, 1, 2, 3 along each axis
+  unsigned c;        // the point itself (clamped into the grid)
+  unsigned b[4];     // staged sums q = t + 128 j of this thread: offset without the axis differenced,
+  int p[4];          // and the place of the centre along that axis in the offset tables
+  double r[3];       // h_x / h_d (unequal spacing)
+};
+
+__device__ __forceinline__ long long ldv(const char* __restrict__ base, unsigned o) {
+  return __ldg(reinterpret_cast<const long long*>(base + o));
+}
+__device__ __forceinline__ double ldd(const char* __restrict__ base, unsigned o) {
+  return __ldg(reinterpret_cast<const double*>(base + o));
+}
+
+template <class T, bool EQ>
+struct DiffGroup {
+  const int t;     // thread of the group = point of the tile
+  const int g;     // group
+  double* sA;      // region A + t
+  double* sB;      // region B + t
+  int4* sDy;       // staged D_y sums, the D_z sums after them
+  unsigned* xw;    // periodic offsets: columns i0 - 3 .., then rows, then planes
+  int* ex;         // reference exponents
+  int* rec;        // largest exponents written so far (all groups)
+
+  __device__ __forceinline__ void sync() const { bar_sync(BAR_GROUP + g, SPLIT_PTS); }
+
+  // Offsets of the tile for this group; every thread of the group calls it.
+  __device__ __forceinline__ void begin(const StageArgs& a, const SplitTile& w, DiffCtx& x) const {
+    sync();  // the group is done with the tables of the tile before
+    constexpr int NSLOT = 24 + (T::SCALAR ? 2 : 0);
+    const unsigned row = 8u * (unsigned)a.g.pitch, plane = row * (unsigned)a.g.ny;
+    if (t < SPLIT_NXW)
+      xw[t] = 8u * (unsigned)wrap_index(w.i0 - 3 + t, a.g.nx);
+    else if (t < SPLIT_NXW + SPLIT_NYW)
+      xw[t] = row * (unsigned)wrap_index(w.j0 - 3 + t - SPLIT_NXW, a.g.ny);
+    else if (t < SPLIT_NXW + SPLIT_NYW + SPLIT_NZW)
+      xw[t] = plane * (unsigned)wrap_index(w.k - 3 + t - SPLIT_NXW - SPLIT_NYW, a.g.nz);
+    else if (t >= 64 && t < 64 + NSLOT)
+      ex[t - 64] = max(a.E[t - 64], 1);
+    sync();
+    const unsigned *yw = xw + SPLIT_NXW, *zw = yw + SPLIT_NYW;
+    // threads past the edge take the last column / row: their results are not stored
+    const int tx = min(t % SPLIT_TX, a.g.nx - 1 - w.i0), ty = min(t / SPLIT_TX, a.g.ny - 1 - w.j0);
+    const unsigned cx = xw[tx + 3], cy = yw[ty + 3], cz = zw[3];
+    x.c = cx + cy + cz;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const int p = q < 3 ? q : q + 1;
+      x.o[0][q] = xw[tx + p] + cy + cz;
+      x.o[1][q] = cx + yw[ty + p] + cz;
+      x.o[2][q] = cx + cy + zw[p];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int q = t + SPLIT_PTS * j, z = q - SPLIT_NDY;
+      if (q < SPLIT_NDY) {
+        x.b[j] = xw[q % SPLIT_XH + 1] + cz;
+        x.p[j] = SPLIT_NXW + q / SPLIT_XH + 3;
+      } else {
+        x.b[j] = q < SPLIT_NDY + SPLIT_NDZ ? xw[z % SPLIT_XH + 1] + yw[z / SPLIT_XH + 1] : 0u;
+        x.p[j] = SPLIT_NXW + SPLIT_NYW + 3;
+      }
+    }
+    x.L = reinterpret_cast<const char*>(a.L);
+    x.U = reinterpret_cast<const char*>(a.U);
+    x.fb = 8 * a.g.fstride;
+    if (!EQ) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x.r[d] = a.ratio[d];
+    }
+  }
+
+  // The values a point's stencils need, all loads in flight at once.
+  struct Values {
+    long long c, n[3][6];
+  };
+  __device__ __forceinline__ Values load(const DiffCtx& x, const char* __restrict__ L) const {
+    Values v;
+    v.c = ldv(L, x.c);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int q = 0; q < 6; ++q) v.n[d][q] = ldv(L, x.o[d][q]);
+    return v;
+  }
+
+  // D1 sum and s_k = f(+k) + f(-k) along one axis
+  __device__ __forceinline__ static void axis(const long long (&n)[6], Limb& d1, Limb& s1, Limb& s2, Limb& s3) {
+    const Limb p1 = limb_of(n[3]), m1 = limb_of(n[2]), p2 = limb_of(n[4]), m2 = limb_of(n[1]);
+    d1 = l_d1(l_sub(p1, m1), l_sub(p2, m2));
+    s1 = l_add(p1, m1);
+    s2 = l_add(p2, m2);
+    s3 = l_add(limb_of(n[5]), limb_of(n[0]));
+  }
+  // 3 (16 s1 - s2 - 30 f0), f30 = 30 f0: 2^2 of the factor 12 goes into the exponent
+  __device__ __forceinline__ static Limb second(Limb s1, Limb s2, Limb f30) {
+    return l_mul(l_sub(l_sub(l_mul(s1, 16), s2), f30), 3);
+  }
+  // s3 - 6 s2 + 15 s1 - f20, f20 = 20 f0 per axis in the sums
+  __device__ __forceinline__ static Limb bracket(Limb s1, Limb s2, Limb s3, Limb f20) {
+    return l_add(s3, l_sub(l_mul(l_sub(l_mul(s1, 5), l_mul(s2, 2)), 3), f20));
+  }
+
+  // Ten slots of a second-derivative field (all of degree 0): d_k, dd_p, KO bracket.
+  template <bool ODD>
+  __device__ __forceinline__ void d2_slots(const DiffCtx& x, const char* __restrict__ L, int e, double* dst) const {
+    // D_y and D_z sums of the tile with their halos; every load in flight before the first use
+    long long r[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (t + SPLIT_PTS * j < SPLIT_NDY + SPLIT_NDZ) {
+        r[j][0] = ldv(L, x.b[j] + xw[x.p[j] - 2]);
+        r[j][1] = ldv(L, x.b[j] + xw[x.p[j] - 1]);
+        r[j][2] = ldv(L, x.b[j] + xw[x.p[j] + 1]);
+        r[j][3] = ldv(L, x.b[j] + xw[x.p[j] + 2]);
+      }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (t + SPLIT_PTS * j < SPLIT_NDY + SPLIT_NDZ)
+        sDy[t + SPLIT_PTS * j] =
+            p4(l_d1(l_sub(limb_of(r[j][2]), limb_of(r[j][1])), l_sub(limb_of(r[j][3]), limb_of(r[j][0]))));
+    const Values n = load(x, L);
+    const Limb f0 = limb_of(n.c), f30 = l_mul(f0, 30);
+    Limb d1, s1, s2, s3;
+    if (EQ) {
+      Limb P1, P2, P3, yy;
+      axis(n.n[0], d1, P1, P2, P3);
+      {
+        const Limb S[2] = {d1, second(P1, P2, f30)};
+        const int ee[2] = {e, e + 2};
+        double v[2];
+        limb_values<ODD>(S, ee, v);
+        dst[0] = v[0];
+        dst[3 * SPLIT_PTS] = v[1];
+      }
+      axis(n.n[1], d1, s1, s2, s3);
+      yy = second(s1, s2, f30);
+      P1 = l_add(P1, s1);
+      P2 = l_add(P2, s2);
+      P3 = l_add(P3, s3);
+      axis(n.n[2], d1, s1, s2, s3);
+      P1 = l_add(P1, s1);
+      P2 = l_add(P2, s2);
+      P3 = l_add(P3, s3);
+      const Limb S[3] = {yy, second(s1, s2, f30), bracket(P1, P2, P3, l_mul(f30, 2))};
+      const int ee[3] = {e + 2, e + 2, e};
+      double v[3];
+      limb_values<ODD>(S, ee, v);
+      dst[6 * SPLIT_PTS] = v[0];
+      dst[8 * SPLIT_PTS] = v[1];
+      dst[9 * SPLIT_PTS] = v[2];
+    } else {
+      const Limb f20 = l_mul(f0, 20);
+      double ko = 0.0;
+#define COSMOS_SPLIT_AXIS(AX, SL)                                               \
+  {                                                                             \
+    axis(n.n[AX], d1, s1, s2, s3);                                              \
+    const Limb S[3] = {d1, second(s1, s2, f30), bracket(s1, s2, s3, f20)};      \
+    const int ee[3] = {e, e + 2, e};                                            \
+    double v[3];                                                                \
+    limb_values<ODD>(S, ee, v);                                                 \
+    if (AX == 0) dst[0] = v[0];                                                 \
+    dst[SL * SPLIT_PTS] = v[1] * (x.r[AX] * x.r[AX]);                           \
+    ko = fma(x.r[AX], v[2], ko);                                                \
+  }
+      COSMOS_SPLIT_AXIS(0, 3)
+      COSMOS_SPLIT_AXIS(1, 6)
+      COSMOS_SPLIT_AXIS(2, 8)
+#undef COSMOS_SPLIT_AXIS
+      dst[9 * SPLIT_PTS] = ko;
+    }
+    sync();
+    const int4* ry = sDy + (t / SPLIT_TX) * SPLIT_XH + t % SPLIT_TX + 2;
+    const int4* rz = sDy + SPLIT_NDY + (t / SPLIT_TX + 2) * SPLIT_XH + t % SPLIT_TX + 2;
+    auto mixed = [](const int4* r, int st) {
+      return l_d1(l_sub(q3(r[st]), q3(r[-st])), l_sub(q3(r[2 * st]), q3(r[-2 * st])));
+    };
+    const Limb S[5] = {q3(ry[0]), q3(rz[0]), mixed(ry, 1), mixed(rz, 1), mixed(rz, SPLIT_XH)};
+    const int ee[5] = {e, e, e, e, e};
+    double v[5];
+    limb_values<ODD>(S, ee, v);
+    if (!EQ) {
+      v[0] *= x.r[1];
+      v[1] *= x.r[2];
+      v[2] *= x.r[1];
+      v[3] *= x.r[2];
+      v[4] *= x.r[1] * x.r[2];
+    }
+    dst[1 * SPLIT_PTS] = v[0];
+    dst[2 * SPLIT_PTS] = v[1];
+    dst[4 * SPLIT_PTS] = v[2];
+    dst[5 * SPLIT_PTS] = v[3];
+    dst[7 * SPLIT_PTS] = v[4];
+    sync();
+  }
+
+  __device__ __forceinline__ void d2_field(const DiffCtx& x, int f, double* dst) const {
+    const int s = ko_slot<T>(f), e = ex[s];
+    const char* __restrict__ L = x.L + s * x.fb;
+    if (limb_odd(e))
+      d2_slots<true>(x, L, e, dst);
+    else
+      d2_slots<false>(x, L, e, dst);
+  }
+
+  // First derivatives (v[0 .. 2]) and KO bracket (v[3]) of field f.
+  template <bool ODD>
+  __device__ __forceinline__ void d1_values(const DiffCtx& x, const char* __restrict__ L, int e, double (&v)[4]) const {
+    const Values n = load(x, L);
+    const Limb f0 = limb_of(n.c);
+    Limb D[3], s1, s2, s3;
+    if (EQ) {
+      Limb P1, P2, P3;
+      axis(n.n[0], D[0], P1, P2, P3);
+      axis(n.n[1], D[1], s1, s2, s3);
+      P1 = l_add(P1, s1);
+      P2 = l_add(P2, s2);
+      P3 = l_add(P3, s3);
+      axis(n.n[2], D[2], s1, s2, s3);
+      P1 = l_add(P1, s1);
+      P2 = l_add(P2, s2);
+      P3 = l_add(P3, s3);
+      const Limb S[4] = {D[0], D[1], D[2], bracket(P1, P2, P3, l_mul(f0, 60))};
+      const int ee[4] = {e, e, e, e};
+      limb_values<ODD>(S, ee, v);
+    } else {
+      const Limb f20 = l_mul(f0, 20);
+      const int ee[2] = {e, e};
+      v[3] = 0.0;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        axis(n.n[d], D[d], s1, s2, s3);
+        const Limb S[2] = {D[d], bracket(s1, s2, s3, f20)};
+        double w[2];
+        limb_values<ODD>(S, ee, w);
+        v[d] = w[0] * x.r[d];
+        v[3] = fma(x.r[d], w[1], v[3]);
+      }
+    }
+  }
+
+  __device__ __forceinline__ void d1_sums(const DiffCtx& x, int f, double (&v)[4]) const {
+    const int s = ko_slot<T>(f), e = ex[s];
+    const char* __restrict__ L = x.L + s * x.fb;
+    if (limb_odd(e))
+      d1_values<true>(x, L, e, v);
+    else
+      d1_values<false>(x, L, e, v);
+  }
+
+  // Four slots of a field.
+  __device__ __forceinline__ void d1_field(const DiffCtx& x, int f, double* dst) const {
+    double v[4];
+    d1_sums(x, f, v);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) dst[q * SPLIT_PTS] = v[q];
+  }
+
+  // State values into their slots (G = the group, known at compile time, so that fields and factors are):
+  // every SPLIT_GROUPS-th slot of the region, all loads in flight at once.
+  template <int G>
+  __device__ __forceinline__ void state_a(const StageArgs& a, const DiffCtx& x) const {
+    using S = Slots<T>;
+    constexpr int N = (S::A_NSTATE - G + SPLIT_GROUPS - 1) / SPLIT_GROUPS;
+    double st[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int f = S::a_state(G + q * SPLIT_GROUPS);
+      st[q] = f < 0 ? ldd(reinterpret_cast<const char*>(a.prim), x.c) : ldd(x.U + f * x.fb, x.c);
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int s = G + q * SPLIT_GROUPS, d = S::state_degree(S::a_state(s));
+      sA[(S::A_STATE + s) * SPLIT_PTS] = d == 2 ? st[q] * a.len2 : (d == 1 ? st[q] * a.len : st[q]);
+    }
+  }
+
+  template <int G>
+  __device__ __forceinline__ void state_b(const StageArgs& a, double kref, const DiffCtx& x) const {
+    using S = Slots<T>;
+    constexpr int N = (S::B_NSTATE - G + SPLIT_GROUPS - 1) / SPLIT_GROUPS;
+    double st[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int f = S::b_state(G + q * SPLIT_GROUPS);
+      st[q] = f < 0 ? ldd(reinterpret_cast<const char*>(a.prim), x.c) : ldd(x.U + f * x.fb, x.c);
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int s = G + q * SPLIT_GROUPS, d = S::state_degree(S::b_state(s));
+      // slot 21 holds K - K_ref, which cancels: formed before any scaling
+      sB[(S::B_STATE + s) * SPLIT_PTS] =
+          s == 21 ? st[q] - kref : (d == 2 ? st[q] * a.len2 : (d == 1 ? st[q] * a.len : st[q]));
+    }
+  }
+
+  __device__ __forceinline__ void fill_a(const StageArgs& a, const SplitTile& w) const {
+    using S = Slots<T>;
+    DiffCtx x;
+    begin(a, w, x);
+    if (g == 0)
+      state_a<0>(a, x);
+    else if (g == 1)
+      state_a<1>(a, x);
+    else
+      state_a<2>(a, x);
+#pragma unroll 1
+    for (int m = g; m < 6; m += SPLIT_GROUPS) d2_field(x, 1 + m, sA + (S::A_GT + 10 * m) * SPLIT_PTS);
+    d1_field(x, 14 + g, sA + (S::A_GAM + 4 * g) * SPLIT_PTS);
+  }
+
+  __device__ __forceinline__ void fill_b(const StageArgs& a, double kref, const SplitTile& w) const {
+    using S = Slots<T>;
+    DiffCtx x;
+    begin(a, w, x);
+    if (g == 0)
+      state_b<0>(a, kref, x);
+    else if (g == 1)
+      state_b<1>(a, kref, x);
+    else
+      state_b<2>(a, kref, x);
+#pragma unroll 1
+    for (int m = g; m < S::ND2B; m += SPLIT_GROUPS) d2_field(x, S::b_d2(m), sB + 10 * m * SPLIT_PTS);
+    // K and the merged advections, 1 + NM first-derivative fields: the group with fewer
+    // second-derivative fields takes more of them
+    constexpr int NG = T::SCALAR ? 4 : 3;
+    const int lo = g * NG, hi = g == SPLIT_GROUPS - 1 ? 1 + S::NM : lo + NG;
+    const double b0 = ldd(x.U + 18 * x.fb, x.c), b1 = ldd(x.U + 19 * x.fb, x.c), b2 = ldd(x.U + 20 * x.fb, x.c);
+#pragma unroll 1
+    for (int m = lo; m < hi; ++m) {
+      if (m == 0) {
+        d1_field(x, 7, sB + S::B_K * SPLIT_PTS);
+        continue;
+      }
+      const int f = S::b_m(m - 1);
+      double v[4];
+      d1_sums(x, f, v);
+      // l (beta^k d_k f + KO term), with the shift switch on the advection of B^i
+      double q = fma(b0, v[0], fma(b1, v[1], b2 * v[2]));
+      if (f >= 21 && f < 24) q *= a.ap.shift_on;
+      sB[(S::B_M + m - 1) * SPLIT_PTS] = a.len * fma(a.ap.ko, v[3], q);
+    }
+  }
+
+  // Stage combine of the tile's outputs (in their region-B slots): fields G, G + SPLIT_GROUPS, ...
+  template <int G>
+  __device__ __forceinline__ void combine(const StageArgs& a, int mode, const SplitTile& w) const {
+    using S = Slots<T>;
+    const int i = w.i0 + t % SPLIT_TX, j = w.j0 + t / SPLIT_TX;
+    const bool valid = i < a.g.nx && j < a.g.ny;
+    const long fb = 8 * a.g.fstride;
+    const unsigned row = 8u * (unsigned)a.g.pitch, plane = row * (unsigned)a.g.ny;
+    const unsigned c = valid ? plane * (unsigned)w.k + row * (unsigned)j + 8u * (unsigned)i : 0u;
+    const bool add = mode == MODE_S23 || mode == MODE_S4;
+    const char* const u0 = mode == MODE_S4 ? reinterpret_cast<const char*>(a.U0w) : reinterpret_cast<const char*>(a.U0);
+    char* const acc = reinterpret_cast<char*>(a.acc);
+    char* const out = reinterpret_cast<char*>(mode == MODE_S4 ? a.U0w : a.out);
+    constexpr int N = (T::NF - G + SPLIT_GROUPS - 1) / SPLIT_GROUPS;
+    double u[N], ac[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {  // every load in flight before the first use
+      const int f = G + q * SPLIT_GROUPS;
+      u[q] = valid && mode != MODE_RHS ? *reinterpret_cast<const double*>(u0 + f * fb + c) : 0.0;
+      ac[q] = valid && add ? *reinterpret_cast<const double*>(acc + f * fb + c) : 0.0;
+    }
+    // the fluid's fluxes: direction d of field 24 + m at 8 (4 d + m) fs
+    constexpr int F = T::FLUID ? 24 + (G + SPLIT_GROUPS - 24 % SPLIT_GROUPS) % SPLIT_GROUPS : T::NF;
+    constexpr int NFL = T::FLUID ? (27 - F) / SPLIT_GROUPS + 1 : 0;
+    double H[NFL > 0 ? NFL : 1][6];
+    if (T::FLUID) {
+      const unsigned cx = c - 8u * (unsigned)i + 8u * (unsigned)wrap_index(i - 1, a.g.nx);
+      const unsigned cy = c + row * (unsigned)(wrap_index(j - 1, a.g.ny) - j);
+      const unsigned cz = c + plane * (unsigned)(wrap_index(w.k - 1, a.g.nz) - w.k);
+#pragma unroll
+      for (int q = 0; q < NFL; ++q)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const char* h = reinterpret_cast<const char*>(a.flux) + (F + q * SPLIT_GROUPS - 24 + 4 * d) * fb;
+          H[q][2 * d] = valid ? ldd(h, c) : 0.0;
+          H[q][2 * d + 1] = valid ? ldd(h, d == 0 ? cx : (d == 1 ? cy : cz)) : 0.0;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int f = G + q * SPLIT_GROUPS;
+      // r in the units of the grid = factor inv_len of the slot's value; the factor is part
+      // of the products below, except for the fluid (flux divergence), formed here
+      double r = sB[T::out_slot(f) * SPLIT_PTS];
+      int s = S::degree(f);
+      if (T::FLUID && f >= 24 && f < 28) {
+        const int m = (f - F) / SPLIT_GROUPS;
+        r *= a.inv_len[s];
+        s = 3;
+        r -= (H[m][0] - H[m][1]) * a.c.ih[0];
+        r -= (H[m][2] - H[m][3]) * a.c.ih[1];
+        r -= (H[m][4] - H[m][5]) * a.c.ih[2];
+      }
+      double* const o = reinterpret_cast<double*>(out + f * fb + c);
+      if (mode == MODE_RHS) {
+        if (valid) *o = r * a.inv_len[s];
+      } else if (mode == MODE_S4) {
+        if (valid) *o = fma(a.cdt, fma(a.inv_len[s], r, ac[q]), u[q]);
+      } else {
+        const double v = fma(a.cdt_len[s], r, u[q]);
+        if (valid) {
+          *o = v;
+          *reinterpret_cast<double*>(acc + f * fb + c) = mode == MODE_S1 ? r * a.inv_len[s] : fma(a.bk_len[s], r, ac[q]);
+        }
+        if (a.E_rec && !(T::FLUID && f >= 24 && f < 28)) {
+          // largest biased exponent of the stored values (the next stage's reference)
+          const unsigned e = valid ? (unsigned)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7FFu) : 0u;
+          const unsigned m = __reduce_max_sync(0xffffffffu, e);
+          if ((t & 31) == 0) atomicMax(rec + ko_slot<T>(f), (int)m);
+        }
+      }
+    }
+  }
+
+  __device__ __forceinline__ void combine(const StageArgs& a, int mode, const SplitTile& w) const {
+    if (g == 0)
+      combine<0>(a, mode, w);
+    else if (g == 1)
+      combine<1>(a, mode, w);
+    else
+      combine<2>(a, mode, w);
+  }
+};
+
+// BATCH: tiles from a list, arguments per instance with K_ref in kref; else
+// the planes k_lo .. of the grid of `one`.
+template <class T, bool BATCH, bool EQ>
+__global__ void __launch_bounds__(SPLIT_THREADS, 1)
+    split_stage_kernel(const __grid_constant__ StageArgs one, const StageArgs* __restrict__ args,
+                       const BatchTile* __restrict__ tiles, long ntiles, const double* __restrict__ kref, int mode) {
+  extern __shared__ double smem[];
+  using S = Slots<T>;
+  double* const A = smem;
+  double* const B = smem + S::A * SPLIT_PTS;
+  int4* const stage = reinterpret_cast<int4*>(B + S::B * SPLIT_PTS);
+  int* const tables = reinterpret_cast<int*>(stage + SPLIT_GROUPS * (SPLIT_NDY + SPLIT_NDZ));
+  int* const rec = tables + SPLIT_GROUPS * 80;
+  constexpr int NSLOT = 24 + (T::SCALAR ? 2 : 0);
+  if (threadIdx.x < 32) rec[threadIdx.x] = 0;
+  __syncthreads();
+  const int t = threadIdx.x % SPLIT_PTS;
+  const int tx = (one.g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = (one.g.ny + SPLIT_TY - 1) / SPLIT_TY;
+  auto tile_at = [&](long w) {
+    if (BATCH) {
+      const BatchTile b = tiles[w];
+      return SplitTile{b.a * SPLIT_TX, b.b * SPLIT_TY, b.c, b.inst};
+    }
+    const int q = (int)w;  // tiles of one grid: less than 2^31
+    return SplitTile{q % tx * SPLIT_TX, q / tx % ty * SPLIT_TY, q / (tx * ty) + one.k_lo, 0};
+  };
+  if (threadIdx.x < SPLIT_PTS) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SPLIT_REG_ALG));
+    for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
+      const bool more = w + gridDim.x < ntiles;
+      AlgebraParams ap = one.ap;
+      if (BATCH) ap = args[tiles[w].inst].ap;
+      bar_sync(BAR_FULL_A, SPLIT_THREADS);
+      T::rhs_split(SlotIn{A + t}, SlotIn{B + t}, SlotOut<T>{B + t},
+                   [&] {
+                     if (more) bar_arrive(BAR_FREE_A, SPLIT_THREADS);
+                     bar_sync(BAR_FULL_B, SPLIT_THREADS);
+                   },
+                   ap);
+      bar_arrive(BAR_DONE_B, SPLIT_THREADS);
+    }
+    return;
+  }
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SPLIT_REG_DIFF));
+  const int g = __shfl_sync(0xffffffffu, (int)threadIdx.x / SPLIT_PTS - 1, 0);  // uniform, and known to be
+  int* const tab = tables + g * 80;
+  int4* const st = stage + g * (SPLIT_NDY + SPLIT_NDZ);
+  const DiffGroup<T, EQ> d{t, g, A + t, B + t, st, reinterpret_cast<unsigned*>(tab), tab + 48, rec};
+  auto flush = [&](const StageArgs& a) {  // the record of the instance that ends here
+    bar_sync(BAR_DIFF, SPLIT_THREADS - SPLIT_PTS);
+    if (g == 0 && t < NSLOT && a.E_rec && mode != MODE_RHS && mode != MODE_S4) {
+      atomicMax(a.E_rec + 32 * t, (unsigned)rec[t]);
+      rec[t] = 0;
+    }
+  };
+  if (blockIdx.x >= ntiles) return;
+  SplitTile cur = tile_at(blockIdx.x);
+  d.fill_a(BATCH ? args[cur.inst] : one, cur);
+  bar_arrive(BAR_FULL_A, SPLIT_THREADS);
+  for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
+    const StageArgs& a = BATCH ? args[cur.inst] : one;
+    d.fill_b(a, BATCH ? kref[cur.inst] : one.ap.Kref, cur);
+    bar_arrive(BAR_FULL_B, SPLIT_THREADS);
+    const bool more = w + gridDim.x < ntiles;
+    SplitTile nxt = cur;
+    if (more) {
+      nxt = tile_at(w + gridDim.x);
+      bar_sync(BAR_FREE_A, SPLIT_THREADS);
+      d.fill_a(BATCH ? args[nxt.inst] : one, nxt);
+      bar_arrive(BAR_FULL_A, SPLIT_THREADS);
+    }
+    bar_sync(BAR_DONE_B, SPLIT_THREADS);
+    d.combine(a, mode, cur);
+    // no group refills region B (or its record) while another still reads it
+    if (!more || nxt.inst != cur.inst) flush(a);
+    bar_sync(BAR_DIFF, SPLIT_THREADS - SPLIT_PTS);
+    cur = nxt;
+  }
+}
+
+// One block per SM, no more than there are tiles.
+template <class T, bool BATCH, bool EQ>
+cudaError_t launch_split_as(const StageArgs& one, const StageArgs* args, const BatchTile* tiles, long ntiles,
+                            const double* kref, int mode, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  constexpr size_t bytes = split_smem_bytes<T>();
+  static_assert(bytes <= 232448, "shared memory of one block");
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(split_stage_kernel<T, BATCH, EQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  const int blocks = (int)(ntiles < sms ? ntiles : sms);
+  split_stage_kernel<T, BATCH, EQ><<<blocks, SPLIT_THREADS, bytes, s>>>(one, args, tiles, ntiles, kref, mode);
+  return cudaGetLastError();
+}
+
+// eq: equal spacing (of every grid of a batch)
+template <class T, bool BATCH>
+cudaError_t launch_split(const StageArgs& one, const StageArgs* args, const BatchTile* tiles, long ntiles,
+                         const double* kref, int mode, bool eq, cudaStream_t s) {
+  if (ntiles <= 0) return cudaSuccess;
+  return eq ? launch_split_as<T, BATCH, true>(one, args, tiles, ntiles, kref, mode, s)
+            : launch_split_as<T, BATCH, false>(one, args, tiles, ntiles, kref, mode, s);
+}
+
+}  // namespace cosmos

@@ -8,10 +8,10 @@ point 0 lies G planes below its first own plane.  Before every RK4 stage:
 
 1. the ghost planes of the stage state are refilled from the neighbouring
    slabs' own planes (periodic in z across the slabs);
-2. every slab's per-field reference exponent of the integer derivative pass
+2. every slab's per-field reference exponent of the integer differences
    (cosmos_field_exponents) is replaced by the largest over all slabs, so that
    each slab rounds its derivatives exactly as the whole grid does;
-3. cosmos_rk4_stage_slab advances the slab's own planes (the algebra pass and
+3. cosmos_rk4_stage_slab advances the slab's own planes (the algebra and
    the stage combine on them only; the derivative and fluid passes read the
    ghost planes).
 
