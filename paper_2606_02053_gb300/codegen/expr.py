@@ -10,7 +10,7 @@ graph, the reverse-mode adjoint of chosen outputs with respect to chosen
 inputs (one adjoint expression per input), which is how the adjoint kernels
 are generated from the forward definition.
 
-Ops: in, param, const, add, sub, mul, neg, rcp (1/x), sqrt, abs, max, min,
+Ops: in, param, const, add, sub, mul, mulr (rounded product), neg, rcp (1/x), sqrt, abs, max, min,
 minmod.  Piecewise ops (abs, max, min, minmod) use one-sided derivatives at
 their kinks (the branch taken), which is what a hand-written adjoint does.
 """
@@ -188,6 +188,12 @@ def fmin(a: Ex, b: Ex) -> Ex:
     return Ex(a.g, a.g._node("min", (x, y)))
 
 
+def mulr(a: Ex, b: Ex) -> Ex:
+    """A product that is rounded by itself: never fused into a sum."""
+    x, y = sorted((a.id, b.id))
+    return Ex(a.g, a.g._node("mulr", (x, y)))
+
+
 def minmod(a: Ex, b: Ex) -> Ex:
     """0 if a, b differ in sign (or one is 0), else the one of smaller modulus."""
     return Ex(a.g, a.g._node("minmod", (a.id, b.id)))
@@ -244,7 +250,7 @@ def vjp(g: Graph, outputs: Sequence[Ex], cotangents: Sequence[Ex], wrt: Sequence
         elif op == "sub":
             push(args[0], A)
             push(args[1], -A)
-        elif op == "mul":
+        elif op in ("mul", "mulr"):
             push(args[0], A * X[1])
             push(args[1], A * X[0])
         elif op == "neg":
@@ -291,6 +297,8 @@ def _expr(g: Graph, n: int, name) -> str:
         return f"{name(a[0])} - {name(a[1])}"
     if op == "mul":
         return f"{name(a[0])} * {name(a[1])}"
+    if op == "mulr":
+        return f"__dmul_rn({name(a[0])}, {name(a[1])})"
     if op == "neg":
         return f"-{name(a[0])}"
     if op == "rcp":
@@ -305,10 +313,8 @@ def _expr(g: Graph, n: int, name) -> str:
         return f"fmax({name(a[0])}, {name(a[1])})"
     if op == "min":
         return f"fmin({name(a[0])}, {name(a[1])})"
-    if op == "minmod":
-        x, y = name(a[0]), name(a[1])
-        return (f"(({x} > 0.0 && {y} > 0.0) ? fmin({x}, {y}) : "
-                f"(({x} < 0.0 && {y} < 0.0) ? fmax({x}, {y}) : 0.0))")
+    if op in ("minmod", "minmod_da", "minmod_db"):  # functions on the bits, beside the header's own code
+        return f"{op}({name(a[0])}, {name(a[1])})"
     if op == "max_da":
         return f"({name(a[0])} >= {name(a[1])} ? 1.0 : 0.0)"
     if op == "max_db":
@@ -317,12 +323,6 @@ def _expr(g: Graph, n: int, name) -> str:
         return f"({name(a[0])} <= {name(a[1])} ? 1.0 : 0.0)"
     if op == "min_db":
         return f"({name(a[0])} <= {name(a[1])} ? 0.0 : 1.0)"
-    if op == "minmod_da":
-        x, y = name(a[0]), name(a[1])
-        return (f"((({x} > 0.0 && {y} > 0.0) && {x} <= {y}) || (({x} < 0.0 && {y} < 0.0) && {x} >= {y}) ? 1.0 : 0.0)")
-    if op == "minmod_db":
-        x, y = name(a[0]), name(a[1])
-        return (f"((({x} > 0.0 && {y} > 0.0) && {x} > {y}) || (({x} < 0.0 && {y} < 0.0) && {x} < {y}) ? 1.0 : 0.0)")
     raise NotImplementedError(op)
 
 
@@ -599,7 +599,7 @@ def evaluate(g: Graph, outputs: Sequence[Ex], inputs: Dict[str, float], params: 
             v = a[0] + a[1]
         elif op == "sub":
             v = a[0] - a[1]
-        elif op == "mul":
+        elif op in ("mul", "mulr"):
             v = a[0] * a[1]
         elif op == "neg":
             v = -a[0]

@@ -137,6 +137,30 @@ struct FluidParams {
   double w;       // P = w rho
   double sqrt_w;  // sound speed
 };
+
+// minmod and its branch selectors on the bits of the values (the comparisons of
+// FP64 numbers run on the FP64 pipe, which bounds the kernels here; the eight
+// limiters of a face took some 48 of them).  Same results: x and y of one sign,
+// neither zero nor NaN, give the one of smaller modulus (x at a tie), else 0.
+__device__ __forceinline__ bool minmod_same(long long a, long long b) {
+  const unsigned long long m = 0x7FFFFFFFFFFFFFFFull, inf = 0x7FF0000000000000ull;
+  return (a ^ b) >= 0 && ((unsigned long long)a & m) - 1ull < inf && ((unsigned long long)b & m) - 1ull < inf;
+}
+__device__ __forceinline__ bool minmod_first(long long a, long long b) {  // |x| <= |y|, of one sign
+  return (unsigned long long)a <= (unsigned long long)b;
+}
+__device__ __forceinline__ double minmod(double x, double y) {
+  const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
+  return __longlong_as_double(minmod_same(a, b) ? (minmod_first(a, b) ? a : b) : 0ll);
+}
+__device__ __forceinline__ double minmod_da(double x, double y) {
+  const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
+  return __longlong_as_double(minmod_same(a, b) && minmod_first(a, b) ? 0x3FF0000000000000ll : 0ll);
+}
+__device__ __forceinline__ double minmod_db(double x, double y) {
+  const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
+  return __longlong_as_double(minmod_same(a, b) && !minmod_first(a, b) ? 0x3FF0000000000000ll : 0ll);
+}
 """
 
 
