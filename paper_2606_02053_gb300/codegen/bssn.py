@@ -87,27 +87,29 @@ def split_layout(fluid: bool, scalar: bool):
     what the first phase reads, region B what the second one does and the slots
     ``r{f}`` that take the outputs of fields without a slot of their own there.
 
-    Per field with second derivatives ten slots (d_k, dd_p, Kreiss-Oliger
-    bracket k), per field with first derivatives four (d_k, k); m{f} of a field
-    whose derivatives only advect it is that whole advection with its
-    dissipation term; kdiff = K - Kref.  ``out`` = the region-B slot that takes
-    output f: its k or m slot (read by that output alone) or r{f}.
+    Per field with second derivatives ten slots (d_k, dd_p, m), per field with
+    first derivatives four (d_k, m), a field whose derivatives only advect it has
+    m alone: its whole advection with the dissipation term (that of the metric
+    and Gamma is read at the end of the first phase).  kdiff = K - Kref.  ``out`` =
+    the region-B slot that takes output f: its m slot (read by that output alone)
+    or r{f}.
 
     Units: lengths in l (the algebra does not see its value but through the
     parameters below).  u of K, At, Pi carries l, u of the fluid fields and rho
-    l^2, m the units of its output; differences, k, u of B^i and kdiff come
-    without the l of their field, which the parameters that multiply them hold: len = l, c75 = 3/4 l, c43 = 4/3
-    l, eta l^2, lapse_c1 l, lapse_c2 l.  out[f] carries one l more than field f.
+    l^2, m the units of its output; differences, u of B^i and kdiff come without
+    the l of their field, which the parameters that multiply them hold: len = l,
+    c75 = 3/4 l, c43 = 4/3 l, eta l^2, lapse_c1 l, lapse_c2 l.  out[f] carries one l
+    more than field f.
 
     The raised At is formed in the first phase (both phases then take about as
     long as the differences of the other region), except with the fluid, whose
     own quantities already fill the registers between the phases."""
 
     def d2(f):
-        return [f"d{f}_{k}" for k in range(3)] + [f"dd{f}_{p}" for p in range(6)] + [f"k{f}"]
+        return [f"d{f}_{k}" for k in range(3)] + [f"dd{f}_{p}" for p in range(6)] + [f"m{f}"]
 
     def d1(f):
-        return [f"d{f}_{k}" for k in range(3)] + [f"k{f}"]
+        return [f"d{f}_{k}" for k in range(3)] + [f"m{f}"]
 
     a, b = [], []
     for f in range(GT, GT + 6):
@@ -130,7 +132,7 @@ def split_layout(fluid: bool, scalar: bool):
         b += [f"u{ph + 1}"]
     b += [f"r{f}" for f in [*range(GT, GT + 6), *range(GAM, GAM + 3)] + [24, 25, 26, 27] * fluid]
     nf = 24 + 4 * fluid + 2 * scalar
-    out = [b.index(next(x for x in (f"k{f}", f"m{f}", f"r{f}") if x in b)) for f in range(nf)]
+    out = [b.index(next(x for x in (f"m{f}", f"r{f}") if x in b)) for f in range(nf)]
     return dict(a=a, b=b, out=out, early=early)
 
 
@@ -154,7 +156,7 @@ def algebra(fluid: bool, scalar: bool, split: bool = False):
 
     eta = g.param("eta")
     if split:
-        ko, ulen, c75, c43 = g.param("ko"), g.param("len"), g.param("c75"), g.param("c43")
+        ulen, c75, c43 = g.param("len"), g.param("c75"), g.param("c43")
     else:
         Kref = g.param("Kref")
         ulen, c75, c43 = 1.0, 0.75, 4.0 / 3.0
@@ -351,20 +353,11 @@ def algebra(fluid: bool, scalar: bool, split: bool = False):
     out = [None] * nf
     divb = dbeta(0, 0) + dbeta(1, 1) + dbeta(2, 2)
 
-    merged = {*range(AT, AT + 6), *range(BB, BB + 3)} | ({24 + 4 * fluid + 1} if scalar else set())
-
     def adv(f):
         """Advection of field f; in the split form with its dissipation term, in the units of the output."""
-        if split and f in merged:
+        if split:
             return g.input(f"m{f}")
-        s = beta[0] * d(f, 0) + beta[1] * d(f, 1) + beta[2] * d(f, 2)
-        if split and not BET <= f < BET + 3:
-            s = ko * g.input(f"k{f}") + s
-            if GT <= f < GT + 6 or GAM <= f < GAM + 3:
-                cut.append(s)
-            if f == TRK or GAM <= f < GAM + 3:
-                s = ulen * s
-        return s
+        return beta[0] * d(f, 0) + beta[1] * d(f, 1) + beta[2] * d(f, 2)
 
     third_div = (1.0 / 3.0) * divb
     out[CHI] = adv(CHI) + (2.0 * chi) * ((1.0 / 3.0) * (alpha * K) - third_div)
@@ -431,11 +424,11 @@ def algebra(fluid: bool, scalar: bool, split: bool = False):
         out[GAM + i] = adv(GAM + i) + s
     out[ALP] = adv(ALP) - alpha * (c1 + c2 * alpha) * (g.input("kdiff") if split else K - Kref)
     for i in range(3):
-        out[BET + i] = shift_on * (adv(BET + i) + c75 * B[i])
-        if split:  # m of B^i has the switch on its advection
-            out[BET + i] = ko * g.input(f"k{BET + i}") + out[BET + i]
+        if split:  # m of beta^i and B^i has the switch on its advection
+            out[BET + i] = adv(BET + i) + shift_on * (c75 * B[i])
             out[BB + i] = adv(BB + i) + shift_on * (Gt_src[i] - eta * B[i])
         else:
+            out[BET + i] = shift_on * (adv(BET + i) + 0.75 * B[i])
             out[BB + i] = shift_on * (adv(BB + i) + Gt_src[i] - eta * B[i])
     if fluid:
         q = 24

@@ -11,7 +11,7 @@ import sys
 
 from . import bssn
 from . import fluid as fluid_dsl
-from .expr import Ex, emit_function, emit_split, op_counts, vjp
+from .expr import Ex, emit_function, emit_fused, emit_split, op_counts, vjp
 
 ADJOINT_VARIANTS = ("vac", "fluid", "scalar", "fluid_scalar")
 
@@ -25,6 +25,8 @@ HEADER = """// GENERATED by paper_2606_02053_gb300/codegen/generate.py -- do not
 // and without the fluid flux divergence), one grid point per call.
 // Input layout and parameters: see paper_2606_02053_gb300/codegen/bssn.py.
 #pragma once
+
+#include "../fp64_regs.cuh"
 
 struct AlgebraParams {
   double eta;       // Gamma-driver damping
@@ -66,7 +68,7 @@ def render() -> dict:
         body.append(f"constexpr bool SPLIT_EARLY = {str(S['early']).lower()};  // At among the states of region A")
         body.append(_table_fn("out_slot", S["out"]))
         body.append(emit_split(gs, "rhs_split", S["a"], S["b"], outs, gs.cut, "AlgebraParams"))
-        body.append(emit_function(g, "constraints", L["names"], g.constraints, ["AlgebraParams"]))
+        body.append(emit_fused(g, "constraints", L["names"], g.constraints, "AlgebraParams"))
         if name in ADJOINT_VARIANTS:
             # reverse mode: in[0 .. NIN) as for rhs, in[NIN + f] = cotangent of out[f];
             # out[k] = sum_f cot_f d out_f / d in[k]
@@ -75,14 +77,14 @@ def render() -> dict:
             adj = vjp(g, out, w, wrt)
             stats.append((name + "_vjp", op_counts(g, adj)))
             body.append(f"// reverse mode of rhs: ops {dict(sorted(op_counts(g, adj).items()))}")
-            body.append(emit_function(g, "rhs_vjp", L["names"] + [f"w{f}" for f in range(L["nf"])], adj,
-                                      ["AlgebraParams"], accessors=True))
+            body.append(emit_fused(g, "rhs_vjp", L["names"] + [f"w{f}" for f in range(L["nf"])], adj, "AlgebraParams",
+                                   accessors=True))
         if name == "vac":
             # reverse mode of H (first constraint) w.r.t. chi, d chi, dd chi: initial-data adjoint
             hb = g.input("hb")
             chi_in = ["u0"] + [f"d0_{k}" for k in range(3)] + [f"dd0_{m}" for m in range(6)]
             adjh = vjp(g, g.constraints[:1], [hb], [Ex(g, g.inputs[nm]) for nm in chi_in])
-            body.append(emit_function(g, "ham_vjp_chi", L["names"] + ["hb"], adjh, ["AlgebraParams"]))
+            body.append(emit_fused(g, "ham_vjp_chi", L["names"] + ["hb"], adjh, "AlgebraParams"))
         body.append(f"}}  // namespace alg_{name}\n")
     files["bssn_algebra.cuh"] = "\n".join(body)
     fb = [FLUID_HEADER]
@@ -93,22 +95,21 @@ def render() -> dict:
     # face flux is symmetric under the exchange of its left and right states (with the odd
     # components negated), and its paired sums (F_L + F_R, U_R - U_L) keep that symmetry bitwise,
     # so mirror-symmetric data keep their velocities exactly zero on the symmetry planes.
-    fb.append(emit_function(g, "fluid_prim", names, out, ["FluidParams"], chains=False))
+    fb.append(emit_fused(g, "fluid_prim", names, out, "FluidParams", chains=False))
     qb = [g.input(f"qb{m}") for m in range(4)]
     adj = vjp(g, out, qb, [Ex(g, g.inputs[nm]) for nm in names])
     fb.append("// reverse mode: in[11 + m] = cotangent of (rho, v0, v1, v2)[m]; out = cotangents of the inputs")
-    fb.append(emit_function(g, "fluid_prim_vjp", names + [f"qb{m}" for m in range(4)], adj, ["FluidParams"],
-                            chains=False))
+    fb.append(emit_fused(g, "fluid_prim_vjp", names + [f"qb{m}" for m in range(4)], adj, "FluidParams", chains=False))
     for d in range(3):
         g, names, out = fluid_dsl.face_flux(d)
         stats.append((f"face{d}", op_counts(g, out)))
         if d == 0:
             fb.append("// face-flux inputs: " + ", ".join(names))
-        fb.append(emit_function(g, f"fluid_face_flux_{d}", names, out, ["FluidParams"], chains=False))
+        fb.append(emit_fused(g, f"fluid_face_flux_{d}", names, out, "FluidParams", chains=False))
         hb = [g.input(f"hb{m}") for m in range(4)]
         adj = vjp(g, out, hb, [Ex(g, g.inputs[nm]) for nm in names])
-        fb.append(emit_function(g, f"fluid_face_flux_{d}_vjp", names + [f"hb{m}" for m in range(4)], adj,
-                                ["FluidParams"], chains=False))
+        fb.append(emit_fused(g, f"fluid_face_flux_{d}_vjp", names + [f"hb{m}" for m in range(4)], adj, "FluidParams",
+                             chains=False))
     files["fluid_algebra.cuh"] = "\n".join(fb)
     return files, stats
 
@@ -132,6 +133,8 @@ FLUID_HEADER = """// GENERATED by paper_2606_02053_gb300/codegen/generate.py -- 
 // Fluid primitive recovery and Kurganov-Tadmor face fluxes (see
 // paper_2606_02053_gb300/codegen/fluid.py for the formulas and the inputs).
 #pragma once
+
+#include "../fp64_regs.cuh"
 
 struct FluidParams {
   double w;       // P = w rho

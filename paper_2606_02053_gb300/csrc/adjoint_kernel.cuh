@@ -74,12 +74,12 @@ __global__ void __launch_bounds__(BX* BY, COSMOS_VJP_MIN_BLOCKS) vjp_pass1_kerne
   const long c = ((long)k * a.g.ny + j) * a.g.pitch + i;
   const VjpIn<T> in{a, fs, c};
   VjpOut out{a.CB, fs, c};
-  T::rhs_vjp(in, out, a.ap);
+  T::rhs_vjp(in, out, a.ap, fp64_regs());
 }
 
 // Face-flux reverse: H_d(p) enters F at p (-1/h) and at p + e_d (+1/h).
 template <int D>
-__device__ __forceinline__ void face_vjp(const VjpArgs& a, const Nbr& n) {
+__device__ __forceinline__ void face_vjp(const VjpArgs& a, const Nbr& n, const Fp64Regs& kr) {
   const long fs = a.g.fstride;
   double in[34 + 4];
 #pragma unroll
@@ -105,9 +105,9 @@ __device__ __forceinline__ void face_vjp(const VjpArgs& a, const Nbr& n) {
     in[34 + m] = (ldg(Wm, up) - ldg(Wm, n.c)) * a.c.ih[D];
   }
   double out[34];
-  if (D == 0) fluid_face_flux_0_vjp(in, out, a.fp);
-  if (D == 1) fluid_face_flux_1_vjp(in, out, a.fp);
-  if (D == 2) fluid_face_flux_2_vjp(in, out, a.fp);
+  if (D == 0) fluid_face_flux_0_vjp(in, out, a.fp, kr);
+  if (D == 1) fluid_face_flux_1_vjp(in, out, a.fp, kr);
+  if (D == 2) fluid_face_flux_2_vjp(in, out, a.fp, kr);
 #pragma unroll
   for (int m = 0; m < 34; ++m) a.FC[(long)(34 * D + m) * fs + n.c] = out[m];
 }
@@ -118,9 +118,10 @@ static __global__ void __launch_bounds__(BX* BY) vjp_face_kernel(const VjpArgs a
   const int k = blockIdx.z;
   if (i >= a.g.nx || j >= a.g.ny) return;
   const Nbr n = make_nbr(a.g, i, j, k);
-  face_vjp<0>(a, n);
-  face_vjp<1>(a, n);
-  face_vjp<2>(a, n);
+  const Fp64Regs kr = fp64_regs();
+  face_vjp<0>(a, n, kr);
+  face_vjp<1>(a, n, kr);
+  face_vjp<2>(a, n, kr);
 }
 
 // Per cell: gather the face-input cotangents that refer to this cell, add the
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(BX* BY) vjp_cell_kernel(const VjpArgs a) {
 #pragma unroll
   for (int m = 0; m < 4; ++m) in[11 + m] = qb[m];
   double pb[11];
-  fluid_prim_vjp(in, pb, a.fp);
+  fluid_prim_vjp(in, pb, a.fp, fp64_regs());
   double vf[T::NF];
 #pragma unroll
   for (int f = 0; f < T::NF; ++f) vf[f] = 0.0;
@@ -244,8 +245,9 @@ struct T_vac_adj {
     __device__ static constexpr int d1_slot(int f) { return alg_##NAME::d1_slot(f); }                          \
     __device__ static constexpr int d2_slot(int f) { return alg_##NAME::d2_slot(f); }                          \
     template <class In, class Out>                                                                              \
-    __device__ static __forceinline__ void rhs_vjp(const In& in, Out&& out, const AlgebraParams& p) {           \
-      alg_##NAME::rhs_vjp(in, out, p);                                                                          \
+    __device__ static __forceinline__ void rhs_vjp(const In& in, Out&& out, const AlgebraParams& p,             \
+                                                   const Fp64Regs& k) {                                         \
+      alg_##NAME::rhs_vjp(in, out, p, k);                                                                       \
     }                                                                                                           \
   };                                                                                                            \
   cudaError_t launch_vjp_##NAME(const VjpArgs& a, cudaStream_t s) {                                             \

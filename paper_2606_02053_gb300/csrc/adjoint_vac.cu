@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(BX* BY) init_ham_vjp_kernel(const DevGrid g, c
   const double Ebar = ldg(lam + 24 * fs, n.c) / (chi * sqrt(chi));
   in[alg_vac::NIN] = Ebar / (16.0 * PI);
   double out[10];
-  alg_vac::ham_vjp_chi(in, out, ap);
+  alg_vac::ham_vjp_chi(in, out, ap, fp64_regs());
 #pragma unroll
   for (int m = 0; m < 10; ++m) CB10[(long)m * fs + n.c] = out[m];
 }

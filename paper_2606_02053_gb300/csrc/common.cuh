@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include "../../include/cosmos.h"
+#include "fp64_regs.cuh"
 #include "generated/bssn_algebra.cuh"
 #include "generated/fluid_algebra.cuh"
 

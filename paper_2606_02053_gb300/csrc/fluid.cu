@@ -7,7 +7,7 @@
 namespace cosmos {
 
 __device__ __forceinline__ void prim_point(const DevGrid& g, const double* __restrict__ U, double* __restrict__ prim,
-                                           const FluidParams& fp, int i, int j, int k) {
+                                           const FluidParams& fp, const Fp64Regs& kr, int i, int j, int k) {
   const long c = ((long)k * g.ny + j) * g.pitch + i;
   const long fs = g.fstride;
   double in[11];
@@ -17,7 +17,7 @@ __device__ __forceinline__ void prim_point(const DevGrid& g, const double* __res
 #pragma unroll
   for (int m = 0; m < 4; ++m) in[7 + m] = ldg(U + (24 + m) * fs, c);
   double out[4];
-  fluid_prim(in, out, fp);
+  fluid_prim(in, out, fp, kr);
 #pragma unroll
   for (int m = 0; m < 4; ++m) prim[m * fs + c] = out[m];
 }
@@ -28,12 +28,12 @@ __global__ void __launch_bounds__(BX* BY) prim_kernel(const DevGrid g, const dou
   const int j = blockIdx.y * BY + threadIdx.y;
   const int k = blockIdx.z;
   if (i >= g.nx || j >= g.ny) return;
-  prim_point(g, U, prim, fp, i, j, k);
+  prim_point(g, U, prim, fp, fp64_regs(), i, j, k);
 }
 
 template <int D>
 __device__ __forceinline__ void face(const double* __restrict__ U, const double* __restrict__ prim, const Nbr& n,
-                                     long fs, const FluidParams& fp, double* __restrict__ H) {
+                                     long fs, const FluidParams& fp, const Fp64Regs& kr, double* __restrict__ H) {
   double in[34];
 #pragma unroll
   for (int o = 0; o < 4; ++o) {
@@ -52,20 +52,20 @@ __device__ __forceinline__ void face(const double* __restrict__ U, const double*
     for (int m = 0; m < 6; ++m) q[3 + m] = ldg(U + (1 + m) * fs, off);
   }
   double out[4];
-  if (D == 0) fluid_face_flux_0(in, out, fp);
-  if (D == 1) fluid_face_flux_1(in, out, fp);
-  if (D == 2) fluid_face_flux_2(in, out, fp);
+  if (D == 0) fluid_face_flux_0(in, out, fp, kr);
+  if (D == 1) fluid_face_flux_1(in, out, fp, kr);
+  if (D == 2) fluid_face_flux_2(in, out, fp, kr);
 #pragma unroll
   for (int m = 0; m < 4; ++m) H[(4 * D + m) * fs + n.c] = out[m];
 }
 
 __device__ __forceinline__ void flux_point(const DevGrid& g, const double* __restrict__ U,
                                            const double* __restrict__ prim, double* __restrict__ H,
-                                           const FluidParams& fp, int i, int j, int k) {
+                                           const FluidParams& fp, const Fp64Regs& kr, int i, int j, int k) {
   const Nbr n = make_nbr(g, i, j, k);
-  face<0>(U, prim, n, g.fstride, fp, H);
-  face<1>(U, prim, n, g.fstride, fp, H);
-  face<2>(U, prim, n, g.fstride, fp, H);
+  face<0>(U, prim, n, g.fstride, fp, kr, H);
+  face<1>(U, prim, n, g.fstride, fp, kr, H);
+  face<2>(U, prim, n, g.fstride, fp, kr, H);
 }
 
 __global__ void __launch_bounds__(BX* BY) flux_kernel(const DevGrid g, const double* __restrict__ U,
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(BX* BY) flux_kernel(const DevGrid g, const dou
   const int j = blockIdx.y * BY + threadIdx.y;
   const int k = blockIdx.z;
   if (i >= g.nx || j >= g.ny) return;
-  flux_point(g, U, prim, H, fp, i, j, k);
+  flux_point(g, U, prim, H, fp, fp64_regs(), i, j, k);
 }
 
 // Batched passes: blocks stride over the flat work list of every instance
@@ -83,22 +83,24 @@ __global__ void __launch_bounds__(BX* BY) flux_kernel(const DevGrid g, const dou
 __global__ void __launch_bounds__(BX* BY) batch_prim_kernel(const StageArgs* __restrict__ args,
                                                             const BatchTile* __restrict__ tiles, long ntiles,
                                                             int mapping, const FluidParams fp) {
+  const Fp64Regs kr = fp64_regs();
   for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
     const BatchTile t = tiles[w];
     const StageArgs& a = args[t.inst];
     int i, j, k;
-    if (batch_point(t, a.g, mapping, i, j, k)) prim_point(a.g, a.U, const_cast<double*>(a.prim), fp, i, j, k);
+    if (batch_point(t, a.g, mapping, i, j, k)) prim_point(a.g, a.U, const_cast<double*>(a.prim), fp, kr, i, j, k);
   }
 }
 
 __global__ void __launch_bounds__(BX* BY) batch_flux_kernel(const StageArgs* __restrict__ args,
                                                             const BatchTile* __restrict__ tiles, long ntiles,
                                                             int mapping, const FluidParams fp) {
+  const Fp64Regs kr = fp64_regs();
   for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
     const BatchTile t = tiles[w];
     const StageArgs& a = args[t.inst];
     int i, j, k;
-    if (batch_point(t, a.g, mapping, i, j, k)) flux_point(a.g, a.U, a.prim, const_cast<double*>(a.flux), fp, i, j, k);
+    if (batch_point(t, a.g, mapping, i, j, k)) flux_point(a.g, a.U, a.prim, const_cast<double*>(a.flux), fp, kr, i, j, k);
   }
 }
 

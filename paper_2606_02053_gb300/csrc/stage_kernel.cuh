@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(BX* BY, 2) constraint_kernel(const ConstraintA
     const long fs = a.g.fstride;
     double in[T::NIN];
     gather<T>(a.U, a.prim, n, a.c, fs, in);
-    T::constraints(in, v, a.ap);
+    T::constraints(in, v, a.ap, fp64_regs());
     if (a.hm) {
 #pragma unroll
       for (int m = 0; m < 4; ++m) a.hm[(long)m * fs + n.c] = v[m];
@@ -237,11 +237,12 @@ __global__ void __launch_bounds__(BX* BY, 2) constraint_kernel(const ConstraintA
     __device__ static constexpr int out_slot(int f) { return alg_##NAME::out_slot(f); }                             \
     template <class InA, class InB, class Out, class Next>                                                          \
     __device__ static __forceinline__ void rhs_split(const InA& ina, const InB& inb, Out&& out, Next&& next,        \
-                                                     const AlgebraParams& p) {                                      \
-      alg_##NAME::rhs_split(ina, inb, out, next, p);                                                                \
+                                                     const AlgebraParams& p, const Fp64Regs& k) {                   \
+      alg_##NAME::rhs_split(ina, inb, out, next, p, k);                                                           \
     }                                                                                                               \
-    __device__ static __forceinline__ void constraints(const double* in, double* out, const AlgebraParams& p) {  \
-      alg_##NAME::constraints(in, out, p);                                                                      \
+    __device__ static __forceinline__ void constraints(const double* in, double* out, const AlgebraParams& p,       \
+                                                       const Fp64Regs& k) {                                       \
+      alg_##NAME::constraints(in, out, p, k);                                                                     \
     }                                                                                                           \
   };                                                                                                            \
   cudaError_t launch_stage_##NAME(const StageArgs& a, int mode, int k_cnt, cudaStream_t s) {                        \

@@ -77,6 +77,7 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 template <class T>
 struct Slots {
   static constexpr int A = T::SA, B = T::SB;
+  // (d_k, dd_p, m of a second-derivative field; d_k, m of a first-derivative one)
   // region A: 6 x 10 (metric), 3 x 4 (Gamma), metric, shift, At (SPLIT_EARLY), fluid: chi, tau, S_i, rho
   static constexpr int A_GT = 0, A_GAM = 60, A_STATE = 72;
   static constexpr int A_NSTATE = 9 + (T::SPLIT_EARLY ? 6 : 0) + (T::FLUID ? 6 : 0);
@@ -144,10 +145,10 @@ struct DiffCtx {
   const char* L;
   const char* U;
   long fb;           // bytes of one field
-  unsigned o[3][6];  // neighbours -3, -2, -1, 1, 2, 3 along each axis
   unsigned c;        // the point itself (clamped into the grid)
-  unsigned b[4];     // staged sums q = t + 128 j of this thread: offset without the axis differenced,
-  int p[4];          // and the place of the centre along that axis in the offset tables
+  unsigned o[3];     // that without its offset along each axis,
+  int p[3];          // and its place along each axis in the offset tables
+  unsigned b[4];     // staged sums q = t + 128 j of this thread: offset without the axis differenced
   double r[3];       // h_x / h_d (unequal spacing)
 };
 
@@ -190,23 +191,17 @@ struct DiffGroup {
     const int tx = min(t % SPLIT_TX, a.g.nx - 1 - w.i0), ty = min(t / SPLIT_TX, a.g.ny - 1 - w.j0);
     const unsigned cx = xw[tx + 3], cy = yw[ty + 3], cz = zw[3];
     x.c = cx + cy + cz;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const int p = q < 3 ? q : q + 1;
-      x.o[0][q] = xw[tx + p] + cy + cz;
-      x.o[1][q] = cx + yw[ty + p] + cz;
-      x.o[2][q] = cx + cy + zw[p];
-    }
+    x.o[0] = cy + cz;
+    x.o[1] = cx + cz;
+    x.o[2] = cx + cy;
+    x.p[0] = tx + 3;
+    x.p[1] = SPLIT_NXW + ty + 3;
+    x.p[2] = SPLIT_NXW + SPLIT_NYW + 3;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int q = t + SPLIT_PTS * j, z = q - SPLIT_NDY;
-      if (q < SPLIT_NDY) {
-        x.b[j] = xw[q % SPLIT_XH + 1] + cz;
-        x.p[j] = SPLIT_NXW + q / SPLIT_XH + 3;
-      } else {
-        x.b[j] = q < SPLIT_NDY + SPLIT_NDZ ? xw[z % SPLIT_XH + 1] + yw[z / SPLIT_XH + 1] : 0u;
-        x.p[j] = SPLIT_NXW + SPLIT_NYW + 3;
-      }
+      x.b[j] = q < SPLIT_NDY ? xw[q % SPLIT_XH + 1] + cz
+                             : (q < SPLIT_NDY + SPLIT_NDZ ? xw[z % SPLIT_XH + 1] + yw[z / SPLIT_XH + 1] : 0u);
     }
     x.L = reinterpret_cast<const char*>(a.L);
     x.U = reinterpret_cast<const char*>(a.U);
@@ -217,18 +212,18 @@ struct DiffGroup {
     }
   }
 
-  // The values a point's stencils need, all loads in flight at once.
-  struct Values {
-    long long c, n[3][6];
-  };
-  __device__ __forceinline__ Values load(const DiffCtx& x, const char* __restrict__ L) const {
-    Values v;
-    v.c = ldv(L, x.c);
+  // Place of the centre of staged sum q = t + 128 j along the differenced axis in the offset tables.
+  __device__ __forceinline__ int centre(int j) const {
+    const int q = t + SPLIT_PTS * j;
+    return q < SPLIT_NDY ? SPLIT_NXW + 3 + q / SPLIT_XH : SPLIT_NXW + SPLIT_NYW + 3;
+  }
+
+  // The six neighbours -3, -2, -1, 1, 2, 3 along axis d.  Their offsets come from the tables each
+  // time: held in registers they would spill others.
+  __device__ __forceinline__ void load(const char* __restrict__ L, const DiffCtx& x, int d, long long (&n)[6]) const {
+    const unsigned* const o = xw + x.p[d];
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
-#pragma unroll
-      for (int q = 0; q < 6; ++q) v.n[d][q] = ldv(L, x.o[d][q]);
-    return v;
+    for (int q = 0; q < 6; ++q) n[q] = ldv(L, x.o[d] + o[q < 3 ? q - 3 : q - 2]);
   }
 
   // D1 sum and s_k = f(+k) + f(-k) along one axis
@@ -248,44 +243,53 @@ struct DiffGroup {
     return l_add(s3, l_sub(l_mul(l_sub(l_mul(s1, 5), l_mul(s2, 2)), 3), f20));
   }
 
-  // Ten slots of a second-derivative field (all of degree 0): d_k, dd_p, KO bracket.
+  // Ten slots of a second-derivative field (all of degree 0): d_k, dd_p, and b^k d_k with the KO term.
   template <bool ODD>
-  __device__ __forceinline__ void d2_slots(const DiffCtx& x, const char* __restrict__ L, int e, double* dst) const {
+  __device__ __forceinline__ void d2_slots(const DiffCtx& x, const char* __restrict__ L, int e, double kos,
+                                           const double* b, double* dst) const {
     // D_y and D_z sums of the tile with their halos; every load in flight before the first use
     long long r[4][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       if (t + SPLIT_PTS * j < SPLIT_NDY + SPLIT_NDZ) {
-        r[j][0] = ldv(L, x.b[j] + xw[x.p[j] - 2]);
-        r[j][1] = ldv(L, x.b[j] + xw[x.p[j] - 1]);
-        r[j][2] = ldv(L, x.b[j] + xw[x.p[j] + 1]);
-        r[j][3] = ldv(L, x.b[j] + xw[x.p[j] + 2]);
+        const unsigned* const o = xw + centre(j);
+        r[j][0] = ldv(L, x.b[j] + o[-2]);
+        r[j][1] = ldv(L, x.b[j] + o[-1]);
+        r[j][2] = ldv(L, x.b[j] + o[1]);
+        r[j][3] = ldv(L, x.b[j] + o[2]);
       }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       if (t + SPLIT_PTS * j < SPLIT_NDY + SPLIT_NDZ)
         sDy[t + SPLIT_PTS * j] =
             p4(l_d1(l_sub(limb_of(r[j][2]), limb_of(r[j][1])), l_sub(limb_of(r[j][3]), limb_of(r[j][0]))));
-    const Values n = load(x, L);
-    const Limb f0 = limb_of(n.c), f30 = l_mul(f0, 30);
+    // two axes' loads in flight while the third's are issued behind the first axis
+    long long n0[6], n1[6], n2[6];
+    const long long nc = ldv(L, x.c);
+    load(L, x, 0, n0);
+    load(L, x, 1, n1);
+    const Limb f0 = limb_of(nc), f30 = l_mul(f0, 30);
     Limb d1, s1, s2, s3;
+    double dx, ko = 0.0;
     if (EQ) {
       Limb P1, P2, P3, yy;
-      axis(n.n[0], d1, P1, P2, P3);
+      axis(n0, d1, P1, P2, P3);
+      load(L, x, 2, n2);
       {
         const Limb S[2] = {d1, second(P1, P2, f30)};
         const int ee[2] = {e, e + 2};
         double v[2];
         limb_values<ODD>(S, ee, v);
+        dx = v[0];
         dst[0] = v[0];
         dst[3 * SPLIT_PTS] = v[1];
       }
-      axis(n.n[1], d1, s1, s2, s3);
+      axis(n1, d1, s1, s2, s3);
       yy = second(s1, s2, f30);
       P1 = l_add(P1, s1);
       P2 = l_add(P2, s2);
       P3 = l_add(P3, s3);
-      axis(n.n[2], d1, s1, s2, s3);
+      axis(n2, d1, s1, s2, s3);
       P1 = l_add(P1, s1);
       P2 = l_add(P2, s2);
       P3 = l_add(P3, s3);
@@ -295,18 +299,18 @@ struct DiffGroup {
       limb_values<ODD>(S, ee, v);
       dst[6 * SPLIT_PTS] = v[0];
       dst[8 * SPLIT_PTS] = v[1];
-      dst[9 * SPLIT_PTS] = v[2];
+      ko = v[2];
     } else {
       const Limb f20 = l_mul(f0, 20);
-      double ko = 0.0;
+      load(L, x, 2, n2);
 #define COSMOS_SPLIT_AXIS(AX, SL)                                               \
   {                                                                             \
-    axis(n.n[AX], d1, s1, s2, s3);                                              \
+    axis(n##AX, d1, s1, s2, s3);                                                \
     const Limb S[3] = {d1, second(s1, s2, f30), bracket(s1, s2, s3, f20)};      \
     const int ee[3] = {e, e + 2, e};                                            \
     double v[3];                                                                \
     limb_values<ODD>(S, ee, v);                                                 \
-    if (AX == 0) dst[0] = v[0];                                                 \
+    if (AX == 0) dst[0] = dx = v[0];                                            \
     dst[SL * SPLIT_PTS] = v[1] * (x.r[AX] * x.r[AX]);                           \
     ko = fma(x.r[AX], v[2], ko);                                                \
   }
@@ -314,7 +318,6 @@ struct DiffGroup {
       COSMOS_SPLIT_AXIS(1, 6)
       COSMOS_SPLIT_AXIS(2, 8)
 #undef COSMOS_SPLIT_AXIS
-      dst[9 * SPLIT_PTS] = ko;
     }
     sync();
     const int4* ry = sDy + (t / SPLIT_TX) * SPLIT_XH + t % SPLIT_TX + 2;
@@ -338,32 +341,37 @@ struct DiffGroup {
     dst[4 * SPLIT_PTS] = v[2];
     dst[5 * SPLIT_PTS] = v[3];
     dst[7 * SPLIT_PTS] = v[4];
+    double m = kos * ko;
+    if (b) m = fma(b[0], dx, fma(b[SPLIT_PTS], v[0], fma(b[2 * SPLIT_PTS], v[1], m)));
+    dst[9 * SPLIT_PTS] = m;
     sync();
   }
 
-  __device__ __forceinline__ void d2_field(const DiffCtx& x, int f, double* dst) const {
+  __device__ __forceinline__ void d2_field(const DiffCtx& x, int f, double kos, const double* b, double* dst) const {
     const int s = ko_slot<T>(f), e = ex[s];
     const char* __restrict__ L = x.L + s * x.fb;
     if (limb_odd(e))
-      d2_slots<true>(x, L, e, dst);
+      d2_slots<true>(x, L, e, kos, b, dst);
     else
-      d2_slots<false>(x, L, e, dst);
+      d2_slots<false>(x, L, e, kos, b, dst);
   }
 
   // First derivatives (v[0 .. 2]) and KO bracket (v[3]) of field f.
   template <bool ODD>
   __device__ __forceinline__ void d1_values(const DiffCtx& x, const char* __restrict__ L, int e, double (&v)[4]) const {
-    const Values n = load(x, L);
-    const Limb f0 = limb_of(n.c);
+    long long n[3][6];
+    const Limb f0 = limb_of(ldv(L, x.c));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) load(L, x, d, n[d]);
     Limb D[3], s1, s2, s3;
     if (EQ) {
       Limb P1, P2, P3;
-      axis(n.n[0], D[0], P1, P2, P3);
-      axis(n.n[1], D[1], s1, s2, s3);
+      axis(n[0], D[0], P1, P2, P3);
+      axis(n[1], D[1], s1, s2, s3);
       P1 = l_add(P1, s1);
       P2 = l_add(P2, s2);
       P3 = l_add(P3, s3);
-      axis(n.n[2], D[2], s1, s2, s3);
+      axis(n[2], D[2], s1, s2, s3);
       P1 = l_add(P1, s1);
       P2 = l_add(P2, s2);
       P3 = l_add(P3, s3);
@@ -376,7 +384,7 @@ struct DiffGroup {
       v[3] = 0.0;
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        axis(n.n[d], D[d], s1, s2, s3);
+        axis(n[d], D[d], s1, s2, s3);
         const Limb S[2] = {D[d], bracket(s1, s2, s3, f20)};
         double w[2];
         limb_values<ODD>(S, ee, w);
@@ -395,12 +403,19 @@ struct DiffGroup {
       d1_values<false>(x, L, e, v);
   }
 
-  // Four slots of a field.
-  __device__ __forceinline__ void d1_field(const DiffCtx& x, int f, double* dst) const {
+  // l (b^k d_k f + KO term) of a field of degree 1 into m, its differences into dst (if given);
+  // b: slots of the shift (null: not advected).
+  __device__ __forceinline__ void d1_field(const DiffCtx& x, int f, const StageArgs& a, const double* b, double* dst,
+                                           double* m) const {
     double v[4];
     d1_sums(x, f, v);
+    if (dst) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) dst[q * SPLIT_PTS] = v[q];
+      for (int q = 0; q < 3; ++q) dst[q * SPLIT_PTS] = v[q];
+    }
+    double s = a.ap.ko * v[3];
+    if (b) s = fma(b[0], v[0], fma(b[SPLIT_PTS], v[1], fma(b[2 * SPLIT_PTS], v[2], s)));
+    *m = a.len * s;
   }
 
   // State values into their slots (G = the group, known at compile time, so that fields and factors are):
@@ -451,9 +466,12 @@ struct DiffGroup {
       state_a<1>(a, x);
     else
       state_a<2>(a, x);
+    bar_sync(BAR_DIFF, SPLIT_THREADS - SPLIT_PTS);  // the shift's slots, which the groups share, are written
+    const double* const b = sA + (S::A_STATE + 6) * SPLIT_PTS;
 #pragma unroll 1
-    for (int m = g; m < 6; m += SPLIT_GROUPS) d2_field(x, 1 + m, sA + (S::A_GT + 10 * m) * SPLIT_PTS);
-    d1_field(x, 14 + g, sA + (S::A_GAM + 4 * g) * SPLIT_PTS);
+    for (int m = g; m < 6; m += SPLIT_GROUPS) d2_field(x, 1 + m, a.ap.ko, b, sA + (S::A_GT + 10 * m) * SPLIT_PTS);
+    double* const gam = sA + (S::A_GAM + 4 * g) * SPLIT_PTS;
+    d1_field(x, 14 + g, a, b, gam, gam + 3 * SPLIT_PTS);
   }
 
   __device__ __forceinline__ void fill_b(const StageArgs& a, double kref, const SplitTile& w) const {
@@ -466,26 +484,21 @@ struct DiffGroup {
       state_b<1>(a, kref, x);
     else
       state_b<2>(a, kref, x);
+    bar_sync(BAR_DIFF, SPLIT_THREADS - SPLIT_PTS);  // as in fill_a
+    // a frozen shift is not advected: beta^i (blocks 2 to 4) and B^i
+    const double* const b = sB + (S::B_STATE + 15) * SPLIT_PTS;
+    const double* const bs = a.ap.shift_on != 0.0 ? b : nullptr;
 #pragma unroll 1
-    for (int m = g; m < S::ND2B; m += SPLIT_GROUPS) d2_field(x, S::b_d2(m), sB + 10 * m * SPLIT_PTS);
+    for (int m = g; m < S::ND2B; m += SPLIT_GROUPS)
+      d2_field(x, S::b_d2(m), a.ap.ko, m >= 2 && m < 5 ? bs : b, sB + 10 * m * SPLIT_PTS);
     // K and the merged advections, 1 + NM first-derivative fields: the group with fewer
     // second-derivative fields takes more of them
     constexpr int NG = T::SCALAR ? 4 : 3;
     const int lo = g * NG, hi = g == SPLIT_GROUPS - 1 ? 1 + S::NM : lo + NG;
-    const double b0 = ldd(x.U + 18 * x.fb, x.c), b1 = ldd(x.U + 19 * x.fb, x.c), b2 = ldd(x.U + 20 * x.fb, x.c);
 #pragma unroll 1
     for (int m = lo; m < hi; ++m) {
-      if (m == 0) {
-        d1_field(x, 7, sB + S::B_K * SPLIT_PTS);
-        continue;
-      }
-      const int f = S::b_m(m - 1);
-      double v[4];
-      d1_sums(x, f, v);
-      // l (beta^k d_k f + KO term), with the shift switch on the advection of B^i
-      double q = fma(b0, v[0], fma(b1, v[1], b2 * v[2]));
-      if (f >= 21 && f < 24) q *= a.ap.shift_on;
-      sB[(S::B_M + m - 1) * SPLIT_PTS] = a.len * fma(a.ap.ko, v[3], q);
+      const int f = m == 0 ? 7 : S::b_m(m - 1);
+      d1_field(x, f, a, f >= 21 && f < 24 ? bs : b, m == 0 ? sB + S::B_K * SPLIT_PTS : nullptr, sB + (m == 0 ? S::B_K + 3 : S::B_M + m - 1) * SPLIT_PTS);
     }
   }
 
@@ -601,6 +614,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   };
   if (threadIdx.x < SPLIT_PTS) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SPLIT_REG_ALG));
+    const Fp64Regs k = fp64_regs();
     for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
       const bool more = w + gridDim.x < ntiles;
       AlgebraParams ap = one.ap;
@@ -611,7 +625,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
                      if (more) bar_arrive(BAR_FREE_A, SPLIT_THREADS);
                      bar_sync(BAR_FULL_B, SPLIT_THREADS);
                    },
-                   ap);
+                   ap, k);
       bar_arrive(BAR_DONE_B, SPLIT_THREADS);
     }
     return;

@@ -16,7 +16,7 @@ from paper_2606_02053_gb300.codegen.expr import emit_split, evaluate
 VARIANTS = [(False, False), (True, False), (False, True), (True, True)]
 LEN, KO, KREF = 0.37, 0.021, -0.4  # unit of length, sigma / 64 per axis sum, background trace
 PLAIN = dict(eta=1.5, Kref=KREF, lapse_c1=2.0, lapse_c2=0.3, shift_on=1.0, w=1.0 / 3.0)
-SPLIT = dict(eta=1.5 * LEN ** 2, lapse_c1=2.0 * LEN, lapse_c2=0.3 * LEN, shift_on=1.0, w=1.0 / 3.0, ko=KO, len=LEN,
+SPLIT = dict(eta=1.5 * LEN ** 2, lapse_c1=2.0 * LEN, lapse_c2=0.3 * LEN, shift_on=1.0, w=1.0 / 3.0, len=LEN,
              c75=0.75 * LEN, c43=4.0 / 3.0 * LEN)
 
 
@@ -39,20 +39,17 @@ def plain_inputs(fluid, scalar, rng):
 def slots(L, v, fluid, scalar):
     """The split form's inputs: differences in units of l without their field's l."""
     out = {}
-    merged = [*range(8, 14), *range(21, 24)] + [25 + 4 * fluid] * scalar
     for f in range(L["nf"]):
         d = 0 if 21 <= f < 24 else degree(f, fluid, scalar)
         out[f"u{f}"] = v[f"u{f}"] * LEN ** d
         if f in L["d1"]:
             for k in range(3):
                 out[f"d{f}_{k}"] = v[f"d{f}_{k}"] * LEN
-            out[f"k{f}"] = v[f"k{f}"]
+            adv = sum(v[f"u{18 + k}"] * out[f"d{f}_{k}"] for k in range(3))
+            out[f"m{f}"] = LEN ** degree(f, fluid, scalar) * (KO * v[f"k{f}"] + adv)
         if f in L["d2"]:
             for p in range(6):
                 out[f"dd{f}_{p}"] = v[f"dd{f}_{p}"] * LEN ** 2
-        if f in merged:
-            adv = sum(v[f"u{18 + k}"] * out[f"d{f}_{k}"] for k in range(3))
-            out[f"m{f}"] = LEN * (KO * v[f"k{f}"] + adv)
     out["kdiff"] = v["u7"] - KREF
     if fluid:
         out["rho"] = v["rho"] * LEN ** 2
@@ -85,7 +82,8 @@ def test_emitted_phases_read_their_own_region(fluid, scalar):
     L, v = plain_inputs(fluid, scalar, rng)
     val = slots(L, v, fluid, scalar)
     want = np.array(evaluate(g, out, val, SPLIT), dtype=float)
-    env = {"ina": [val[nm] for nm in S["a"]], "p": type("P", (), SPLIT), "sqrt": math.sqrt}
+    env = {"ina": [val[nm] for nm in S["a"]], "p": type("P", (), SPLIT), "sqrt": math.sqrt,
+           "k": type("K", (), dict(nz=-0.0, one=1.0, two=2.0, half=0.5)), "fma": lambda a, b, c: a * b + c}
     got = np.full(len(out), np.nan)
     body = src[src.index("{") + 1:src.rindex("}")]
     for line in body.split("\n"):
