@@ -186,10 +186,89 @@ __global__ void __launch_bounds__(BX* BY) vjp_cell_kernel(const VjpArgs a) {
   for (int f = 0; f < T::NF; ++f) a.VF[(long)f * fs + n.c] = vf[f];
 }
 
+// Stencils of the reverse sweep, in three-register multiply-adds (fp64_regs.cuh)
+// with the coefficients in registers.
+struct RevCoef {
+  double d1a[3], d1b[3], d2a[3], d2b[3];
+  Fp64Regs k;
+};
+
+// The coefficients through shared memory: read from there they are registers
+// for the compiler, read from the kernel's arguments they become constant operands.
+__device__ __forceinline__ RevCoef rev_coef(const Coef& c, double (&s)[12]) {
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  if (t == 0) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      s[d] = c.d1a[d];
+      s[3 + d] = c.d1b[d];
+      s[6 + d] = c.d2a[d];
+      s[9 + d] = c.d2b[d];
+    }
+  }
+  __syncthreads();
+  RevCoef r;
+  const volatile double* v = s;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    r.d1a[d] = v[d];
+    r.d1b[d] = v[3 + d];
+    r.d2a[d] = v[6 + d];
+    r.d2b[d] = v[9 + d];
+  }
+  r.k = fp64_regs();
+  return r;
+}
+
+// v - D_d F
+template <int D>
+__device__ __forceinline__ double sub_d1(double v, const double* __restrict__ F, const Nbr& n, const RevCoef& c) {
+  const double a = sub3(ldg(F, disp<D>(n, 1)), ldg(F, disp<D>(n, -1)), c.k);
+  const double b = sub3(ldg(F, disp<D>(n, 2)), ldg(F, disp<D>(n, -2)), c.k);
+  return fma(-c.d1a[D], a, fma(c.d1b[D], b, v));
+}
+
+// v + D_dd F
+template <int D>
+__device__ __forceinline__ double add_d2(double v, const double* __restrict__ F, const Nbr& n, const RevCoef& c) {
+  const double f0 = ldg(F, n.c);
+  const double s1 = add3(sub3(ldg(F, disp<D>(n, 1)), f0, c.k), sub3(ldg(F, disp<D>(n, -1)), f0, c.k), c.k);
+  const double s2 = add3(sub3(ldg(F, disp<D>(n, 2)), f0, c.k), sub3(ldg(F, disp<D>(n, -2)), f0, c.k), c.k);
+  return fma(c.d2a[D], s1, fma(-c.d2b[D], s2, v));
+}
+
+// First half of the transposed mixed stencils.  With the second-derivative
+// cotangents c_ab of a field and its first-derivative ones d_a,
+//   -D_x d_x + D_x D_y c_xy + D_x D_z c_xz = -D_x (d_x - D_y c_xy - D_z c_xz),
+//   -D_y d_y + D_y D_z c_yz = -D_y (d_y - D_z c_yz):
+// the brackets replace d_x and d_y here, three first derivatives per field instead of
+// three 16-point stencils in the second half (FP64-bound: 250 against 720 operations
+// per point for the 11 fields).
+template <class T>
+__global__ void __launch_bounds__(BX* BY) vjp_fold_kernel(const VjpArgs a) {
+  __shared__ double cf[12];
+  const RevCoef c = rev_coef(a.c, cf);
+  const int i = blockIdx.x * BX + threadIdx.x;
+  const int j = blockIdx.y * BY + threadIdx.y;
+  const int k = blockIdx.z;
+  if (i >= a.g.nx || j >= a.g.ny) return;
+  const Nbr n = make_nbr(a.g, i, j, k);
+  const long fs = a.g.fstride;
+#pragma unroll 1
+  for (int m2 = 0; m2 < T::ND2; ++m2) {
+    double* d = a.CB + (long)(T::NF + 3 * T::d1_slot(T::d2_field(m2))) * fs;
+    const double* C = a.CB + (long)(T::NF + 3 * T::ND1 + 6 * m2) * fs;
+    d[n.c] = sub_d1<1>(sub_d1<2>(d[n.c], C + 2 * fs, n, c), C + fs, n, c);
+    d[fs + n.c] = sub_d1<2>(d[fs + n.c], C + 4 * fs, n, c);
+  }
+}
+
 // Transposed stencils + RK4 reverse-sweep accumulation, one field at a time
-// (each v_f depends on the cotangents of field f only).
+// (each v_f depends on the cotangents of field f only), after vjp_fold_kernel.
 template <class T>
 __global__ void __launch_bounds__(BX* BY, 3) vjp_pass2_kernel(const VjpArgs a) {
+  __shared__ double cf[12];
+  const RevCoef c = rev_coef(a.c, cf);
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y * BY + threadIdx.y;
   const int k = blockIdx.z;
@@ -203,24 +282,18 @@ __global__ void __launch_bounds__(BX* BY, 3) vjp_pass2_kernel(const VjpArgs a) {
     const int m = T::d1_slot(f);
     if (m >= 0) {
       const double* G = a.CB + (long)(T::NF + 3 * m) * fs;
-      v -= fd1<0>(G, n, a.c) + fd1<1>(G + fs, n, a.c) + fd1<2>(G + 2 * fs, n, a.c);
+      v = sub_d1<2>(sub_d1<1>(sub_d1<0>(v, G, n, c), G + fs, n, c), G + 2 * fs, n, c);
     }
     const int m2 = T::d2_slot(f);
     if (m2 >= 0) {
       const double* G = a.CB + (long)(T::NF + 3 * T::ND1 + 6 * m2) * fs;
-      double s = fd2<0>(G, n, a.c, ldg(G, n.c));
-      s += fdmix<0, 1>(G + fs, n, a.c.mix[0]);
-      s += fdmix<0, 2>(G + 2 * fs, n, a.c.mix[1]);
-      s += fd2<1>(G + 3 * fs, n, a.c, ldg(G + 3 * fs, n.c));
-      s += fdmix<1, 2>(G + 4 * fs, n, a.c.mix[2]);
-      s += fd2<2>(G + 5 * fs, n, a.c, ldg(G + 5 * fs, n.c));
-      v += s;
+      v = add_d2<2>(add_d2<1>(add_d2<0>(v, G, n, c), G + 3 * fs, n, c), G + 5 * fs, n, c);
     }
     if (!(T::FLUID && f >= 24 && f < 28)) {  // KO is symmetric: KO^T w = KO w
       const double* Wf = a.W + (long)f * fs;
-      v = ko_equal ? v + ko_uniform(Wf, n, a.c, ldg(Wf, n.c)) : ko_add(Wf, n, a.c, ldg(Wf, n.c), v);
+      v = ko_equal ? ko_add_uniform(Wf, n, a.c, ldg(Wf, n.c), v, c.k) : ko_add(Wf, n, a.c, ldg(Wf, n.c), v);
     }
-    if constexpr (T::FLUID) v += ldg(a.VF + (long)f * fs, n.c);
+    if constexpr (T::FLUID) v = add3(v, ldg(a.VF + (long)f * fs, n.c), c.k);
     const long o = (long)f * fs + n.c;
     a.lam[o] += v;
     if (a.knext) a.knext[o] = a.a_lam * ldg(a.lam0, o) + a.a_v * v;
@@ -261,6 +334,8 @@ struct T_vac_adj {
       vjp_cell_kernel<A_##NAME><<<grid, block, 0, s>>>(a);                                                      \
       if ((e = cudaGetLastError()) != cudaSuccess) return e;                                                    \
     }                                                                                                           \
+    vjp_fold_kernel<A_##NAME><<<grid, block, 0, s>>>(a);                                                        \
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;                                                      \
     vjp_pass2_kernel<A_##NAME><<<grid, block, 0, s>>>(a);                                                       \
     return cudaGetLastError();                                                                                  \
   }

@@ -79,26 +79,22 @@ __device__ __forceinline__ double ko_add(const double* __restrict__ F, const Nbr
   return r;
 }
 
-// Kreiss-Oliger term of a field on a grid with equal spacing along the three
-// axes (one coefficient c.ko[0]): the bracket is linear in s_k, so the three
+// v + the Kreiss-Oliger term of a field on a grid with equal spacing along the
+// three axes (one coefficient c.ko[0]): the bracket is linear in s_k, so the three
 // axes are summed first, P_k = sum_d (f(+k e_d) + f(-k e_d)), and combined once:
 // (P3 - P2) - 5 (P2 - P1) + 10 (P1 - 6 f0).  For a constant field every P_k and
 // 6 f0 are the same single rounding of 6 f0, so each bracket is exactly zero.
-// ko_bracket returns the bracket; the term is c.ko[0] times it.
-__device__ __forceinline__ double ko_bracket(const double* __restrict__ F, const Nbr& n, double f0) {
+__device__ __forceinline__ double ko_add_uniform(const double* __restrict__ F, const Nbr& n, const Coef& c, double f0,
+                                                 double v, const Fp64Regs& k) {
   double P[3];
 #pragma unroll
-  for (int k = 1; k <= 3; ++k)
-    P[k - 1] = ((ldg(F, disp<0>(n, k)) + ldg(F, disp<0>(n, -k))) + (ldg(F, disp<1>(n, k)) + ldg(F, disp<1>(n, -k)))) +
-               (ldg(F, disp<2>(n, k)) + ldg(F, disp<2>(n, -k)));
-  const double t = P[0] - __dmul_rn(6.0, f0);  // __dmul_rn: the product is rounded, never fused
-  return fma(10.0, t, fma(-5.0, P[1] - P[0], P[2] - P[1]));
+  for (int o = 1; o <= 3; ++o)
+    P[o - 1] = add3(add3(add3(ldg(F, disp<0>(n, o)), ldg(F, disp<0>(n, -o)), k),
+                         add3(ldg(F, disp<1>(n, o)), ldg(F, disp<1>(n, -o)), k), k),
+                    add3(ldg(F, disp<2>(n, o)), ldg(F, disp<2>(n, -o)), k), k);
+  const double t = sub3(P[0], __dmul_rn(6.0, f0), k);  // __dmul_rn: the product is rounded, never fused
+  return fma(c.ko[0], fma(10.0, t, fma(-5.0, sub3(P[1], P[0], k), sub3(P[2], P[1], k))), v);
 }
-
-__device__ __forceinline__ double ko_uniform(const double* __restrict__ F, const Nbr& n, const Coef& c, double f0) {
-  return c.ko[0] * ko_bracket(F, n, f0);
-}
-
 
 // Inputs of the generated algebra at one point (layout documented in codegen/bssn.py).
 template <class T>
