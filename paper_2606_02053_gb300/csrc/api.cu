@@ -388,10 +388,10 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
   const int nslot = 24 + 2 * p->scalar;
   if (expo_flags & 2) {
     a.E_rec = (unsigned*)(ws + L.erec);
+    a.E_next = (int*)(ws + L.expo);
     if (expo_flags & 4) CK(cudaMemsetAsync(a.E_rec, 0, sizeof(unsigned) * 32 * nslot, s));
   }
   if (pass_mask & 4) CK(stage_launcher(p)(a, mode, k_cnt > 0 ? k_cnt : g->nz, s));
-  if ((expo_flags & 2) && (pass_mask & 4)) CK(launch_exponents_from_record(a.E_rec, (int*)(ws + L.expo), nslot, s));
   return COSMOS_OK;
 }
 

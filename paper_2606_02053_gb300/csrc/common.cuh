@@ -102,6 +102,8 @@ struct StageArgs {
   const int* __restrict__ E;       // reference exponent of each limb slot
   unsigned* E_rec;                 // stages 1-3: records the largest biased exponent of each limb
                                    // slot of U_next at E_rec[32 slot] (null: no record)
+  int* E_next;                     // one grid: the block that ends last moves the record there and clears it
+                                   // (E_rec[1] counts the blocks that have ended; null: it stays)
 };
 // Fills the units of `a` (its grid, ap, cdt given) for dissipation sigma.
 void set_units(StageArgs* a, double sigma, double bk);

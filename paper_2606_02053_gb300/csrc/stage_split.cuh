@@ -641,6 +641,19 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       atomicMax(a.E_rec + 32 * t, (unsigned)rec[t]);
       rec[t] = 0;
     }
+    if (!BATCH && g == 0 && a.E_rec && a.E_next) {
+      // the last block to end (no block waits for another) leaves the record as the exponents of
+      // the next stage, and clean; every block has read the exponents of this stage by then
+      __threadfence();
+      bar_sync(BAR_GROUP, SPLIT_PTS);
+      if (t == 0) rec[31] = (int)atomicAdd(a.E_rec + 1, 1u);
+      bar_sync(BAR_GROUP, SPLIT_PTS);
+      if (rec[31] == (int)gridDim.x - 1) {
+        __threadfence();
+        if (t < NSLOT) a.E_next[t] = (int)atomicExch(a.E_rec + 32 * t, 0u);
+        if (t == 0) a.E_rec[1] = 0u;
+      }
+    }
   };
   if (blockIdx.x >= ntiles) return;
   SplitTile cur = tile_at(blockIdx.x);
