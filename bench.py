@@ -176,7 +176,7 @@ def flrw_workload(args):
                                              "Linf_My", "Linf_Mz"],
                                  "rows": [[s] + v for s, v in norms]},
             "initial_data_ms": init_ms, "constraints_ms_per_evaluation": constraints_ms,
-            "gpu_launches": steps * 4 * 6}  # per stage: primitives, fluxes, exponents, limbs, derivative, algebra
+            "gpu_launches": steps * 17}  # exponent scan, 4 x (primitives, fluxes, limb copy, stage)
     print(json.dumps(line), flush=True)
 
 
@@ -219,7 +219,7 @@ def isocurvature_workload(args):
                        "sigma": 0.125, "q": [1.0, 0.9, 1.1], "H0L": 40.0, "dt_over_h": 0.25},
             "constraint_norms": {"columns": ["L2_H", "L2_Mx", "L2_My", "L2_Mz", "Linf_H", "Linf_Mx", "Linf_My",
                                              "Linf_Mz"], "start": norms0, "end": norms1},
-            "gpu_launches": steps * 4 * 6}
+            "gpu_launches": steps * 17}
     print(json.dumps(line), flush=True)
 
 
@@ -270,7 +270,7 @@ def mode_workload(args):
             "config": {"workload": "single_mode_128^3_radiation_fluid", "grid": n, "eps": eps, "H0": H0,
                        "t_end": steps * dt, "dt_over_h": 0.25, "slicing": "harmonic", "shift": "frozen"},
             "K_mode_amplitude_end": [amp.real, amp.imag],
-            "gpu_launches": steps * 4 * 6}
+            "gpu_launches": steps * 17}
     print(json.dumps(line), flush=True)
 
 
@@ -342,7 +342,7 @@ def fmr_workload(args):
     ms_plain = e0.elapsed_time(e1)
     del evs
     value = interior * args.steps / (ms * 1e-3)
-    launches_per_level_step = 24  # 4 stages x (primitives, fluxes, exponents, limbs, derivative, algebra)
+    launches_per_level_step = 20  # 4 stages x (primitives, fluxes, exponents, limb copy, stage)
     launches_per_fill = 4         # time interpolation, x, y and z passes
     launches = sum(2 ** l * (launches_per_level_step + (4 * launches_per_fill if l else 0)) for l in range(nlev))
     launches += sum(2 ** (l - 1) for l in range(1, nlev))  # injections
@@ -430,7 +430,7 @@ def measure_scan(n_instances, K, W, rank=0, world=1, autotune=True):
             "per_instance_loop_value": total_pts * K / t_loop, "speedup": t_loop / t_batch,
             "ms_per_step": 1e3 * t_batch / K, "loop_ms_per_step": 1e3 * t_loop / K,
             "max_abs_diff_vs_loop": max_diff, "max_rel_diff_vs_loop": max_diff / scale, "autotune": tune,
-            "gpu_launches": K * 4 * 6}  # per stage: primitives, fluxes, exponents, limbs, derivative, algebra
+            "gpu_launches": K * 20}  # exponent scan, 4 x (primitives, fluxes, limb copy, stage), 3 x exponent record
 
 
 def scan_workload(args):
@@ -682,7 +682,7 @@ def measure_adjoint(n, steps, every=16, point_checks=True):
            "peak_shell": rec["kstar"], "dmin_dmu": float(g_mu_min), "dcomp_dmu": g_mu_comp,
            "mu_fd_rel_diff_min_lapse": rel(mu_check["fd_min_lapse"], float(g_mu_min)),
            "mu_fd_rel_diff_compaction": rel(mu_check["fd_compaction"], g_mu_comp),
-           "gpu_launches_per_forward_step": 16 + 8 + 1}  # 4 stages x 6 kernels + the central-lapse read
+           "gpu_launches_per_forward_step": 17 + 1}  # exponent scan, 4 stages x 4 kernels, the central-lapse read
     if point_checks:
         res["fd_checks"] = checks
         res["worst_rel_diff_min_lapse"] = max(rel(c["fd_min_lapse"], c["adj_min_lapse"]) for c in checks)
@@ -767,7 +767,7 @@ def decomposed_workload(args):
                 "config": {"workload": WORKLOAD, "grid": n, "fields": STATE_FIELDS, "dt_over_h": 0.25,
                            "parallelism": f"z-slabs x{ws_} (3 ghost planes a side, exchange every stage)",
                            "l2": "inputs larger than L2 (3.2 GB state per level)"},
-                "gpu_launches": 16 * args.steps, "clocks": clk}
+                "gpu_launches": 12 * args.steps, "clocks": clk}  # 4 x (exponent scan, limb copy, stage)
         print(json.dumps(line), flush=True)
     if ws_ > 1:
         tdist.destroy_process_group()
@@ -876,9 +876,8 @@ def main():
     nranks = ws_
     pts = float(n) ** 3
     value = nranks * pts * args.steps / elapsed
-    # per step: exponent scan (stage 1), 4 x (limb copy, stage kernel), exponent record compaction
-    # (stages 1-3)
-    gpu_launches = 12 * args.steps
+    # per step: exponent scan (stage 1), 4 x (limb copy, stage kernel)
+    gpu_launches = 9 * args.steps
 
     # ---- end to end through the C ABI with host buffers (pinned) ----
     # Every step copies its inputs from pinned host memory and reads its result
@@ -996,9 +995,9 @@ def main():
         # loops form every symmetric component twice) and its stencils as FP64 operations.
         alg_flops = generated_algebra_ops("vac") + 2 * STATE_FIELDS + combine
         oracle_flops = {"stencils": fl(parts["derivatives"]) + fl(parts["ko"]), "algebra": fl(parts["algebra"]) + combine}
-        # the state read and its limb copy written; the limb copy read and the stage's states
-        bytes_point = {"limbs": 8 * 2 * STATE_FIELDS,
-                       "stage": 8 * STATE_FIELDS + statistics.mean(BYTES_PER_POINT_STAGE)}
+        # the state read, its limb copy, inverse metric and 1/chi written; these read and the stage's states
+        bytes_point = {"limbs": 8 * (2 * STATE_FIELDS + 7),
+                       "stage": 8 * (STATE_FIELDS + 7) + statistics.mean(BYTES_PER_POINT_STAGE)}
         peak = fp64_peak / 1e12
         hbm_peak, hbm_src = hbm_peak_gbs()
         traffic_ok = kernel_sources_hash() == NCU_TRAFFIC["sources_sha256_16"]

@@ -32,7 +32,9 @@ summed before it does, and what the trace-free projection removes is not
 formed.  Vacuum: 817 FP64 instructions per point (765 products, 651 sums)
 against 973 for the textbook grouping, fluid 939 against 1148, reverse mode
 2117 against 2480, constraints 571 against 777; a 256^3 vacuum RK4 step went
-from 169.0 to 153.3 ms and a 128^3 fluid one from 39.1 to 36.3 ms.
+from 169.0 to 153.3 ms and a 128^3 fluid one from 39.1 to 36.3 ms.  The stage
+kernel's form (inverse metric, 1/chi and the advection formed elsewhere) has 718
+in vacuum, 840 with the fluid.
 """
 from __future__ import annotations
 
@@ -90,7 +92,9 @@ def split_layout(fluid: bool, scalar: bool):
     Per field with second derivatives ten slots (d_k, dd_p, m), per field with
     first derivatives four (d_k, m), a field whose derivatives only advect it has
     m alone: its whole advection with the dissipation term (that of the metric
-    and Gamma is read at the end of the first phase).  kdiff = K - Kref.  ``out`` =
+    and Gamma is read at the end of the first phase).  The inverse metric gu, 1/chi
+    (ichi) and kdiff = K - Kref are formed outside; the shift's slots serve the
+    advections, the algebra does not read them.  ``out`` =
     the region-B slot that takes output f: its m slot (read by that output alone)
     or r{f}.
 
@@ -117,7 +121,8 @@ def split_layout(fluid: bool, scalar: bool):
     for f in range(GAM, GAM + 3):
         a += d1(f)
     early = not fluid
-    a += [f"u{f}" for f in [*range(GT, GT + 6), *range(BET, BET + 3)] + [*range(AT, AT + 6)] * early]
+    a += [f"u{f}" for f in [*range(GT, GT + 6), *range(BET, BET + 3)]] + [f"gu{m}" for m in range(6)]
+    a += [f"u{f}" for f in range(AT, AT + 6)] * early
     if fluid:
         a += ["u0", "u24", "u25", "u26", "u27", "rho"]
     ph = 24 + 4 * fluid
@@ -125,7 +130,7 @@ def split_layout(fluid: bool, scalar: bool):
         b += d2(f)
     b += d1(TRK)
     b += [f"m{f}" for f in [*range(AT, AT + 6), *range(BB, BB + 3)] + [ph + 1] * scalar]
-    b += [f"u{f}" for f in [*range(0, GAM), *range(ALP, 24)]] + ["kdiff"]
+    b += [f"u{f}" for f in [*range(0, GAM), ALP, *range(BB, BB + 3)]] + ["kdiff", "ichi"]
     if fluid:
         b += ["u24", "u25", "u26", "u27", "rho"]
     if scalar:
@@ -199,9 +204,9 @@ def algebra(fluid: bool, scalar: bool, split: bool = False):
     c12 = gt[0, 1] * gt[0, 2] - gt[0, 0] * gt[1, 2]
     c22 = gt[0, 0] * gt[1, 1] - gt[0, 1] * gt[0, 1]
     idet = (gt[0, 0] * c00 + gt[0, 1] * c01 + gt[0, 2] * c02).rcp()
-    gu = Sym([c00 * idet, c01 * idet, c02 * idet, c11 * idet, c12 * idet, c22 * idet])
+    gu = Sym([g.input(f"gu{m}") if split else c * idet for m, c in enumerate([c00, c01, c02, c11, c12, c22])])
     gu2 = [gu[i, j] * (1.0 if i == j else 2.0) for (i, j) in PAIRS]  # doubled off-diagonals
-    ichi = chi.rcp()
+    ichi = g.input("ichi") if split else chi.rcp()
 
     # ---- Christoffels.  Gl2[k][(i,j)] = 2 Gamma_kij (first kind, doubled: the
     # factors 1/2 cost nothing where they are folded into factors formed once) ----

@@ -17,7 +17,7 @@ constexpr int kAlphaField = 17;  // the lapse's place in the state's field order
 static size_t a256(size_t doubles) { return ((doubles * 8 + 255) & ~(size_t)255) / 8; }
 
 struct AdjLayout {
-  size_t U2, U3, U4, KB, KB2, LAM, Dfw, CB, prim, flux, vprim, FC, VF, CB10, limbs, expo, total_bytes;
+  size_t U2, U3, U4, KB, KB2, LAM, Dfw, CB, prim, flux, vprim, FC, VF, CB10, limbs, G, expo, total_bytes;
 };
 
 static int nin_of(const cosmos_params* p) {
@@ -67,6 +67,7 @@ static AdjLayout adj_layout(const cosmos_grid* g, const cosmos_params* p, int op
     // linearisation points
     const int nslot = 24 + 2 * p->scalar;
     L.limbs = take((size_t)nslot * fs);
+    if (op == COSMOS_OP_ADJOINT) L.G = take(7 * fs);  // of the forward stages
     L.expo = take(((size_t)nslot + 1) / 2);
     L.CB = take(nin_of(p) * fs);
     if (p->fluid) {
@@ -98,11 +99,11 @@ static int check_ws_adj(size_t need, void* ws, size_t ws_bytes) {
 
 // Limb copy of every derivative field of U.
 static cudaError_t limbs_of(const cosmos_params* p, const DevGrid& g, const double* U, double* ws, const AdjLayout& L,
-                            StageArgs& a, cudaStream_t s) {
+                            StageArgs& a, double* G, cudaStream_t s) {
   const int nslot = 24 + 2 * p->scalar;
   a.L = (const long long*)(ws + L.limbs);
   a.E = (const int*)(ws + L.expo);
-  return launch_limbs(g, U, p->fluid, 0, nslot, (int*)(ws + L.expo), (long long*)(ws + L.limbs), s);
+  return launch_limbs(g, U, p->fluid, 0, nslot, (int*)(ws + L.expo), (long long*)(ws + L.limbs), G, s);
 }
 
 static FluidParams fparams(double w) {
@@ -142,7 +143,7 @@ static cudaError_t vjp_once(const cosmos_grid* g, const cosmos_params* p, const 
   d.need = ~0u;
   a.D = d.D;
   {
-    cudaError_t e = limbs_of(p, d.g, U, ws, L, d, s);
+    cudaError_t e = limbs_of(p, d.g, U, ws, L, d, nullptr, s);
     if (e == cudaSuccess) e = launch_deriv_for(p, d, s);
     if (e != cudaSuccess) return e;
   }
@@ -182,6 +183,7 @@ static cudaError_t fwd_stage(const cosmos_grid* g, const cosmos_params* p, const
   a.out = out;
   a.acc = acc;
   a.cdt = cdt;
+  a.G = ws + L.G;
   set_units(&a, p->ko_sigma, 2.0);
   if (p->fluid) {
     cudaError_t e = launch_fluid_prim(a.g, U_s, ws + L.prim, p->w, s);
@@ -190,7 +192,7 @@ static cudaError_t fwd_stage(const cosmos_grid* g, const cosmos_params* p, const
     a.prim = ws + L.prim;
     a.flux = ws + L.flux;
   }
-  const cudaError_t e = limbs_of(p, a.g, U_s, ws, L, a, s);
+  const cudaError_t e = limbs_of(p, a.g, U_s, ws, L, a, ws + L.G, s);
   if (e != cudaSuccess) return e;
   return launch_stage_for(p, a, MODE_S1, g->nz, s);
 }

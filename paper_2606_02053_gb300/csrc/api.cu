@@ -147,6 +147,7 @@ WsLayout ws_layout(const cosmos_grid* g, const cosmos_params* p, int op) {
     // derivatives, and their exponents
     const int nslot = 24 + 2 * p->scalar;
     L.limbs = take((size_t)nslot * fs);
+    L.G = take(7 * fs);  // inverse conformal metric, 1/chi
     L.expo = take(((size_t)nslot + 1) / 2);
     L.erec = take(16 * (size_t)nslot);  // 32 unsigned per slot, one cache line each
     if (op == COSMOS_OP_RK4) {
@@ -387,6 +388,7 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
   set_units(&a, p->ko_sigma, bk);
   a.L = (const long long*)(ws + L.limbs);
   a.E = E_ext ? E_ext : (const int*)(ws + L.expo);
+  a.G = ws + L.G;
   if (p->fluid) {
     double* prim = ws + L.prim;
     double* flux = ws + L.flux;
@@ -408,11 +410,11 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
       s_hi = sl + 1 > s_hi ? sl + 1 : s_hi;
     }
     if (E_ext) {
-      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, E_ext, (long long*)(ws + L.limbs), s));
+      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, E_ext, (long long*)(ws + L.limbs), ws + L.G, s));
     } else if (expo_flags & 1) {  // exponents recorded by the previous stage
-      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, a.E, (long long*)(ws + L.limbs), s));
+      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, a.E, (long long*)(ws + L.limbs), ws + L.G, s));
     } else {
-      CK(launch_limbs(a.g, U_s, p->fluid, s_lo, s_hi, (int*)(ws + L.expo), (long long*)(ws + L.limbs), s));
+      CK(launch_limbs(a.g, U_s, p->fluid, s_lo, s_hi, (int*)(ws + L.expo), (long long*)(ws + L.limbs), ws + L.G, s));
     }
   }
   const int nslot = 24 + 2 * p->scalar;
@@ -887,7 +889,7 @@ int cosmos_constraints(const cosmos_grid* g, const cosmos_params* p, const doubl
     d.dfs = plane * L.chunk;
     // all fields but the lapse, the shift and B^i (slots 17 .. 23) and Pi (25)
     d.need = ~(0x7Fu << 17 | 1u << 25);
-    CK(launch_limbs(d.g, state, p->fluid, 0, nslot, (int*)(w + L.expo), (long long*)(w + L.limbs), s));
+    CK(launch_limbs(d.g, state, p->fluid, 0, nslot, (int*)(w + L.expo), (long long*)(w + L.limbs), nullptr, s));
     for (int k0 = 0; k0 < g->nz; k0 += L.chunk) {
       d.k_lo = c.k_lo = k0;
       c.k_cnt = std::min(L.chunk, g->nz - k0);

@@ -46,7 +46,7 @@ static long max_tiles(const cosmos_grid& g) {
 }
 
 struct BatchLayout {
-  std::vector<size_t> A, B, acc, prim, flux, limbs;  // per instance, in doubles from ws
+  std::vector<size_t> A, B, acc, prim, flux, limbs, G;  // per instance, in doubles from ws
   size_t args, tiles, stiles, kref, expo, erec;         // byte offsets (expo: n x nslot exponents; erec:
                                                         // the stages' record, 32 unsigned per slot)
   size_t total;
@@ -78,6 +78,7 @@ static BatchLayout batch_layout(int n, const cosmos_grid* grids, const cosmos_pa
     L.prim.push_back(p->fluid ? take(4 * fs * 8) / 8 : 0);
     L.flux.push_back(p->fluid ? take(12 * fs * 8) / 8 : 0);
     L.limbs.push_back(take((size_t)nslot_of(p) * fs * 8) / 8);
+    L.G.push_back(take(7 * fs * 8) / 8);
     tiles += max_tiles(grids[i]);
     stiles += stage_tiles(grids[i]);
   }
@@ -230,6 +231,7 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
       set_units(&a, p->ko_sigma, 2.0);
       b->eq = b->eq && a.eq;
       a.L = (const long long*)(wsd + L.limbs[i]);
+      a.G = wsd + L.G[i];
       a.E = (const int*)(b->ws + L.expo) + (size_t)i * nslot_of(p);
       // stages 1-3 record the exponents of the state they write for the next stage
       if (s < 3) a.E_rec = (unsigned*)(b->ws + L.erec) + 32 * (size_t)i * nslot_of(p);

@@ -6,7 +6,9 @@
 // which nothing reads; the scan leaves them out), LIMB_RUN values per block and
 // turn, LIMB_EACH of them in flight per thread.  By rows, a 32-point row kept half
 // of a block idle: 24 fields of 32^3: copy 15.3 -> 4.7 us, scan 33 -> 5.3; 64^3: copy
-// 50 -> 14 us; 256^3: 0.89 ms, 7.2 TB/s.
+// 50 -> 14 us; 256^3: 0.89 ms, 7.2 TB/s.  With the inverse metric and 1/chi beside it
+// 256^3 takes 1.1 ms, and the step, whose algebra no longer forms them, 132.6 ->
+// 127.1 ms (generic 250 x 198 x 203: 80.3 -> 78.2).
 #include "stage_kernel.cuh"
 
 namespace cosmos {
@@ -39,8 +41,8 @@ __device__ __forceinline__ void scan_slot(const DevGrid& g, const double* __rest
 }
 
 __device__ __forceinline__ void copy_slot(const DevGrid& g, const double* __restrict__ F, int e_ref,
-                                          long long* __restrict__ L) {
-  for (long o = (long)blockIdx.x * LIMB_RUN + threadIdx.x; o < g.fstride; o += (long)gridDim.x * LIMB_RUN) {
+                                          long long* __restrict__ L, long first, long stride) {
+  for (long o = first * LIMB_RUN + threadIdx.x; o < g.fstride; o += stride * LIMB_RUN) {
     double v[LIMB_EACH];
 #pragma unroll
     for (int q = 0; q < LIMB_EACH; ++q) v[q] = o + q * LIMB_THREADS < g.fstride ? __ldg(F + o + q * LIMB_THREADS) : 0.0;
@@ -50,10 +52,53 @@ __device__ __forceinline__ void copy_slot(const DevGrid& g, const double* __rest
   }
 }
 
+// Limb copies of chi and the conformal metric (slots 0 .. 6) and, of the same loads, the inverse metric and
+// 1/chi of each point into G: blocks first, first + stride, .. of LIMB_THREADS points.  The stage's algebra
+// has one warp per scheduler, which the latency of the determinant and its reciprocal bounds; here many warps
+// are in flight and the FP64 instructions run beside the copies of the other slots, whose bound is memory.
+__device__ __forceinline__ void copy_metric(const DevGrid& g, const double* __restrict__ U, const int* __restrict__ E,
+                                            long long* __restrict__ L, double* __restrict__ G, long first, long stride) {
+  const Fp64Regs k = fp64_regs();
+  const long fs = g.fstride;
+  for (long o = first * LIMB_THREADS + threadIdx.x; o < fs; o += stride * LIMB_THREADS) {
+    double v[7];
+#pragma unroll
+    for (int m = 0; m < 7; ++m) v[m] = __ldg(U + m * fs + o);
+    if (L) {  // null: G alone
+#pragma unroll
+      for (int m = 0; m < 7; ++m) L[m * fs + o] = to_limbs(v[m], max(E[m], 1));
+    }
+    const double* q = v + 1;  // xx xy xz yy yz zz
+    const double c[6] = {fma(-q[4], q[4], mul3(q[3], q[5], k)), fma(-q[1], q[5], mul3(q[2], q[4], k)),
+                         fma(-q[2], q[3], mul3(q[1], q[4], k)), fma(-q[2], q[2], mul3(q[0], q[5], k)),
+                         fma(-q[0], q[4], mul3(q[1], q[2], k)), fma(-q[1], q[1], mul3(q[0], q[3], k))};
+    const double idet = 1.0 / fma(q[2], c[2], fma(q[1], c[1], mul3(q[0], c[0], k)));
+#pragma unroll
+    for (int m = 0; m < 6; ++m) G[m * fs + o] = mul3(c[m], idet, k);
+    G[6 * fs + o] = 1.0 / v[0];
+  }
+}
+
+// Work of one block in a pass over all slots below s_hi (> 6) with G: of every LIMB_EACH + s_hi - 7 blocks, the
+// first LIMB_EACH take LIMB_RUN points of chi and the metric, the others LIMB_RUN points of one slot each, so
+// that the two kinds are on an SM together.
+__device__ __forceinline__ void copy_all(const DevGrid& g, const double* __restrict__ U, int s_hi, int fluid,
+                                         const int* __restrict__ E, long long* __restrict__ L, double* __restrict__ G) {
+  const int each = LIMB_EACH + s_hi - 7, q = blockIdx.x % each;
+  const long c = blockIdx.x / each, nc = gridDim.x / each;
+  if (q < LIMB_EACH) {
+    copy_metric(g, U, E, L, G, c * LIMB_EACH + q, nc * LIMB_EACH);
+  } else {
+    const int s = 7 + q - LIMB_EACH;
+    copy_slot(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride, c, nc);
+  }
+}
+
 // blockIdx.y = slot (from s_lo)
 __global__ void __launch_bounds__(LIMB_THREADS) field_exponent_kernel(const DevGrid g, const double* __restrict__ U,
                                                                       int s_lo, int fluid, int* __restrict__ E) {
   const int s = s_lo + blockIdx.y;
+  grid_trigger();
   scan_slot(g, U + (long)limb_field(s, fluid) * g.fstride, (unsigned*)E + s);
 }
 
@@ -61,7 +106,21 @@ __global__ void __launch_bounds__(LIMB_THREADS) to_limbs_kernel(const DevGrid g,
                                                                 int fluid, const int* __restrict__ E,
                                                                 long long* __restrict__ L) {
   const int s = s_lo + blockIdx.y;
-  copy_slot(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride);
+  copy_slot(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride, blockIdx.x, gridDim.x);
+}
+
+// all slots below s_hi (> 6) with G
+__global__ void __launch_bounds__(LIMB_THREADS) to_limbs_all_kernel(const DevGrid g, const double* __restrict__ U,
+                                                                    int s_hi, int fluid, const int* __restrict__ E,
+                                                                    long long* __restrict__ L, double* __restrict__ G) {
+  grid_wait();
+  copy_all(g, U, s_hi, fluid, E, L, G);
+}
+
+// G alone
+__global__ void __launch_bounds__(LIMB_THREADS) metric_kernel(const DevGrid g, const double* __restrict__ U,
+                                                              double* __restrict__ G) {
+  copy_metric(g, U, nullptr, nullptr, G, blockIdx.x, gridDim.x);
 }
 
 // The same for a batch: blockIdx.z = instance; the arguments of instance i are
@@ -72,11 +131,12 @@ __global__ void __launch_bounds__(LIMB_THREADS) batch_field_exponent_kernel(cons
   scan_slot(g, a.U + (long)limb_field(blockIdx.y, fluid) * g.fstride, (unsigned*)a.E + blockIdx.y);
 }
 
-__global__ void __launch_bounds__(LIMB_THREADS) batch_to_limbs_kernel(const StageArgs* __restrict__ args, int fluid) {
-  const StageArgs& a = args[blockIdx.z];
-  const DevGrid g = a.g;
-  copy_slot(g, a.U + (long)limb_field(blockIdx.y, fluid) * g.fstride, max(a.E[blockIdx.y], 1),
-            const_cast<long long*>(a.L) + (long)blockIdx.y * g.fstride);
+// blockIdx.y = instance
+__global__ void __launch_bounds__(LIMB_THREADS) batch_to_limbs_kernel(const StageArgs* __restrict__ args, int nslot,
+                                                                      int fluid) {
+  grid_wait();
+  const StageArgs& a = args[blockIdx.y];
+  copy_all(a.g, a.U, nslot, fluid, a.E, const_cast<long long*>(a.L), const_cast<double*>(a.G));
 }
 
 // Blocks along a slot: the copy has no turn to repeat up to the largest grids;
@@ -97,17 +157,27 @@ cudaError_t launch_batch_limbs(const StageArgs* args, int n, int nslot, int flui
 }
 
 cudaError_t launch_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, int* E, long long* L,
-                         cudaStream_t s) {
+                         double* G, cudaStream_t s) {
   const cudaError_t e = launch_field_exponents(g, U, fluid, s_lo, s_hi, E, s);
-  return e != cudaSuccess ? e : launch_to_limbs(g, U, fluid, s_lo, s_hi, E, L, s);
+  return e != cudaSuccess ? e : launch_to_limbs(g, U, fluid, s_lo, s_hi, E, L, G, s);
 }
 
 // The limb copy of slots s_lo .. s_hi - 1 with the reference exponents given
 // in E (no scan).
 cudaError_t launch_to_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, const int* E,
-                            long long* L, cudaStream_t s) {
+                            long long* L, double* G, cudaStream_t s) {
   if (s_hi <= s_lo) return cudaSuccess;
-  to_limbs_kernel<<<dim3(copy_blocks(g), (unsigned)(s_hi - s_lo)), LIMB_THREADS, 0, s>>>(g, U, s_lo, fluid, E, L);
+  const unsigned blocks = copy_blocks(g);
+  if (G && s_lo == 0 && s_hi > 6) {
+    return launch_early(to_limbs_all_kernel, dim3(blocks * (unsigned)(LIMB_EACH + s_hi - 7)), LIMB_THREADS, 0, s, g, U,
+                        s_hi, fluid, E, L, G);
+  }
+  if (G && s_lo <= 6 && s_hi > 6) {
+    metric_kernel<<<blocks * LIMB_EACH, LIMB_THREADS, 0, s>>>(g, U, G);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  to_limbs_kernel<<<dim3(blocks, (unsigned)(s_hi - s_lo)), LIMB_THREADS, 0, s>>>(g, U, s_lo, fluid, E, L);
   return cudaGetLastError();
 }
 
@@ -135,8 +205,8 @@ cudaError_t launch_exponents_from_record(unsigned* rec, int* E, int nslot, cudaS
 
 // The batched limb copy with the exponents already in args[i].E (no scan).
 cudaError_t launch_batch_to_limbs(const StageArgs* args, int n, int nslot, int fluid, cudaStream_t s) {
-  batch_to_limbs_kernel<<<dim3(BATCH_BLOCKS, (unsigned)nslot, (unsigned)n), LIMB_THREADS, 0, s>>>(args, fluid);
-  return cudaGetLastError();
+  return launch_early(batch_to_limbs_kernel, dim3(BATCH_BLOCKS * (unsigned)(LIMB_EACH + nslot - 7), (unsigned)n),
+                      LIMB_THREADS, 0, s, args, nslot, fluid);
 }
 
 }  // namespace cosmos

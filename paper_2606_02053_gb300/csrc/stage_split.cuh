@@ -1,8 +1,8 @@
 // One RK4 stage as one persistent kernel: finite differences, pointwise
 // algebra and stage combine of a tile side by side in one block.
 //
-// What bounds it: the algebra is FP64 work (799 instructions per point in
-// vacuum, Kreiss-Oliger terms included) at 2 multiply-adds per clock per SM
+// What bounds it: the algebra is FP64 work (718 instructions per point in
+// vacuum, 190 more in the advection, dissipation and combine beside it) at 2 multiply-adds per clock per SM
 // (lone multiplies and adds 1.7), and one warp per scheduler nearly keeps that
 // pipe full (a dependent chain of one warp issues one multiply-add per 64
 // cycles, its whole rate).  The finite differences are integer work
@@ -12,9 +12,8 @@
 // with 200 registers a thread and SPLIT_GROUPS difference warpgroups with 104,
 // and the differences of a tile (SPLIT_TX x SPLIT_TY points of one z-plane, a
 // point per algebra thread) go through shared memory.  256^3 vacuum stage: 10.0
-// + 27.5 ms as two kernels, 32.5 ms as this one (FP64 pipe 83% busy; its algebra
-// alone 29.5, its differences alone 25); 128^3 fluid 5.4 -> 4.8 ms; 20 x 12 x 9 145 ->
-// 40 us.  The algebra with 240 or 224 registers, the difference warps with 88 or 96,
+// + 27.5 ms as two kernels, 30.3 ms as this one (its algebra warps wait for the
+// others in under 3% of their time); 128^3 fluid 5.4 -> 4.6 ms.  The algebra with 240 or 224 registers, the difference warps with 88 or 96,
 // and four groups of 64 were within 1 to 3% and slower.
 //
 // The algebra runs in two phases of about equal length (codegen/bssn.py,
@@ -78,13 +77,15 @@ template <class T>
 struct Slots {
   static constexpr int A = T::SA, B = T::SB;
   // (d_k, dd_p, m of a second-derivative field; d_k, m of a first-derivative one)
-  // region A: 6 x 10 (metric), 3 x 4 (Gamma), metric, shift, At (SPLIT_EARLY), fluid: chi, tau, S_i, rho
+  // region A: 6 x 10 (metric), 3 x 4 (Gamma), metric, shift, inverse metric, At (SPLIT_EARLY), fluid: chi,
+  // tau, S_i, rho
   static constexpr int A_GT = 0, A_GAM = 60, A_STATE = 72;
-  static constexpr int A_NSTATE = 9 + (T::SPLIT_EARLY ? 6 : 0) + (T::FLUID ? 6 : 0);
+  static constexpr int A_NSTATE = 15 + (T::SPLIT_EARLY ? 6 : 0) + (T::FLUID ? 6 : 0);
   // region B: ND2B x 10 (chi, alpha, beta^i, phi), K (4), merged advections, states, output slots
   static constexpr int ND2B = 5 + (T::SCALAR ? 1 : 0), NM = 9 + (T::SCALAR ? 1 : 0);
   static constexpr int B_K = 10 * ND2B, B_M = B_K + 4, B_STATE = B_M + NM;
-  static constexpr int B_NSTATE = 22 + (T::FLUID ? 5 : 0) + (T::SCALAR ? 1 : 0);
+  static constexpr int B_NSTATE = 20 + (T::FLUID ? 5 : 0) + (T::SCALAR ? 1 : 0);
+  static constexpr int B_KDIFF = 18;  // K - K_ref
   static constexpr int PHI = T::FLUID ? 28 : 24;
   static_assert(A == A_STATE + A_NSTATE, "region A");
   static_assert(B == B_STATE + B_NSTATE + 9 + (T::FLUID ? 4 : 0), "region B");
@@ -92,17 +93,23 @@ struct Slots {
   __device__ static __forceinline__ int b_d2(int m) { return m == 0 ? 0 : (m == 1 ? 17 : (m < 5 ? 16 + m : PHI)); }
   // field of the m-th merged advection
   __device__ static __forceinline__ int b_m(int m) { return m < 6 ? 8 + m : (m < 9 ? 15 + m : PHI + 1); }
-  // field of the s-th state of each region, -1 for rho
+  // field of the s-th state of each region, -1 for rho, -2 - m for field m of G
   __device__ static constexpr int a_state(int s) {
-    constexpr int E = T::SPLIT_EARLY ? 15 : 9;
-    return s < 6 ? 1 + s : (s < 9 ? 12 + s : (s < E ? s - 1 : (s == E ? 0 : (s < E + 5 ? 23 + s - E : -1))));
+    constexpr int E = T::SPLIT_EARLY ? 21 : 15;
+    return s < 6 ? 1 + s
+                 : (s < 9 ? 12 + s : (s < 15 ? 7 - s : (s < E ? s - 7 : (s == E ? 0 : (s < E + 5 ? 23 + s - E : -1)))));
   }
-  __device__ static constexpr int b_state(int s) {  // slot 21 is K - K_ref
-    return s < 14 ? s : (s < 21 ? s + 3 : (s == 21 ? 7 : (T::FLUID ? (s < 26 ? s + 2 : (s == 26 ? -1 : 29)) : 25)));
+  __device__ static constexpr int b_state(int s) {
+    return s < 14 ? s
+                  : (s == 14 ? 17
+                             : (s < 18 ? s + 6
+                                       : (s == B_KDIFF ? 7
+                                                       : (s == 19 ? -8 : (T::FLUID ? (s < 24 ? s + 4 : (s == 24 ? -1 : 29))
+                                                                                   : 25)))));
   }
   // powers of the unit of length on a state (B^i enters without its own)
   __device__ static constexpr int state_degree(int f) {
-    return f < 0 ? 2 : (f >= 21 && f < 24 ? 0 : degree(f));
+    return f == -1 ? 2 : (f < 0 || (f >= 21 && f < 24) ? 0 : degree(f));
   }
   // powers of the unit of length that field f (and its time derivative, one more) carries
   __device__ static constexpr int degree(int f) {
@@ -418,6 +425,13 @@ struct DiffGroup {
     *m = a.len * s;
   }
 
+  // f: field of U, -1 for rho, -2 - m for field m of G
+  __device__ __forceinline__ static double state(const StageArgs& a, const DiffCtx& x, int f) {
+    if (f == -1) return ldd(reinterpret_cast<const char*>(a.prim), x.c);
+    if (f < 0) return ldd(reinterpret_cast<const char*>(a.G) + (-2 - f) * x.fb, x.c);
+    return ldd(x.U + f * x.fb, x.c);
+  }
+
   // State values into their slots (G = the group, known at compile time, so that fields and factors are):
   // every SPLIT_GROUPS-th slot of the region, all loads in flight at once.
   template <int G>
@@ -427,8 +441,7 @@ struct DiffGroup {
     double st[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-      const int f = S::a_state(G + q * SPLIT_GROUPS);
-      st[q] = f < 0 ? ldd(reinterpret_cast<const char*>(a.prim), x.c) : ldd(x.U + f * x.fb, x.c);
+      st[q] = state(a, x, S::a_state(G + q * SPLIT_GROUPS));
     }
 #pragma unroll
     for (int q = 0; q < N; ++q) {
@@ -444,15 +457,14 @@ struct DiffGroup {
     double st[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-      const int f = S::b_state(G + q * SPLIT_GROUPS);
-      st[q] = f < 0 ? ldd(reinterpret_cast<const char*>(a.prim), x.c) : ldd(x.U + f * x.fb, x.c);
+      st[q] = state(a, x, S::b_state(G + q * SPLIT_GROUPS));
     }
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       const int s = G + q * SPLIT_GROUPS, d = S::state_degree(S::b_state(s));
-      // slot 21 holds K - K_ref, which cancels: formed before any scaling
+      // K - K_ref cancels: formed before any scaling
       sB[(S::B_STATE + s) * SPLIT_PTS] =
-          s == 21 ? st[q] - kref : (d == 2 ? st[q] * a.len2 : (d == 1 ? st[q] * a.len : st[q]));
+          s == S::B_KDIFF ? st[q] - kref : (d == 2 ? st[q] * a.len2 : (d == 1 ? st[q] * a.len : st[q]));
     }
   }
 
@@ -484,9 +496,9 @@ struct DiffGroup {
       state_b<1>(a, kref, x);
     else
       state_b<2>(a, kref, x);
-    bar_sync(BAR_DIFF, SPLIT_THREADS - SPLIT_PTS);  // as in fill_a
-    // a frozen shift is not advected: beta^i (blocks 2 to 4) and B^i
-    const double* const b = sB + (S::B_STATE + 15) * SPLIT_PTS;
+    // the shift's slots are those of region A, which is filled again only after every group is here
+    // through; a frozen shift is not advected: beta^i (blocks 2 to 4) and B^i
+    const double* const b = sA + (S::A_STATE + 6) * SPLIT_PTS;
     const double* const bs = a.ap.shift_on != 0.0 ? b : nullptr;
 #pragma unroll 1
     for (int m = g; m < S::ND2B; m += SPLIT_GROUPS)
@@ -601,6 +613,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   int* const rec = tables + SPLIT_GROUPS * 80;
   constexpr int NSLOT = 24 + (T::SCALAR ? 2 : 0);
   if (threadIdx.x < 32) rec[threadIdx.x] = 0;
+  grid_wait();
   __syncthreads();
   const int t = threadIdx.x % SPLIT_PTS;
   const int tx = (one.g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = (one.g.ny + SPLIT_TY - 1) / SPLIT_TY;
@@ -693,8 +706,8 @@ cudaError_t launch_split_as(const StageArgs& one, const StageArgs* args, const B
     e = cudaFuncSetAttribute(split_stage_kernel<T, BATCH, EQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   const int blocks = (int)(ntiles < sms ? ntiles : sms);
-  split_stage_kernel<T, BATCH, EQ><<<blocks, SPLIT_THREADS, bytes, s>>>(one, args, tiles, ntiles, kref, mode);
-  return cudaGetLastError();
+  return launch_early(split_stage_kernel<T, BATCH, EQ>, dim3(blocks), SPLIT_THREADS, bytes, s, one, args, tiles, ntiles,
+                      kref, mode);
 }
 
 // eq: equal spacing (of every grid of a batch)

@@ -51,6 +51,10 @@ def slots(L, v, fluid, scalar):
             for p in range(6):
                 out[f"dd{f}_{p}"] = v[f"dd{f}_{p}"] * LEN ** 2
     out["kdiff"] = v["u7"] - KREF
+    out["ichi"] = 1.0 / v["u0"]
+    gt = np.array([[v["u1"], v["u2"], v["u3"]], [v["u2"], v["u4"], v["u5"]], [v["u3"], v["u5"], v["u6"]]])
+    for m, (a, b) in enumerate([(0, 0), (0, 1), (0, 2), (1, 1), (1, 2), (2, 2)]):
+        out[f"gu{m}"] = np.linalg.inv(gt)[a, b]
     if fluid:
         out["rho"] = v["rho"] * LEN ** 2
     return out
