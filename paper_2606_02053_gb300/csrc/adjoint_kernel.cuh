@@ -66,10 +66,8 @@ struct VjpOut {
 
 template <class T>
 __global__ void __launch_bounds__(BX* BY, COSMOS_VJP_MIN_BLOCKS) vjp_pass1_kernel(const VjpArgs a) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= a.g.nx || j >= a.g.ny) return;
+  int i, j, k;
+  if (!point_of<true>(a.g, i, j, k)) return;
   const long fs = a.g.fstride;
   const long c = ((long)k * a.g.ny + j) * a.g.pitch + i;
   const VjpIn<T> in{a, fs, c};
@@ -113,10 +111,8 @@ __device__ __forceinline__ void face_vjp(const VjpArgs& a, const Nbr& n, const F
 }
 
 static __global__ void __launch_bounds__(BX* BY) vjp_face_kernel(const VjpArgs a) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= a.g.nx || j >= a.g.ny) return;
+  int i, j, k;
+  if (!point_of<true>(a.g, i, j, k)) return;
   const Nbr n = make_nbr(a.g, i, j, k);
   const Fp64Regs kr = fp64_regs();
   face_vjp<0>(a, n, kr);
@@ -146,10 +142,8 @@ __device__ __forceinline__ void gather_face_cot(const VjpArgs& a, const Nbr& n, 
 
 template <class T>
 __global__ void __launch_bounds__(BX* BY) vjp_cell_kernel(const VjpArgs a) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= a.g.nx || j >= a.g.ny) return;
+  int i, j, k;
+  if (!point_of<true>(a.g, i, j, k)) return;
   const Nbr n = make_nbr(a.g, i, j, k);
   const long fs = a.g.fstride;
   double qb[4] = {ldg(a.CB + (long)(T::NIN - 1) * fs, n.c), 0.0, 0.0, 0.0};  // d/d rho from the algebra
@@ -248,10 +242,8 @@ template <class T>
 __global__ void __launch_bounds__(BX* BY) vjp_fold_kernel(const VjpArgs a) {
   __shared__ double cf[12];
   const RevCoef c = rev_coef(a.c, cf);
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= a.g.nx || j >= a.g.ny) return;
+  int i, j, k;
+  if (!point_of<true>(a.g, i, j, k)) return;
   const Nbr n = make_nbr(a.g, i, j, k);
   const long fs = a.g.fstride;
 #pragma unroll 1
@@ -269,10 +261,8 @@ template <class T>
 __global__ void __launch_bounds__(BX* BY, 3) vjp_pass2_kernel(const VjpArgs a) {
   __shared__ double cf[12];
   const RevCoef c = rev_coef(a.c, cf);
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= a.g.nx || j >= a.g.ny) return;
+  int i, j, k;
+  if (!point_of<true>(a.g, i, j, k)) return;
   const Nbr n = make_nbr(a.g, i, j, k);
   const long fs = a.g.fstride;
   const bool ko_equal = a.c.ko[0] == a.c.ko[1] && a.c.ko[1] == a.c.ko[2];
@@ -324,7 +314,8 @@ struct T_vac_adj {
     }                                                                                                           \
   };                                                                                                            \
   cudaError_t launch_vjp_##NAME(const VjpArgs& a, cudaStream_t s) {                                             \
-    const dim3 grid = point_grid(a.g), block(BX, BY);                                                          \
+    const unsigned grid = flat_grid(a.g);                                                                       \
+    const int block = BX * BY;                                                                                  \
     vjp_pass1_kernel<A_##NAME><<<grid, block, 0, s>>>(a);                                                       \
     cudaError_t e = cudaGetLastError();                                                                         \
     if (e != cudaSuccess) return e;                                                                             \

@@ -22,12 +22,11 @@ __device__ __forceinline__ void prim_point(const DevGrid& g, const double* __res
   for (int m = 0; m < 4; ++m) prim[m * fs + c] = out[m];
 }
 
+template <bool FLAT>
 __global__ void __launch_bounds__(BX* BY) prim_kernel(const DevGrid g, const double* __restrict__ U,
                                                       double* __restrict__ prim, const FluidParams fp) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= g.nx || j >= g.ny) return;
+  int i, j, k;
+  if (!point_of<FLAT>(g, i, j, k)) return;
   prim_point(g, U, prim, fp, fp64_regs(), i, j, k);
 }
 
@@ -68,13 +67,12 @@ __device__ __forceinline__ void flux_point(const DevGrid& g, const double* __res
   face<2>(U, prim, n, g.fstride, fp, kr, H);
 }
 
+template <bool FLAT>
 __global__ void __launch_bounds__(BX* BY) flux_kernel(const DevGrid g, const double* __restrict__ U,
                                                       const double* __restrict__ prim, double* __restrict__ H,
                                                       const FluidParams fp) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= g.nx || j >= g.ny) return;
+  int i, j, k;
+  if (!point_of<FLAT>(g, i, j, k)) return;
   flux_point(g, U, prim, H, fp, fp64_regs(), i, j, k);
 }
 
@@ -112,7 +110,10 @@ static FluidParams fluid_params(double w) {
 }
 
 cudaError_t launch_fluid_prim(const DevGrid& g, const double* U, double* prim, double w, cudaStream_t s) {
-  prim_kernel<<<point_grid(g), dim3(BX, BY), 0, s>>>(g, U, prim, fluid_params(w));
+  if (tiles_exact(g))
+    prim_kernel<false><<<point_grid(g), dim3(BX, BY), 0, s>>>(g, U, prim, fluid_params(w));
+  else
+    prim_kernel<true><<<flat_grid(g), BX * BY, 0, s>>>(g, U, prim, fluid_params(w));
   return cudaGetLastError();
 }
 
@@ -127,7 +128,10 @@ cudaError_t launch_batch_fluid(const StageArgs* args, const BatchTile* tiles, lo
 
 cudaError_t launch_fluid_flux(const DevGrid& g, const double* U, const double* prim, double* flux, double w,
                               int /*nf_offset_fluid*/, cudaStream_t s) {
-  flux_kernel<<<point_grid(g), dim3(BX, BY), 0, s>>>(g, U, prim, flux, fluid_params(w));
+  if (tiles_exact(g))
+    flux_kernel<false><<<point_grid(g), dim3(BX, BY), 0, s>>>(g, U, prim, flux, fluid_params(w));
+  else
+    flux_kernel<true><<<flat_grid(g), BX * BY, 0, s>>>(g, U, prim, flux, fluid_params(w));
   return cudaGetLastError();
 }
 
