@@ -235,19 +235,19 @@ cudaError_t launch_fluid_flux(const DevGrid& g, const double* U, const double* p
 
 inline dim3 point_grid(const DevGrid& g) { return dim3((g.nx + BX - 1) / BX, (g.ny + BY - 1) / BY, g.nz); }
 
-// A point per thread of the reverse mode's and the fluid's FP64 kernels, in runs of BX BY points of the whole
+// A point per thread of the reverse mode's and the fluid's FP64 kernels, in runs (one block each) of the whole
 // grid, so that every lane has one: BX x BY tiles of a plane of 45 x 33 points leave 42% of the lanes without
 // (a VJP of 45 x 33 x 28: 698 -> 473 us), of 97 x 80 points 24% (an RK4 step with fluid and scalar of
 // 97 x 80 x 66: 10.47 -> 9.68 ms).  On a plane that the tiles cover exactly both are the same work; there the fluid
 // kernels keep the tiles, which take no division (128^3: 0.3% of a step).
 inline bool tiles_exact(const DevGrid& g) { return g.nx % BX == 0 && g.ny % BY == 0; }
-inline unsigned flat_grid(const DevGrid& g) {
-  return (unsigned)(((long)g.nx * g.ny * g.nz + BX * BY - 1) / (BX * BY));
+inline unsigned flat_grid(const DevGrid& g, int threads) {
+  return (unsigned)(((long)g.nx * g.ny * g.nz + threads - 1) / threads);
 }
 template <bool FLAT>
 __device__ __forceinline__ bool point_of(const DevGrid& g, int& i, int& j, int& k) {
   if (FLAT) {
-    const unsigned p = blockIdx.x * (BX * BY) + threadIdx.x;  // grids have less than 2^31 points
+    const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;  // grids have less than 2^31 points
     const unsigned row = p / (unsigned)g.nx;
     i = (int)(p - row * (unsigned)g.nx);
     k = (int)(row / (unsigned)g.ny);

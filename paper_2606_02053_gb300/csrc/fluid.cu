@@ -113,7 +113,7 @@ cudaError_t launch_fluid_prim(const DevGrid& g, const double* U, double* prim, d
   if (tiles_exact(g))
     prim_kernel<false><<<point_grid(g), dim3(BX, BY), 0, s>>>(g, U, prim, fluid_params(w));
   else
-    prim_kernel<true><<<flat_grid(g), BX * BY, 0, s>>>(g, U, prim, fluid_params(w));
+    prim_kernel<true><<<flat_grid(g, BX * BY), BX * BY, 0, s>>>(g, U, prim, fluid_params(w));
   return cudaGetLastError();
 }
 
@@ -131,7 +131,7 @@ cudaError_t launch_fluid_flux(const DevGrid& g, const double* U, const double* p
   if (tiles_exact(g))
     flux_kernel<false><<<point_grid(g), dim3(BX, BY), 0, s>>>(g, U, prim, flux, fluid_params(w));
   else
-    flux_kernel<true><<<flat_grid(g), BX * BY, 0, s>>>(g, U, prim, flux, fluid_params(w));
+    flux_kernel<true><<<flat_grid(g, BX * BY), BX * BY, 0, s>>>(g, U, prim, flux, fluid_params(w));
   return cudaGetLastError();
 }
 
