@@ -68,7 +68,7 @@ def render() -> dict:
         body.append(f"constexpr bool SPLIT_EARLY = {str(S['early']).lower()};  // At among the states of region A")
         body.append(_table_fn("out_slot", S["out"]))
         body.append(emit_split(gs, "rhs_split", S["a"], S["b"], outs, gs.cut, "AlgebraParams"))
-        body.append(emit_fused(g, "constraints", L["names"], g.constraints, "AlgebraParams", accessors=True))
+        body.append(emit_fused(g, "constraints", L["names"], g.constraints, "AlgebraParams"))
         if name in ADJOINT_VARIANTS:
             # reverse mode: in[0 .. NIN) as for rhs, in[NIN + f] = cotangent of out[f];
             # out[k] = sum_f cot_f d out_f / d in[k]

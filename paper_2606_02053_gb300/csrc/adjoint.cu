@@ -32,8 +32,8 @@ static cudaError_t launch_stage_for(const cosmos_params* p, const StageArgs& a, 
 }
 
 static cudaError_t launch_deriv_for(const cosmos_params* p, const StageArgs& a, cudaStream_t s) {
-  if (p->fluid) return p->scalar ? launch_deriv_fluid_scalar(a, a.g.nz, s) : launch_deriv_fluid(a, a.g.nz, s);
-  return p->scalar ? launch_deriv_scalar(a, a.g.nz, s) : launch_deriv_vac(a, a.g.nz, s);
+  if (p->fluid) return p->scalar ? launch_deriv_fluid_scalar(a, s) : launch_deriv_fluid(a, s);
+  return p->scalar ? launch_deriv_scalar(a, s) : launch_deriv_vac(a, s);
 }
 
 static cudaError_t launch_vjp_for(const cosmos_params* p, const VjpArgs& a, cudaStream_t s) {
@@ -139,8 +139,6 @@ static cudaError_t vjp_once(const cosmos_grid* g, const cosmos_params* p, const 
   d.c = a.c;
   d.U = U;
   d.D = ws + L.Dfw;
-  d.dfs = d.g.fstride;
-  d.need = ~0u;
   a.D = d.D;
   {
     cudaError_t e = limbs_of(p, d.g, U, ws, L, d, nullptr, s);

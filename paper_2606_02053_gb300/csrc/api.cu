@@ -119,12 +119,6 @@ int validate(const cosmos_grid* g, const cosmos_params* p) {
   return COSMOS_OK;
 }
 
-// The constraints' differences are formed a chunk of planes at a time, about
-// CON_CHUNK points (2.4 GB of differences), from a limb copy of the state.  Beyond
-// CON_DIFF_MAX points that copy, as large as the state, is not asked for: such a
-// grid takes constraint_kernel, which needs no more than its partial sums.
-static constexpr size_t CON_CHUNK = (size_t)1 << 21, CON_DIFF_MAX = (size_t)1 << 27;
-
 WsLayout ws_layout(const cosmos_grid* g, const cosmos_params* p, int op) {
   const DevGrid d = make_devgrid(g);
   const size_t fs = (size_t)d.fstride;
@@ -158,14 +152,6 @@ WsLayout ws_layout(const cosmos_grid* g, const cosmos_params* p, int op) {
   } else if (op == COSMOS_OP_CONSTRAINTS || op == COSMOS_OP_INIT) {
     if (fluid) L.prim = take(4 * fs);
     if (op == COSMOS_OP_INIT) L.hm = take(4 * fs);
-    if (op == COSMOS_OP_CONSTRAINTS && fs <= CON_DIFF_MAX) {
-      const int nslot = 24 + 2 * p->scalar;
-      const size_t plane = fs / d.nz;
-      L.chunk = (int)std::min<size_t>(d.nz, std::max<size_t>(CON_CHUNK / plane, CON_PLANES));
-      L.limbs = take((size_t)nslot * fs);
-      L.expo = take(((size_t)nslot + 1) / 2);
-      L.D = take((size_t)nder(p->scalar) * plane * L.chunk);
-    }
     L.partial = take(8 * n_blocks(d));
     L.final_ = take(8);
   } else if (op == COSMOS_OP_SCAN) {
@@ -340,22 +326,6 @@ static StageLauncher stage_launcher(const cosmos_params* p) {
   if (p->fluid) return launch_stage_fluid;
   if (p->scalar) return launch_stage_scalar;
   return launch_stage_vac;
-}
-
-typedef cudaError_t (*DerivLauncher)(const StageArgs&, int, cudaStream_t);
-
-static DerivLauncher deriv_launcher(const cosmos_params* p) {
-  if (p->fluid && p->scalar) return launch_deriv_fluid_scalar;
-  if (p->fluid) return launch_deriv_fluid;
-  if (p->scalar) return launch_deriv_scalar;
-  return launch_deriv_vac;
-}
-
-static ConstraintLauncher constraint_diff_launcher(const cosmos_params* p) {
-  if (p->fluid && p->scalar) return launch_constraints_diff_fluid_scalar;
-  if (p->fluid) return launch_constraints_diff_fluid;
-  if (p->scalar) return launch_constraints_diff_scalar;
-  return launch_constraints_diff_vac;
 }
 
 static ConstraintLauncher constraint_launcher(const cosmos_params* p) {
@@ -876,37 +846,8 @@ int cosmos_constraints(const cosmos_grid* g, const cosmos_params* p, const doubl
     CK(launch_fluid_prim(c.g, state, w + L.prim, p->w, s));
     c.prim = w + L.prim;
   }
-  long blocks = 0;
-  if (L.chunk) {
-    const int nslot = 24 + 2 * p->scalar;
-    const long plane = (long)g->ny * g->pitch;
-    StageArgs d;
-    memset(&d, 0, sizeof(d));
-    d.g = c.g;
-    d.c = c.c;
-    d.L = (const long long*)(w + L.limbs);
-    d.E = (const int*)(w + L.expo);
-    d.dfs = plane * L.chunk;
-    // all fields but the lapse, the shift and B^i (slots 17 .. 23) and Pi (25)
-    d.need = ~(0x7Fu << 17 | 1u << 25);
-    CK(launch_limbs(d.g, state, p->fluid, 0, nslot, (int*)(w + L.expo), (long long*)(w + L.limbs), nullptr, s));
-    for (int k0 = 0; k0 < g->nz; k0 += L.chunk) {
-      d.k_lo = c.k_lo = k0;
-      c.k_cnt = std::min(L.chunk, g->nz - k0);
-      d.D = w + L.D - (ptrdiff_t)(plane * k0);  // addressed by the points' offsets in the grid
-      c.D = d.D;
-      c.dfs = d.dfs;
-      c.partial = w + L.partial + 8 * blocks;
-      CK(deriv_launcher(p)(d, c.k_cnt, s));
-      CK(constraint_diff_launcher(p)(c, s));
-      const dim3 b = constraint_grid(c.g, c.k_cnt);
-      blocks += (long)b.x * b.y * b.z;
-    }
-  } else {
-    CK(constraint_launcher(p)(c, s));
-    blocks = n_blocks(c.g);
-  }
-  reduce_partials<<<1, 256, 0, s>>>(w + L.partial, blocks, w + L.final_);
+  CK(constraint_launcher(p)(c, s));
+  reduce_partials<<<1, 256, 0, s>>>(w + L.partial, n_blocks(c.g), w + L.final_);
   CK(cudaGetLastError());
   double r[8];
   CK(cudaMemcpyAsync(r, w + L.final_, sizeof(r), cudaMemcpyDeviceToHost, s));

@@ -114,9 +114,7 @@ struct StageArgs {
   double* acc;                     // accumulator
   const double* __restrict__ prim; // fluid primitives [4][pts] (fluid only)
   const double* __restrict__ flux; // fluid face fluxes [3][4][pts] (fluid only)
-  double* D;                       // finite differences of U (ideriv_kernel only): slot s of point c at D[s dfs + c]
-  long dfs;                        // doubles between the slots of D
-  unsigned need;                   // bit s: the differences of limb slot s are wanted (ideriv_kernel only)
+  double* D;                       // finite differences of U for the reverse mode (ideriv_kernel only)
   double cdt;                      // dt * c_{s+1}, or dt/6 in MODE_S4
   double len, len2;                // l = 12 h_x, l^2
   double inv_len[4];               // 1/l, 1/l^2, 1/l^3 (per degree of the field, stage_split.cuh), 1
@@ -154,16 +152,7 @@ struct ConstraintArgs {
   const double* __restrict__ prim;
   double* hm;        // [4][pts] or null
   double* partial;   // [nblocks][8]: sum of squares (4) and max abs (4)
-  // constraint_diff_kernel: the differences of planes k_lo .. k_lo + k_cnt - 1 (slot s of point c at D[s dfs + c])
-  const double* __restrict__ D;
-  long dfs;
-  int k_lo, k_cnt;
 };
-constexpr int CON_PLANES = 4;  // planes per thread of constraint_diff_kernel
-// Blocks (partials) of constraint_diff_kernel for k_cnt planes.
-inline dim3 constraint_grid(const DevGrid& g, int k_cnt) {
-  return dim3((g.nx + BX - 1) / BX, (g.ny + BY - 1) / BY, (k_cnt + CON_PLANES - 1) / CON_PLANES);
-}
 
 #ifndef COSMOS_IDERIV_MIN_BLOCKS
 #define COSMOS_IDERIV_MIN_BLOCKS 4  // integer derivative pass: resident blocks (of BX x DBY threads) per SM
@@ -175,11 +164,10 @@ cudaError_t launch_stage_vac(const StageArgs& a, int mode, int k_cnt, cudaStream
 cudaError_t launch_stage_fluid(const StageArgs& a, int mode, int k_cnt, cudaStream_t s);
 cudaError_t launch_stage_scalar(const StageArgs& a, int mode, int k_cnt, cudaStream_t s);
 cudaError_t launch_stage_fluid_scalar(const StageArgs& a, int mode, int k_cnt, cudaStream_t s);
-// finite differences of k_cnt planes from a.k_lo into a.D
-cudaError_t launch_deriv_vac(const StageArgs& a, int k_cnt, cudaStream_t s);
-cudaError_t launch_deriv_fluid(const StageArgs& a, int k_cnt, cudaStream_t s);
-cudaError_t launch_deriv_scalar(const StageArgs& a, int k_cnt, cudaStream_t s);
-cudaError_t launch_deriv_fluid_scalar(const StageArgs& a, int k_cnt, cudaStream_t s);
+cudaError_t launch_deriv_vac(const StageArgs& a, cudaStream_t s);  // finite differences into a.D
+cudaError_t launch_deriv_fluid(const StageArgs& a, cudaStream_t s);
+cudaError_t launch_deriv_scalar(const StageArgs& a, cudaStream_t s);
+cudaError_t launch_deriv_fluid_scalar(const StageArgs& a, cudaStream_t s);
 // batched stage over the tile list (SPLIT_TX x SPLIT_TY of one plane), K_ref per instance;
 // eq: every grid has equal spacing
 typedef cudaError_t (*BatchStageLauncher)(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
@@ -190,11 +178,6 @@ cudaError_t launch_batch_stage_fluid_scalar(const StageArgs*, const BatchTile*, 
                                             cudaStream_t);
 cudaError_t launch_batch_fluid(const StageArgs* args, const BatchTile* tiles, long ntiles, int mapping, double w,
                                dim3 grid, dim3 block, cudaStream_t s);
-// constraints from differences in memory (constraint_diff_kernel)
-cudaError_t launch_constraints_diff_vac(const ConstraintArgs& a, cudaStream_t s);
-cudaError_t launch_constraints_diff_fluid(const ConstraintArgs& a, cudaStream_t s);
-cudaError_t launch_constraints_diff_scalar(const ConstraintArgs& a, cudaStream_t s);
-cudaError_t launch_constraints_diff_fluid_scalar(const ConstraintArgs& a, cudaStream_t s);
 cudaError_t launch_constraints_vac(const ConstraintArgs& a, cudaStream_t s);
 cudaError_t launch_constraints_fluid(const ConstraintArgs& a, cudaStream_t s);
 cudaError_t launch_constraints_scalar(const ConstraintArgs& a, cudaStream_t s);
@@ -260,9 +243,7 @@ __device__ __forceinline__ bool point_of(const DevGrid& g, int& i, int& j, int& 
   return i < g.nx && j < g.ny;
 }
 // reverse mode's derivative pass: one BX x DBY tile of one z-plane per block
-inline dim3 ideriv_grid(const DevGrid& g, int k_cnt) {
-  return dim3((g.nx + BX - 1) / BX, (g.ny + DBY - 1) / DBY, k_cnt);
-}
+inline dim3 ideriv_grid(const DevGrid& g) { return dim3((g.nx + BX - 1) / BX, (g.ny + DBY - 1) / DBY, g.nz); }
 // Every index the integer derivative pass forms for a tile lies in [-n, 2n)
 // along each axis, so one compare and select wraps it (stage_int.cuh,
 // wrap_near): x in [i0 - 3, i0 + BX + 2] with i0 <= nx - 1, y in

@@ -257,9 +257,9 @@ __device__ __forceinline__ Limb id1(const long long* __restrict__ L, const NbrI&
 // First derivatives of a field that has no second ones.
 template <class T, bool ODD>
 __device__ __forceinline__ void ideriv_d1_point(const StageArgs& a, int m, const NbrI& n, int e) {
-  const long fs = a.dfs;
+  const long fs = a.g.fstride;
   const int s = ko_slot<T>(T::d1_field(m));
-  const long long* Lf = a.L + (long)s * a.g.fstride;
+  const long long* Lf = a.L + (long)s * fs;
   double* __restrict__ D = a.D + (long)(3 * m) * fs + n.c;
   D[0] = limb_value<ODD>(id1<0>(Lf, n), e) * a.c.d1b[0];
   D[fs] = limb_value<ODD>(id1<1>(Lf, n), e) * a.c.d1b[1];
@@ -272,12 +272,12 @@ template <class T, bool ODD>
 __device__ __forceinline__ void ideriv_d2_point(const StageArgs& a, int m2, const NbrI& n, int e, int tx, int ty,
                                                 const int4* __restrict__ sDy, const int4* __restrict__ sDz) {
   constexpr int TXH = BX + 4;
-  const long fs = a.dfs;
+  const long fs = a.g.fstride;
   const Coef& c = a.c;
   double* __restrict__ D = a.D;
   const int f = T::d2_field(m2);
   const int s = ko_slot<T>(f);
-  const long long* Lf = a.L + (long)s * a.g.fstride;
+  const long long* Lf = a.L + (long)s * fs;
   const int m1 = T::d1_slot(f);
   const long b = (long)(3 * T::ND1 + 6 * m2) * fs + n.c;
   const Limb f30 = l_mul(ldl(Lf, n.c), 30);
@@ -315,7 +315,7 @@ __device__ __forceinline__ void ideriv_tile(const StageArgs& a, int i0, int j0, 
   const long fs = a.g.fstride;
 #pragma unroll 1
   for (int m = 0; m < T::ND1; ++m) {
-    if (T::d2_slot(T::d1_field(m)) >= 0 || !(a.need >> ko_slot<T>(T::d1_field(m)) & 1u)) continue;
+    if (T::d2_slot(T::d1_field(m)) >= 0) continue;
     const int e = max(a.E[ko_slot<T>(T::d1_field(m))], 1);
     if (!valid) continue;
     if (limb_odd(e))
@@ -326,7 +326,6 @@ __device__ __forceinline__ void ideriv_tile(const StageArgs& a, int i0, int j0, 
 #pragma unroll 1
   for (int m2 = 0; m2 < T::ND2; ++m2) {
     const int f = T::d2_field(m2);
-    if (!(a.need >> ko_slot<T>(f) & 1u)) continue;  // uniform across the block
     stage_dydz_int<NEAR>(a.g, a.L + (long)ko_slot<T>(f) * fs, i0, j0, k, tid, sDy, sDz);
     __syncthreads();
     if (valid) {
@@ -344,7 +343,7 @@ __device__ __forceinline__ void ideriv_tile(const StageArgs& a, int i0, int j0, 
 template <class T, bool NEAR>
 __global__ void __launch_bounds__(BX* DBY, COSMOS_IDERIV_MIN_BLOCKS) ideriv_kernel(const StageArgs a) {
   __shared__ int4 sDy[(BX + 4) * DBY], sDz[(BX + 4) * (DBY + 4)];
-  ideriv_tile<T, NEAR>(a, blockIdx.x * BX, blockIdx.y * DBY, blockIdx.z + a.k_lo, sDy, sDz);
+  ideriv_tile<T, NEAR>(a, blockIdx.x * BX, blockIdx.y * DBY, blockIdx.z, sDy, sDz);
 }
 
 }  // namespace cosmos

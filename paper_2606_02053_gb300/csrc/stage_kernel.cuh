@@ -163,8 +163,35 @@ __device__ __forceinline__ bool batch_point(const BatchTile& t, const DevGrid& g
   return true;
 }
 
-// Sum of squares (r[0 .. 3]) and largest modulus (r[4 .. 7]) of the block into its partial b.
-__device__ __forceinline__ void block_norms(double (&r)[8], double* __restrict__ partial, long b) {
+// Constraints H, M^i per point plus per-block partial norms.  The differences are FP64 differences of
+// neighbouring values (770 of the kernel's 1335 FP64 instructions per point; 128^3 with the fluid 5.6 ms),
+// so that small values of a field keep their relative accuracy and a NaN stays in its stencil neighbourhood:
+// the integer differences of stage_int.cuh (3.6 ms, 24 doubles a point of workspace) are exact relative to a
+// field's largest value over the grid only, and one NaN spoils them everywhere.
+template <class T>
+__global__ void __launch_bounds__(BX* BY, 2) constraint_kernel(const ConstraintArgs a) {
+  const int i = blockIdx.x * BX + threadIdx.x;
+  const int j = blockIdx.y * BY + threadIdx.y;
+  const int k = blockIdx.z;
+  const bool valid = (i < a.g.nx) && (j < a.g.ny);
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  if (valid) {
+    const Nbr n = make_nbr(a.g, i, j, k);
+    const long fs = a.g.fstride;
+    double in[T::NIN];
+    gather<T>(a.U, a.prim, n, a.c, fs, in);
+    T::constraints(in, v, a.ap, fp64_regs());
+    if (a.hm) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) a.hm[(long)m * fs + n.c] = v[m];
+    }
+  }
+  double r[8];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    r[m] = v[m] * v[m];
+    r[4 + m] = fabs(v[m]);
+  }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
 #pragma unroll
@@ -190,92 +217,10 @@ __device__ __forceinline__ void block_norms(double (&r)[8], double* __restrict__
         s[4 + m] = fmax(s[4 + m], red[w][4 + m]);
       }
     }
+    const long b = ((long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) partial[b * 8 + m] = s[m];
+    for (int m = 0; m < 8; ++m) a.partial[b * 8 + m] = s[m];
   }
-}
-
-__device__ __forceinline__ long block_index() {
-  return ((long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-}
-
-// Constraints H, M^i per point plus per-block partial norms, with the finite
-// differences formed here in FP64: for callers without a workspace for them
-// (initial data, cosmos_constraints_noalloc, grids beyond 2^27 points).
-template <class T>
-__global__ void __launch_bounds__(BX* BY, 2) constraint_kernel(const ConstraintArgs a) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int k = blockIdx.z;
-  const bool valid = (i < a.g.nx) && (j < a.g.ny);
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-  if (valid) {
-    const Nbr n = make_nbr(a.g, i, j, k);
-    const long fs = a.g.fstride;
-    double in[T::NIN];
-    gather<T>(a.U, a.prim, n, a.c, fs, in);
-    T::constraints(in, v, a.ap, fp64_regs());
-    if (a.hm) {
-#pragma unroll
-      for (int m = 0; m < 4; ++m) a.hm[(long)m * fs + n.c] = v[m];
-    }
-  }
-  double r[8];
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    r[m] = v[m] * v[m];
-    r[4 + m] = fabs(v[m]);
-  }
-  block_norms(r, a.partial, block_index());
-}
-
-// Inputs of the constraints at one point, read from global memory where the
-// generated code uses them (state values, then the differences, then the fluid density).
-template <class T>
-struct DiffIn {
-  const double* __restrict__ U;
-  const double* __restrict__ D;
-  const double* __restrict__ prim;
-  long fs, dfs, c;
-  __device__ __forceinline__ double operator[](int k) const {
-    constexpr int NDER0 = 3 * T::ND1 + 6 * T::ND2;
-    if (k < T::NF) return ldg(U + (long)k * fs, c);
-    if (k < T::NF + NDER0) return ldg(D + (long)(k - T::NF) * dfs, c);
-    return ldg(prim, c);
-  }
-};
-
-// The same with the differences in memory (ideriv_kernel, a chunk of planes at a
-// time).  FP64-bound: the differences in integer arithmetic take 770 of the 1335
-// FP64 instructions of constraint_kernel off the pipe, and CON_PLANES planes per
-// thread the norms' 40 per point (shuffled maxima run on it) to a quarter.
-// 128^3 with the fluid: 5.3 ms -> 2.2 (95% of its FP64 time), 0.7 for the differences and 0.2 for the copy.
-template <class T>
-__global__ void __launch_bounds__(BX* BY, 3) constraint_diff_kernel(const ConstraintArgs a) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const bool valid = (i < a.g.nx) && (j < a.g.ny);
-  const Fp64Regs kr = fp64_regs();
-  const long fs = a.g.fstride;
-  double r[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  const int k0 = a.k_lo + blockIdx.z * CON_PLANES, k1 = min(k0 + CON_PLANES, a.k_lo + a.k_cnt);
-  if (valid) {
-#pragma unroll 1
-    for (int k = k0; k < k1; ++k) {
-      const long c = ((long)k * a.g.ny + j) * a.g.pitch + i;
-      double v[4];
-      T::constraints(DiffIn<T>{a.U, a.D, a.prim, fs, a.dfs, c}, v, a.ap, kr);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        if (a.hm) a.hm[(long)m * fs + c] = v[m];
-        r[m] = fma(v[m], v[m], r[m]);
-        // the larger modulus on the bits, NaN left out as fmax does
-        const long long b = __double_as_longlong(v[m]) & 0x7FFFFFFFFFFFFFFFll;
-        if (b <= 0x7FF0000000000000ll && b > __double_as_longlong(r[4 + m])) r[4 + m] = __longlong_as_double(b);
-      }
-    }
-  }
-  block_norms(r, a.partial, block_index());
 }
 
 #define COSMOS_DEFINE_VARIANT(NAME, IS_FLUID, IS_SCALAR)                                                          \
@@ -295,9 +240,8 @@ __global__ void __launch_bounds__(BX* BY, 3) constraint_diff_kernel(const Constr
                                                      const AlgebraParams& p, const Fp64Regs& k) {                   \
       alg_##NAME::rhs_split(ina, inb, out, next, p, k);                                                           \
     }                                                                                                               \
-    template <class In, class Out>                                                                                  \
-    __device__ static __forceinline__ void constraints(const In& in, Out&& out, const AlgebraParams& p,             \
-                                                       const Fp64Regs& k) {                                         \
+    __device__ static __forceinline__ void constraints(const double* in, double* out, const AlgebraParams& p,       \
+                                                       const Fp64Regs& k) {                                       \
       alg_##NAME::constraints(in, out, p, k);                                                                     \
     }                                                                                                           \
   };                                                                                                            \
@@ -306,12 +250,12 @@ __global__ void __launch_bounds__(BX* BY, 3) constraint_diff_kernel(const Constr
     const long tiles = (long)((a.g.nx + SPLIT_TX - 1) / SPLIT_TX) * ((a.g.ny + SPLIT_TY - 1) / SPLIT_TY) * k_cnt;   \
     return launch_split<T_##NAME, false>(a, nullptr, nullptr, tiles, nullptr, mode, a.eq, s);                             \
   }                                                                                                                 \
-  cudaError_t launch_deriv_##NAME(const StageArgs& a, int k_cnt, cudaStream_t s) {                                             \
+  cudaError_t launch_deriv_##NAME(const StageArgs& a, cudaStream_t s) {                                             \
     if (!a.L) return cudaErrorInvalidValue;                                                                         \
     if (near_indices(a.g))                                                                                          \
-      ideriv_kernel<T_##NAME, true><<<ideriv_grid(a.g, k_cnt), dim3(BX, DBY), 0, s>>>(a);                                  \
+      ideriv_kernel<T_##NAME, true><<<ideriv_grid(a.g), dim3(BX, DBY), 0, s>>>(a);                                  \
     else                                                                                                            \
-      ideriv_kernel<T_##NAME, false><<<ideriv_grid(a.g, k_cnt), dim3(BX, DBY), 0, s>>>(a);                                 \
+      ideriv_kernel<T_##NAME, false><<<ideriv_grid(a.g), dim3(BX, DBY), 0, s>>>(a);                                 \
     return cudaGetLastError();                                                                                      \
   }                                                                                                                 \
   cudaError_t launch_batch_stage_##NAME(const StageArgs* args, const BatchTile* tiles, long ntiles,                 \
@@ -319,10 +263,6 @@ __global__ void __launch_bounds__(BX* BY, 3) constraint_diff_kernel(const Constr
     StageArgs none;                                                                                                 \
     memset(&none, 0, sizeof(none));                                                                                 \
     return launch_split<T_##NAME, true>(none, args, tiles, ntiles, kref, mode, eq, s);                                  \
-  }                                                                                                                 \
-  cudaError_t launch_constraints_diff_##NAME(const ConstraintArgs& a, cudaStream_t s) {                             \
-    constraint_diff_kernel<T_##NAME><<<constraint_grid(a.g, a.k_cnt), dim3(BX, BY), 0, s>>>(a);                     \
-    return cudaGetLastError();                                                                                      \
   }                                                                                                                 \
   cudaError_t launch_constraints_##NAME(const ConstraintArgs& a, cudaStream_t s) {                              \
     constraint_kernel<T_##NAME><<<point_grid(a.g), dim3(BX, BY), 0, s>>>(a);                                    \
