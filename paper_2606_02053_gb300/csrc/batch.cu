@@ -105,10 +105,9 @@ struct cosmos_batch_s {
   int sms = 0;
   char* ws = nullptr;
   BatchLayout L;
-  long ntiles = 0, nstiles = 0;
+  long ntiles = 0, nstiles = 0, nstiles_eq = 0;  // nstiles_eq: those of the grids with equal spacing, the first
   StageArgs* d_args = nullptr;  // [4][n]
   BatchTile* d_tiles = nullptr;
-  bool eq = true;                 // every grid has equal spacing
   BatchTile* d_stiles = nullptr;  // stage-kernel tiles (SPLIT_TX x SPLIT_TY of one z-plane; c = the plane)
   double* d_kref = nullptr;     // [max_steps][4][n]
   cudaGraphExec_t gexec = nullptr;
@@ -229,7 +228,6 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
       a.acc = acc;
       a.cdt = cdt[s];
       set_units(&a, p->ko_sigma, 2.0);
-      b->eq = b->eq && a.eq;
       a.L = (const long long*)(wsd + L.limbs[i]);
       a.G = wsd + L.G[i];
       a.E = (const int*)(b->ws + L.expo) + (size_t)i * nslot_of(p);
@@ -261,13 +259,19 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
   {
     // Tiles instance by instance, plane by plane: the blocks of the persistent
     // stage kernel then work on neighbouring planes of one grid, whose z-stencils
-    // share their planes in L2.
+    // share their planes in L2.  The grids with equal spacing come first: the stage
+    // kernel's forms for equal and unequal spacing round the dissipation differently,
+    // and each instance takes that of cosmos_rk4_step on its own grid.
     std::vector<BatchTile> st;
-    for (int i = 0; i < n; ++i) {
-      const cosmos_grid& g = grids[i];
-      const int tx = (g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = (g.ny + SPLIT_TY - 1) / SPLIT_TY;
-      for (long w = 0; w < stage_tiles(g); ++w)
-        st.push_back(BatchTile{i, (int)(w % tx), (int)((w / tx) % ty), (int)(w / ((long)tx * ty))});
+    for (int eq = 1; eq >= 0; --eq) {
+      for (int i = 0; i < n; ++i) {
+        const cosmos_grid& g = grids[i];
+        if (args[i].eq != eq) continue;
+        const int tx = (g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = (g.ny + SPLIT_TY - 1) / SPLIT_TY;
+        for (long w = 0; w < stage_tiles(g); ++w)
+          st.push_back(BatchTile{i, (int)(w % tx), (int)((w / tx) % ty), (int)(w / ((long)tx * ty))});
+      }
+      if (eq) b->nstiles_eq = (long)st.size();
     }
     b->nstiles = (long)st.size();
     if (cudaMemcpy(b->d_stiles, st.data(), sizeof(BatchTile) * st.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -291,14 +295,17 @@ int cosmos_batch_set_tuning(cosmos_batch b, const cosmos_batch_tuning* tuning) {
   return upload_tiles(b);
 }
 
+// The stage kernel over every instance: the tiles of the grids with equal spacing, then the others.
+static cudaError_t launch_stage(cosmos_batch b, const StageArgs* args, const double* kref, int mode, cudaStream_t s) {
+  const BatchStageLauncher launch =
+      b->p.fluid ? (b->p.scalar ? launch_batch_stage_fluid_scalar : launch_batch_stage_fluid)
+                 : (b->p.scalar ? launch_batch_stage_scalar : launch_batch_stage_vac);
+  const cudaError_t e = launch(args, b->d_stiles, b->nstiles_eq, kref, mode, true, s);
+  if (e != cudaSuccess) return e;
+  return launch(args, b->d_stiles + b->nstiles_eq, b->nstiles - b->nstiles_eq, kref, mode, false, s);
+}
+
 static int batch_launch_steps(cosmos_batch b, int first_step, int steps, cudaStream_t s) {
-  BatchStageLauncher launch = launch_batch_stage_vac;
-  if (b->p.fluid && b->p.scalar)
-    launch = launch_batch_stage_fluid_scalar;
-  else if (b->p.fluid)
-    launch = launch_batch_stage_fluid;
-  else if (b->p.scalar)
-    launch = launch_batch_stage_scalar;
   const dim3 grid(b->sms * b->tune.blocks_per_sm), block(b->tune.block_x, b->tune.block_y);
   static const int modes[4] = {MODE_S1, MODE_S23, MODE_S23, MODE_S4};
   for (int st = first_step; st < first_step + steps; ++st)
@@ -310,12 +317,11 @@ static int batch_launch_steps(cosmos_batch b, int first_step, int steps, cudaStr
       const double* kref = b->d_kref + ((size_t)st * 4 + stage) * b->n;
       const int ns = nslot_of(&b->p);
       // stage 1 scans every instance's state; stages 2-4 take the exponents the previous
-      // stage's stage recorded
+      // stage recorded
       const cudaError_t le = stage == 0
                                  ? launch_batch_limbs(args, b->n, ns, b->p.fluid, (int*)(b->ws + b->L.expo), s)
                                  : launch_batch_to_limbs(args, b->n, ns, b->p.fluid, s);
-      if (le != cudaSuccess ||
-          launch(args, b->d_stiles, b->nstiles, kref, modes[stage], b->eq, s) != cudaSuccess)
+      if (le != cudaSuccess || launch_stage(b, args, kref, modes[stage], s) != cudaSuccess)
         return COSMOS_ECUDA;
       if (stage < 3 && launch_exponents_from_record((unsigned*)(b->ws + b->L.erec), (int*)(b->ws + b->L.expo),
                                                     b->n * ns, s) != cudaSuccess)
@@ -355,8 +361,6 @@ int cosmos_batch_run(cosmos_batch b, int first_step, int steps, int use_graph, v
 int cosmos_batch_time_stage(cosmos_batch b, int reps, double* ms_out, void* stream) {
   if (!b || reps < 1 || !ms_out) return COSMOS_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
-  BatchStageLauncher launch = b->p.fluid ? (b->p.scalar ? launch_batch_stage_fluid_scalar : launch_batch_stage_fluid)
-                                         : (b->p.scalar ? launch_batch_stage_scalar : launch_batch_stage_vac);
   const dim3 grid(b->sms * b->tune.blocks_per_sm), block(b->tune.block_x, b->tune.block_y);
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return COSMOS_ECUDA;
@@ -372,7 +376,7 @@ int cosmos_batch_time_stage(cosmos_batch b, int reps, double* ms_out, void* stre
       rc = COSMOS_ECUDA;
     if (rc == COSMOS_OK &&
         (launch_batch_limbs(b->d_args, b->n, nslot_of(&b->p), b->p.fluid, (int*)(b->ws + b->L.expo), s) != cudaSuccess ||
-         launch(b->d_args, b->d_stiles, b->nstiles, b->d_kref, MODE_S1, b->eq, s) != cudaSuccess ||
+         launch_stage(b, b->d_args, b->d_kref, MODE_S1, s) != cudaSuccess ||
          launch_exponents_from_record((unsigned*)(b->ws + b->L.erec), (int*)(b->ws + b->L.expo),
                                       b->n * nslot_of(&b->p), s) != cudaSuccess))  // leaves the record cleared
       rc = COSMOS_ECUDA;

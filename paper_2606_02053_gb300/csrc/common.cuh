@@ -169,7 +169,7 @@ cudaError_t launch_deriv_fluid(const StageArgs& a, cudaStream_t s);
 cudaError_t launch_deriv_scalar(const StageArgs& a, cudaStream_t s);
 cudaError_t launch_deriv_fluid_scalar(const StageArgs& a, cudaStream_t s);
 // batched stage over the tile list (SPLIT_TX x SPLIT_TY of one plane), K_ref per instance;
-// eq: every grid has equal spacing
+// eq: every grid of the list has equal spacing
 typedef cudaError_t (*BatchStageLauncher)(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
 cudaError_t launch_batch_stage_vac(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
 cudaError_t launch_batch_stage_fluid(const StageArgs*, const BatchTile*, long, const double*, int, bool, cudaStream_t);
