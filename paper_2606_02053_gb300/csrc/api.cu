@@ -143,6 +143,7 @@ WsLayout ws_layout(const cosmos_grid* g, const cosmos_params* p, int op) {
     L.limbs = take((size_t)nslot * fs);
     L.G = take(7 * fs);  // inverse conformal metric, 1/chi
     L.expo = take(((size_t)nslot + 1) / 2);
+    L.enext = take(((size_t)nslot + 1) / 2);  // those of the stage written, from its record
     L.erec = take(16 * (size_t)nslot);  // 32 unsigned per slot, one cache line each
     if (op == COSMOS_OP_RK4) {
       L.stageA = take(nf * fs);
@@ -380,9 +381,10 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
       s_hi = sl + 1 > s_hi ? sl + 1 : s_hi;
     }
     if (E_ext) {
-      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, E_ext, (long long*)(ws + L.limbs), ws + L.G, s));
+      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, E_ext, nullptr, (long long*)(ws + L.limbs), ws + L.G, s));
     } else if (expo_flags & 1) {  // exponents recorded by the previous stage
-      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, a.E, (long long*)(ws + L.limbs), ws + L.G, s));
+      CK(launch_to_limbs(a.g, U_s, p->fluid, s_lo, s_hi, (const int*)(ws + L.enext), (int*)(ws + L.expo),
+                         (long long*)(ws + L.limbs), ws + L.G, s));
     } else {
       CK(launch_limbs(a.g, U_s, p->fluid, s_lo, s_hi, (int*)(ws + L.expo), (long long*)(ws + L.limbs), ws + L.G, s));
     }
@@ -390,7 +392,7 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
   const int nslot = 24 + 2 * p->scalar;
   if (expo_flags & 2) {
     a.E_rec = (unsigned*)(ws + L.erec);
-    a.E_next = (int*)(ws + L.expo);
+    a.E_next = (int*)(ws + L.enext);
     if (expo_flags & 4) CK(cudaMemsetAsync(a.E_rec, 0, sizeof(unsigned) * 32 * nslot, s));
   }
   if (pass_mask & 4) CK(stage_launcher(p)(a, mode, k_cnt > 0 ? k_cnt : g->nz, s));

@@ -198,8 +198,8 @@ cudaError_t launch_init_zeta_vjp(const DevGrid& g, const Coef& c, const AlgebraP
 // conformal metric and 1/chi into G (7 fields)
 cudaError_t launch_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, int* E, long long* L,
                          double* G, cudaStream_t s);
-// the limb copy (and G) with given exponents E (no scan); the exponent scan alone
-cudaError_t launch_to_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, const int* E,
+// the limb copy (and G) with given exponents E (no scan), left in keep too unless that is null; the exponent scan alone
+cudaError_t launch_to_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, const int* E, int* keep,
                             long long* L, double* G, cudaStream_t s);
 cudaError_t launch_field_exponents(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, int* E,
                                    cudaStream_t s);

@@ -9,7 +9,7 @@ namespace cosmos {
 // Workspace sub-buffers of the single-grid calls (each 256-byte aligned), in
 // doubles from the workspace pointer; total_bytes is the size the op needs.
 struct WsLayout {
-  size_t prim, flux, stageA, stageB, acc, hm, partial, final_, limbs, G, expo, erec, scan, total_bytes;
+  size_t prim, flux, stageA, stageB, acc, hm, partial, final_, limbs, G, expo, enext, erec, scan, total_bytes;
 };
 WsLayout ws_layout(const cosmos_grid* g, const cosmos_params* p, int op);
 int check_ws(const WsLayout& L, void* ws, size_t ws_bytes);  // COSMOS_OK, EINVAL, EWORKSPACE or EALIGN
@@ -25,7 +25,8 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
               const int* E_ext = nullptr, int expo_flags = 0);
 // expo_flags (full stages of one grid): 1 = the limb copy takes the exponents left in
 // the workspace by the previous stage's record instead of scanning U_s; 2 = the stage
-// records the exponents of U_next and leaves them there; 4 = zero the record first.
+// records the exponents of U_next and leaves them there (beside those it reads, so that it
+// can be run again); 4 = zero the record first.
 // cosmos_init_grid with the gauge wave's wavelength given (Lx_wave > 0) instead
 // of the grid's own length nx h_x.
 int init_grid(const cosmos_grid* g, const cosmos_params* p, const cosmos_id* id, double* state, void* ws,

@@ -109,11 +109,13 @@ __global__ void __launch_bounds__(LIMB_THREADS) to_limbs_kernel(const DevGrid g,
   copy_slot(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride, blockIdx.x, gridDim.x);
 }
 
-// all slots below s_hi (> 6) with G
+// all slots below s_hi (> 6) with G; keep: E is left there too (null: not)
 __global__ void __launch_bounds__(LIMB_THREADS) to_limbs_all_kernel(const DevGrid g, const double* __restrict__ U,
                                                                     int s_hi, int fluid, const int* __restrict__ E,
-                                                                    long long* __restrict__ L, double* __restrict__ G) {
+                                                                    int* __restrict__ keep, long long* __restrict__ L,
+                                                                    double* __restrict__ G) {
   grid_wait();
+  if (keep && blockIdx.x == 0 && threadIdx.x < s_hi) keep[threadIdx.x] = E[threadIdx.x];
   copy_all(g, U, s_hi, fluid, E, L, G);
 }
 
@@ -159,18 +161,22 @@ cudaError_t launch_batch_limbs(const StageArgs* args, int n, int nslot, int flui
 cudaError_t launch_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, int* E, long long* L,
                          double* G, cudaStream_t s) {
   const cudaError_t e = launch_field_exponents(g, U, fluid, s_lo, s_hi, E, s);
-  return e != cudaSuccess ? e : launch_to_limbs(g, U, fluid, s_lo, s_hi, E, L, G, s);
+  return e != cudaSuccess ? e : launch_to_limbs(g, U, fluid, s_lo, s_hi, E, nullptr, L, G, s);
 }
 
 // The limb copy of slots s_lo .. s_hi - 1 with the reference exponents given
-// in E (no scan).
-cudaError_t launch_to_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, const int* E,
+// in E (no scan), which are left in keep too unless that is null.
+cudaError_t launch_to_limbs(const DevGrid& g, const double* U, int fluid, int s_lo, int s_hi, const int* E, int* keep,
                             long long* L, double* G, cudaStream_t s) {
   if (s_hi <= s_lo) return cudaSuccess;
   const unsigned blocks = copy_blocks(g);
   if (G && s_lo == 0 && s_hi > 6) {
     return launch_early(to_limbs_all_kernel, dim3(blocks * (unsigned)(LIMB_EACH + s_hi - 7)), LIMB_THREADS, 0, s, g, U,
-                        s_hi, fluid, E, L, G);
+                        s_hi, fluid, E, keep, L, G);
+  }
+  if (keep) {
+    const cudaError_t e = cudaMemcpyAsync(keep + s_lo, E + s_lo, sizeof(int) * (s_hi - s_lo), cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) return e;
   }
   if (G && s_lo <= 6 && s_hi > 6) {
     metric_kernel<<<blocks * LIMB_EACH, LIMB_THREADS, 0, s>>>(g, U, G);
