@@ -25,8 +25,11 @@
  *      then (scalar on) phi, Pi  (Pi = -n^mu d_mu phi).
  *    Padding columns i in [nx, pitch) are never read or written.
  *    Limits: nz <= 65535, ceil(ny / 4) <= 65535 and fstride < 2^31 (one
- *    field's element offsets fit in 32 bits; a state of 24 such fields
- *    would exceed the device memory anyway); else COSMOS_EINVAL.
+ *    field's element offsets fit in 32 bits); the calls that evaluate the
+ *    right-hand side or take RK4 stages (cosmos_rhs, _rk4_*, _stage_pass,
+ *    _evolve_host*, _batch_*, _fmr_step, _adjoint_step): fstride <= 2^29 (byte
+ *    offsets in 32 bits; with their buffers 79 fields of that size, 339 GB,
+ *    exceed the device memory anyway); else COSMOS_EINVAL.
  *  - Memory: every pointer named state/rhs/ws/... is DEVICE memory owned by
  *    the caller (e.g. a torch CUDA tensor), 16-byte aligned.  The library
  *    allocates no device memory in any call.  Work buffers are passed as

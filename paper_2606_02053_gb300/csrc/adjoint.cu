@@ -413,7 +413,7 @@ static int adjoint_sweep(const cosmos_grid* g, const cosmos_params* p, const dou
 
 int cosmos_adjoint_step(const cosmos_grid* g, const cosmos_params* p, const double* U_n, const double* lam_np1,
                         double* lam_n, double t, double dt, void* ws, size_t ws_bytes, void* stream) {
-  int e = check_adj(g, p);
+  int e = validate_stage(g, p);
   if (e) return e;
   if (!U_n || !lam_np1 || !lam_n || lam_n == U_n) return COSMOS_EINVAL;
   const AdjLayout L = adj_layout(g, p, COSMOS_OP_ADJOINT);

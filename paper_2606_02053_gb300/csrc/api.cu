@@ -119,6 +119,12 @@ int validate(const cosmos_grid* g, const cosmos_params* p) {
   return COSMOS_OK;
 }
 
+int validate_stage(const cosmos_grid* g, const cosmos_params* p) {
+  const int e = validate(g, p);
+  if (e) return e;
+  return (long long)g->pitch * g->ny * g->nz > (1ll << 29) ? COSMOS_EINVAL : COSMOS_OK;
+}
+
 WsLayout ws_layout(const cosmos_grid* g, const cosmos_params* p, int op) {
   const DevGrid d = make_devgrid(g);
   const size_t fs = (size_t)d.fstride;
@@ -486,7 +492,7 @@ int cosmos_init_grid(const cosmos_grid* g, const cosmos_params* p, const cosmos_
 
 int cosmos_rhs(const cosmos_grid* g, const cosmos_params* p, const double* state, double* rhs, double t, void* ws,
                size_t ws_bytes, void* stream) {
-  int e = validate(g, p);
+  int e = validate_stage(g, p);
   if (e) return e;
   if (!state || !rhs || state == rhs) return COSMOS_EINVAL;
   if (!aligned16(state) || !aligned16(rhs)) return COSMOS_EALIGN;
@@ -498,7 +504,7 @@ int cosmos_rhs(const cosmos_grid* g, const cosmos_params* p, const double* state
 
 int cosmos_rk4_stage(const cosmos_grid* g, const cosmos_params* p, int stage, const double* U_s, double* U_n,
                      double* U_next, double* acc, double t, double dt, void* ws, size_t ws_bytes, void* stream) {
-  int e = validate(g, p);
+  int e = validate_stage(g, p);
   if (e) return e;
   if (stage < 1 || stage > 4 || !U_s || !U_n || !acc) return COSMOS_EINVAL;
   if (stage < 4 && !U_next) return COSMOS_EINVAL;
@@ -527,7 +533,7 @@ int cosmos_field_exponents(const cosmos_grid* g, const cosmos_params* p, const d
 int cosmos_rk4_stage_slab(const cosmos_grid* g, const cosmos_params* p, int stage, const double* U_s, double* U_n,
                           double* U_next, double* acc, double t, double dt, int k_lo, int k_cnt, const int* E,
                           void* ws, size_t ws_bytes, void* stream) {
-  int e = validate(g, p);
+  int e = validate_stage(g, p);
   if (e) return e;
   if (stage < 1 || stage > 4 || !U_s || !U_n || !acc) return COSMOS_EINVAL;
   if (stage < 4 && !U_next) return COSMOS_EINVAL;
@@ -547,7 +553,7 @@ int cosmos_rk4_stage_slab(const cosmos_grid* g, const cosmos_params* p, int stag
 int cosmos_stage_pass(const cosmos_grid* g, const cosmos_params* p, int pass, int stage, const double* U_s,
                       double* U_n, double* U_next, double* acc, double t, double dt, void* ws, size_t ws_bytes,
                       void* stream) {
-  int e = validate(g, p);
+  int e = validate_stage(g, p);
   if (e) return e;
   const int opts = pass & ~3;
   pass &= 3;
@@ -588,7 +594,7 @@ int rk4_on(const cosmos_grid* g, const cosmos_params* p, double* state, double t
 
 int cosmos_rk4_step(const cosmos_grid* g, const cosmos_params* p, double* state, double t, double dt, void* ws,
                     size_t ws_bytes, void* stream) {
-  int e = validate(g, p);
+  int e = validate_stage(g, p);
   if (e) return e;
   if (!state) return COSMOS_EINVAL;
   if (!aligned16(state)) return COSMOS_EALIGN;
@@ -599,7 +605,7 @@ int cosmos_rk4_step(const cosmos_grid* g, const cosmos_params* p, double* state,
 
 int cosmos_rk4_step_stages(const cosmos_grid* g, const cosmos_params* p, double* state, double t, double dt,
                            double* U2, double* U3, double* U4, void* ws, size_t ws_bytes, void* stream) {
-  int e = validate(g, p);
+  int e = validate_stage(g, p);
   if (e) return e;
   if (!state || !U2 || !U3 || !U4) return COSMOS_EINVAL;
   if (U2 == state || U3 == state || U4 == state || U2 == U3 || U2 == U4 || U3 == U4) return COSMOS_EINVAL;
@@ -639,7 +645,7 @@ struct HostPipeline {
 
 int cosmos_evolve_host(const cosmos_grid* g, const cosmos_params* p, const double* host_in, double* host_out,
                        double* dev_state, int steps, double t, double dt, void* ws, size_t ws_bytes, void* stream) {
-  int e = validate(g, p);
+  int e = steps > 0 ? validate_stage(g, p) : validate(g, p);
   if (e) return e;
   if (!host_in || !host_out || !dev_state || steps < 0) return COSMOS_EINVAL;
   if (!aligned16(dev_state)) return COSMOS_EALIGN;
@@ -756,7 +762,7 @@ bool ranges_overlap(const void* a, const void* b, size_t bytes) {
 int cosmos_evolve_host_many(const cosmos_grid* g, const cosmos_params* p, int count, const double* const* host_in,
                             double* const* host_out, double* const* dev_states, int nbuf, int steps, double t,
                             double dt, void* ws, size_t ws_bytes, void* stream) {
-  int e = validate(g, p);
+  int e = steps > 0 ? validate_stage(g, p) : validate(g, p);
   if (e) return e;
   if (count < 0 || steps < 0 || nbuf < 1 || nbuf > MANY_MAX_BUF) return COSMOS_EINVAL;
   if (count == 0) return COSMOS_OK;

@@ -167,7 +167,7 @@ extern "C" {
 size_t cosmos_batch_workspace_bytes(int n, const cosmos_grid* grids, const cosmos_params* p, int max_steps) {
   if (n < 1 || !grids || !p || max_steps < 1) return 0;
   for (int i = 0; i < n; ++i)
-    if (validate(&grids[i], p) != COSMOS_OK) return 0;
+    if (validate_stage(&grids[i], p) != COSMOS_OK) return 0;
   return batch_layout(n, grids, p, max_steps).total;
 }
 
@@ -177,7 +177,7 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
   if (n < 1 || !grids || !p || !dt || !t0 || !states || max_steps < 1 || !plan_out) return COSMOS_EINVAL;
   *plan_out = nullptr;
   for (int i = 0; i < n; ++i) {
-    if (validate(&grids[i], p) != COSMOS_OK) return COSMOS_EINVAL;
+    if (validate_stage(&grids[i], p) != COSMOS_OK) return COSMOS_EINVAL;
     if (!states[i] || !(dt[i] > 0.0)) return COSMOS_EINVAL;
     if ((uintptr_t)states[i] & 15u) return COSMOS_EALIGN;
   }

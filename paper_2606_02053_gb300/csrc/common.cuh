@@ -99,6 +99,9 @@ DevGrid make_devgrid(const cosmos_grid* g);
 double K_ref(const cosmos_params* p, double t);                 // background trace at time t
 AlgebraParams algebra_params(const cosmos_params* p, double t); // runtime parameters of the algebra
 int validate(const cosmos_grid* g, const cosmos_params* p);     // COSMOS_OK or COSMOS_EINVAL
+// The same for a call that launches the stage kernel: its offsets within a field are 32-bit counts of bytes
+// (stage_split.cuh), so a field has at most 2^29 points.
+int validate_stage(const cosmos_grid* g, const cosmos_params* p);
 
 // RK4 stage modes
 enum StageMode { MODE_RHS = 0, MODE_S1 = 1, MODE_S23 = 2, MODE_S4 = 3 };

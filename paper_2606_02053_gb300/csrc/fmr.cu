@@ -461,9 +461,13 @@ int check_states(const Hier& H, double* const* states) {
   return COSMOS_OK;
 }
 
-int prepare(const cosmos_fmr* m, const cosmos_params* p, void* ws, size_t ws_bytes, cudaStream_t s, Ctx* c) {
+// stages: the call takes RK4 stages of every level
+int prepare(const cosmos_fmr* m, const cosmos_params* p, void* ws, size_t ws_bytes, cudaStream_t s, Ctx* c,
+            bool stages = false) {
   int e = describe(m, p, &c->H);
   if (e) return e;
+  for (int l = 0; stages && l < c->H.L; ++l)
+    if ((e = validate_stage(&c->H.lv[l].g, p))) return e;
   c->p = p;
   c->W = plan_ws(c->H, p);
   if (!ws) return COSMOS_EINVAL;
@@ -507,7 +511,7 @@ int cosmos_fmr_init(const cosmos_fmr* m, const cosmos_params* p, const cosmos_id
 int cosmos_fmr_step(const cosmos_fmr* m, const cosmos_params* p, double* const* states, double t, double dt0,
                     void* ws, size_t ws_bytes, void* stream) {
   Ctx c;
-  int e = prepare(m, p, ws, ws_bytes, (cudaStream_t)stream, &c);
+  int e = prepare(m, p, ws, ws_bytes, (cudaStream_t)stream, &c, true);
   if (e) return e;
   if ((e = check_states(c.H, states))) return e;
   if (!(dt0 > 0.0) || !isfinite(dt0)) return COSMOS_EINVAL;

@@ -145,9 +145,9 @@ struct SlotOut {
 };
 
 // What a difference thread needs of a tile and its instance.  Offsets are in
-// bytes within one field, 32 bits (a field of 4 GiB or more cannot be held
-// with the other fields and buffers of a stage in the device's memory): added
-// to a field's base, which is uniform, they need no 64-bit arithmetic.
+// bytes within one field, 32 bits (validate_stage refuses fields beyond 4 GiB,
+// which with the other fields and buffers of a stage exceed the device's memory):
+// added to a field's base, which is uniform, they need no 64-bit arithmetic.
 struct DiffCtx {
   const char* L;
   const char* U;
