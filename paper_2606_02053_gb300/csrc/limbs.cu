@@ -2,8 +2,7 @@
 // exponent of every limb slot, then the limb copy of the stage state.
 //
 // Both are passes over memory.  A slot is taken as one flat run of its
-// fstride values (the copy also converts what stands in the padding columns,
-// which nothing reads; the scan leaves them out), LIMB_RUN values per block and
+// fstride values (without the padding columns), LIMB_RUN values per block and
 // turn, LIMB_EACH of them in flight per thread.  By rows, a 32-point row kept half
 // of a block idle: 24 fields of 32^3: copy 15.3 -> 4.7 us, scan 33 -> 5.3; 64^3: copy
 // 50 -> 14 us; 256^3: 0.89 ms, 7.2 TB/s.  With the inverse metric and 1/chi beside it
@@ -15,6 +14,12 @@ namespace cosmos {
 
 constexpr int LIMB_THREADS = 256, LIMB_EACH = 4, LIMB_RUN = LIMB_THREADS * LIMB_EACH;
 
+// Offset p of a slot's flat run stands for a point of the grid (not for a padding column or beyond the end).
+template <bool PADDED>
+__device__ __forceinline__ bool on_grid(const DevGrid& g, long p) {
+  return p < g.fstride && !(PADDED && (unsigned)p % (unsigned)g.pitch >= (unsigned)g.nx);  // fstride < 2^31
+}
+
 // Largest biased exponent over the points of one slot, into *E (one atomic per block).
 __device__ __forceinline__ void scan_slot(const DevGrid& g, const double* __restrict__ F, unsigned* E) {
   __shared__ unsigned top[LIMB_THREADS / 32];
@@ -25,7 +30,7 @@ __device__ __forceinline__ void scan_slot(const DevGrid& g, const double* __rest
 #pragma unroll
     for (int q = 0; q < LIMB_EACH; ++q) {
       const long p = o + q * LIMB_THREADS;
-      const bool on = p < g.fstride && !(padded && (int)(p % g.pitch) >= g.nx);
+      const bool on = padded ? on_grid<true>(g, p) : on_grid<false>(g, p);
       b[q] = on ? (unsigned long long)__double_as_longlong(__ldg(F + p)) : 0ull;
     }
 #pragma unroll
@@ -40,16 +45,29 @@ __device__ __forceinline__ void scan_slot(const DevGrid& g, const double* __rest
   }
 }
 
-__device__ __forceinline__ void copy_slot(const DevGrid& g, const double* __restrict__ F, int e_ref,
-                                          long long* __restrict__ L, long first, long stride) {
+template <bool PADDED>
+__device__ __forceinline__ void copy_slot_of(const DevGrid& g, const double* __restrict__ F, int e_ref,
+                                             long long* __restrict__ L, long first, long stride) {
   for (long o = first * LIMB_RUN + threadIdx.x; o < g.fstride; o += stride * LIMB_RUN) {
     double v[LIMB_EACH];
+    bool on[LIMB_EACH];
 #pragma unroll
-    for (int q = 0; q < LIMB_EACH; ++q) v[q] = o + q * LIMB_THREADS < g.fstride ? __ldg(F + o + q * LIMB_THREADS) : 0.0;
+    for (int q = 0; q < LIMB_EACH; ++q) {
+      on[q] = on_grid<PADDED>(g, o + q * LIMB_THREADS);
+      v[q] = on[q] ? __ldg(F + o + q * LIMB_THREADS) : 0.0;
+    }
 #pragma unroll
     for (int q = 0; q < LIMB_EACH; ++q)
-      if (o + q * LIMB_THREADS < g.fstride) L[o + q * LIMB_THREADS] = to_limbs(v[q], e_ref);
+      if (on[q]) L[o + q * LIMB_THREADS] = to_limbs(v[q], e_ref);
   }
+}
+
+__device__ __forceinline__ void copy_slot(const DevGrid& g, const double* __restrict__ F, int e_ref,
+                                          long long* __restrict__ L, long first, long stride) {
+  if (g.pitch == g.nx)
+    copy_slot_of<false>(g, F, e_ref, L, first, stride);
+  else
+    copy_slot_of<true>(g, F, e_ref, L, first, stride);
 }
 
 // Limb copies of chi and the conformal metric (slots 0 .. 6) and, of the same loads, the inverse metric and
@@ -60,7 +78,9 @@ __device__ __forceinline__ void copy_metric(const DevGrid& g, const double* __re
                                             long long* __restrict__ L, double* __restrict__ G, long first, long stride) {
   const Fp64Regs k = fp64_regs();
   const long fs = g.fstride;
+  const bool padded = g.pitch != g.nx;
   for (long o = first * LIMB_THREADS + threadIdx.x; o < fs; o += stride * LIMB_THREADS) {
+    if (padded && !on_grid<true>(g, o)) continue;
     double v[7];
 #pragma unroll
     for (int m = 0; m < 7; ++m) v[m] = __ldg(U + m * fs + o);
