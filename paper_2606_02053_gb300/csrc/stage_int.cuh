@@ -65,8 +65,8 @@ __host__ __device__ __forceinline__ bool limb_odd(int e_ref) { return e_ref < 80
 constexpr int LIMB_FIT = (1 << 21) - (1 << 11);  // LIMB_FIT 2^42 + 2^51 < 2^63
 __host__ __device__ __forceinline__ bool limb_big(Limb S) { return (unsigned)(S.h + LIMB_FIT) >= 2u * LIMB_FIT; }
 
-// FP64 value (bits; round to nearest even) of the sum S times 2^(e_ref - 1085);
-// ODD = limb_odd(e_ref); ANY: also for sums with limb_big.
+// FP64 value (bits; round to nearest even) of the sum S times 2^(e_ref + twos - 1085), e_ref the
+// field's exponent (2047: it holds Inf or NaN); ODD = limb_odd(e_ref); ANY: also for sums with limb_big.
 //
 // The sum is taken into one signed 64-bit word; where it does not fit, its low 8
 // or 9 bits are dropped first, their "any set" kept in the lowest bit: at least
@@ -80,9 +80,9 @@ __host__ __device__ __forceinline__ bool limb_big(Limb S) { return (unsigned)(S.
 // large sums, taken by half the warps on data that vary along every axis, cost
 // as many again.
 template <bool ODD, bool ANY>
-__host__ __device__ __forceinline__ unsigned long long limb_bits(Limb S, int e_ref) {
+__host__ __device__ __forceinline__ unsigned long long limb_bits(Limb S, int e_ref, int twos = 0) {
   long long v = (long long)S.w;
-  int ex = e_ref;
+  int ex = e_ref + twos;
   if (ANY) {
     const long long t1 = (long long)(S.w - ((unsigned long long)(unsigned)S.h << 42));  // |t1| < 2^51
     const int ah = S.h < 0 ? -S.h : S.h;
@@ -134,23 +134,23 @@ __host__ __device__ __forceinline__ unsigned long long limb_bits(Limb S, int e_r
 }
 
 template <bool ODD>
-__device__ __forceinline__ double limb_value(Limb S, int e_ref) {
-  return __longlong_as_double((long long)limb_bits<ODD, true>(S, e_ref));
+__device__ __forceinline__ double limb_value(Limb S, int e_ref, int twos = 0) {
+  return __longlong_as_double((long long)limb_bits<ODD, true>(S, e_ref, twos));
 }
 
-// N sums of one warp (every lane takes part) at once: the form without the
-// large sums' part when no lane has one.
+// N sums of one field in one warp (every lane takes part) at once, the q-th times 2^twos[q]: the form
+// without the large sums' part when no lane has one.
 template <bool ODD, int N>
-__device__ __forceinline__ void limb_values(const Limb (&S)[N], const int (&e)[N], double (&v)[N]) {
+__device__ __forceinline__ void limb_values(const Limb (&S)[N], int e, const int (&twos)[N], double (&v)[N]) {
   unsigned top = 0;
 #pragma unroll
   for (int q = 0; q < N; ++q) top = max(top, (unsigned)(S[q].h + LIMB_FIT));
   if (__any_sync(0xffffffffu, top >= 2u * LIMB_FIT)) {
 #pragma unroll
-    for (int q = 0; q < N; ++q) v[q] = limb_value<ODD>(S[q], e[q]);
+    for (int q = 0; q < N; ++q) v[q] = limb_value<ODD>(S[q], e, twos[q]);
   } else {
 #pragma unroll
-    for (int q = 0; q < N; ++q) v[q] = __longlong_as_double((long long)limb_bits<ODD, false>(S[q], e[q]));
+    for (int q = 0; q < N; ++q) v[q] = __longlong_as_double((long long)limb_bits<ODD, false>(S[q], e, twos[q]));
   }
 }
 

@@ -284,9 +284,9 @@ struct DiffGroup {
       load(L, x, 2, n2);
       {
         const Limb S[2] = {d1, second(P1, P2, f30)};
-        const int ee[2] = {e, e + 2};
+        const int twos[2] = {0, 2};
         double v[2];
-        limb_values<ODD>(S, ee, v);
+        limb_values<ODD>(S, e, twos, v);
         dx = v[0];
         dst[0] = v[0];
         dst[3 * SPLIT_PTS] = v[1];
@@ -301,9 +301,9 @@ struct DiffGroup {
       P2 = l_add(P2, s2);
       P3 = l_add(P3, s3);
       const Limb S[3] = {yy, second(s1, s2, f30), bracket(P1, P2, P3, l_mul(f30, 2))};
-      const int ee[3] = {e + 2, e + 2, e};
+      const int twos[3] = {2, 2, 0};
       double v[3];
-      limb_values<ODD>(S, ee, v);
+      limb_values<ODD>(S, e, twos, v);
       dst[6 * SPLIT_PTS] = v[0];
       dst[8 * SPLIT_PTS] = v[1];
       ko = v[2];
@@ -314,9 +314,9 @@ struct DiffGroup {
   {                                                                             \
     axis(n##AX, d1, s1, s2, s3);                                                \
     const Limb S[3] = {d1, second(s1, s2, f30), bracket(s1, s2, s3, f20)};      \
-    const int ee[3] = {e, e + 2, e};                                            \
+    const int twos[3] = {0, 2, 0};                                              \
     double v[3];                                                                \
-    limb_values<ODD>(S, ee, v);                                                 \
+    limb_values<ODD>(S, e, twos, v);                                                 \
     if (AX == 0) dst[0] = dx = v[0];                                            \
     dst[SL * SPLIT_PTS] = v[1] * (x.r[AX] * x.r[AX]);                           \
     ko = fma(x.r[AX], v[2], ko);                                                \
@@ -333,9 +333,9 @@ struct DiffGroup {
       return l_d1(l_sub(q3(r[st]), q3(r[-st])), l_sub(q3(r[2 * st]), q3(r[-2 * st])));
     };
     const Limb S[5] = {q3(ry[0]), q3(rz[0]), mixed(ry, 1), mixed(rz, 1), mixed(rz, SPLIT_XH)};
-    const int ee[5] = {e, e, e, e, e};
+    const int twos[5] = {};
     double v[5];
-    limb_values<ODD>(S, ee, v);
+    limb_values<ODD>(S, e, twos, v);
     if (!EQ) {
       v[0] *= x.r[1];
       v[1] *= x.r[2];
@@ -383,18 +383,18 @@ struct DiffGroup {
       P2 = l_add(P2, s2);
       P3 = l_add(P3, s3);
       const Limb S[4] = {D[0], D[1], D[2], bracket(P1, P2, P3, l_mul(f0, 60))};
-      const int ee[4] = {e, e, e, e};
-      limb_values<ODD>(S, ee, v);
+      const int twos[4] = {};
+      limb_values<ODD>(S, e, twos, v);
     } else {
       const Limb f20 = l_mul(f0, 20);
-      const int ee[2] = {e, e};
+      const int twos[2] = {};
       v[3] = 0.0;
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         axis(n[d], D[d], s1, s2, s3);
         const Limb S[2] = {D[d], bracket(s1, s2, s3, f20)};
         double w[2];
-        limb_values<ODD>(S, ee, w);
+        limb_values<ODD>(S, e, twos, w);
         v[d] = w[0] * x.r[d];
         v[3] = fma(x.r[d], w[1], v[3]);
       }
