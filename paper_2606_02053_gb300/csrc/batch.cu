@@ -108,6 +108,7 @@ struct cosmos_batch_s {
   long ntiles = 0, nstiles = 0, nstiles_eq = 0;  // nstiles_eq: those of the grids with equal spacing, the first
   StageArgs* d_args = nullptr;  // [4][n]
   BatchTile* d_tiles = nullptr;
+  unsigned limb_blocks = 1;       // of the limb copy and its scan (batch_limb_blocks)
   BatchTile* d_stiles = nullptr;  // stage-kernel tiles (SPLIT_TX x SPLIT_TY of one z-plane; c = the plane)
   double* d_kref = nullptr;     // [max_steps][4][n]
   cudaGraphExec_t gexec = nullptr;
@@ -208,6 +209,7 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
   // per-stage, per-instance arguments (same fields as the single-grid stages)
   std::vector<StageArgs> args(4 * (size_t)n);
   for (int i = 0; i < n; ++i) {
+    b->limb_blocks = std::max(b->limb_blocks, batch_limb_blocks(make_devgrid(&grids[i])));
     double* A = wsd + L.A[i];
     double* B = wsd + L.B[i];
     double* acc = wsd + L.acc[i];
@@ -319,8 +321,8 @@ static int batch_launch_steps(cosmos_batch b, int first_step, int steps, cudaStr
       // stage 1 scans every instance's state; stages 2-4 take the exponents the previous
       // stage recorded
       const cudaError_t le = stage == 0
-                                 ? launch_batch_limbs(args, b->n, ns, b->p.fluid, (int*)(b->ws + b->L.expo), s)
-                                 : launch_batch_to_limbs(args, b->n, ns, b->p.fluid, s);
+                                 ? launch_batch_limbs(args, b->n, b->limb_blocks, ns, b->p.fluid, (int*)(b->ws + b->L.expo), s)
+                                 : launch_batch_to_limbs(args, b->n, b->limb_blocks, ns, b->p.fluid, s);
       if (le != cudaSuccess || launch_stage(b, args, kref, modes[stage], s) != cudaSuccess)
         return COSMOS_ECUDA;
       if (stage < 3 && launch_exponents_from_record((unsigned*)(b->ws + b->L.erec), (int*)(b->ws + b->L.expo),
@@ -375,7 +377,8 @@ int cosmos_batch_time_stage(cosmos_batch b, int reps, double* ms_out, void* stre
         launch_batch_fluid(b->d_args, b->d_tiles, b->ntiles, b->tune.mapping, b->p.w, grid, block, s) != cudaSuccess)
       rc = COSMOS_ECUDA;
     if (rc == COSMOS_OK &&
-        (launch_batch_limbs(b->d_args, b->n, nslot_of(&b->p), b->p.fluid, (int*)(b->ws + b->L.expo), s) != cudaSuccess ||
+        (launch_batch_limbs(b->d_args, b->n, b->limb_blocks, nslot_of(&b->p), b->p.fluid, (int*)(b->ws + b->L.expo), s) !=
+             cudaSuccess ||
          launch_stage(b, b->d_args, b->d_kref, MODE_S1, s) != cudaSuccess ||
          launch_exponents_from_record((unsigned*)(b->ws + b->L.erec), (int*)(b->ws + b->L.expo),
                                       b->n * nslot_of(&b->p), s) != cudaSuccess))  // leaves the record cleared

@@ -208,11 +208,13 @@ cudaError_t launch_field_exponents(const DevGrid& g, const double* U, int fluid,
                                    cudaStream_t s);
 // E[s] = rec[32 s] and rec[32 s] = 0 for s < nslot (the exponents a stage recorded)
 cudaError_t launch_exponents_from_record(unsigned* rec, int* E, int nslot, cudaStream_t s);
-// the batched limb copy with the exponents already in args[i].E
-cudaError_t launch_batch_to_limbs(const StageArgs* args, int n, int nslot, int fluid, cudaStream_t s);
+// the batched limb copy with the exponents already in args[i].E; blocks: batch_limb_blocks of the instance with most points
+unsigned batch_limb_blocks(const DevGrid& largest);
+cudaError_t launch_batch_to_limbs(const StageArgs* args, int n, unsigned blocks, int nslot, int fluid, cudaStream_t s);
 // the same for every instance of a batch (args[i] = instance i's stage arguments;
 // E_all = the n x nslot exponents, contiguous, args[i].E = E_all + i nslot)
-cudaError_t launch_batch_limbs(const StageArgs* args, int n, int nslot, int fluid, int* E_all, cudaStream_t s);
+cudaError_t launch_batch_limbs(const StageArgs* args, int n, unsigned blocks, int nslot, int fluid, int* E_all,
+                               cudaStream_t s);
 
 // fluid.cu
 cudaError_t launch_fluid_prim(const DevGrid& g, const double* U, double* prim, double w, cudaStream_t s);
