@@ -71,8 +71,8 @@ def face_flux(d: int):
     a factor 1/4), the inverse metric is never formed (gamma^ij = k c_ij with the
     cofactors c_ij of the doubled metric), reciprocals come in pairs from one
     division, and with s = alpha v^d - beta the fluxes are F_E = E s + alpha P v^d,
-    F_i = J_i s + alpha P delta_id.  The two speeds of a side, (A +- R) - beta with
-    R >= 0, have the largest modulus |A - beta| + R.  A flux is antisymmetric
+    F_i = J_i s + alpha P delta_id.  The two speeds of a side, (A +- R) - beta,
+    have the largest modulus |A - beta| + |R| (R has the sign of the lapse).  A flux is antisymmetric
     bitwise under the exchange of its sides (with the odd components negated):
     what the sides contribute meets only in sums of two rounded terms (mulr)."""
     g = Graph()
@@ -114,7 +114,7 @@ def face_flux(d: int):
         aP = aw * rho
         F.append([E * s + aP * vd] + [J[i] * s + aP if i == d else mulr(J[i], s) for i in range(3)])
         disc = one_v2 * (gdd * one_wv2 - omw * (vd * vd))
-        speed.append(fabs((pre * omw) * vd - beta2) + (pre * sqw) * sqrt(disc))
+        speed.append(fabs((pre * omw) * vd - beta2) + fabs(pre * sqw) * sqrt(disc))
     a = fmax(speed[0], speed[1])
     out = [hs * ((F[0][m] + F[1][m]) - a * (U[1][m] - U[0][m])) for m in range(4)]
     return g, names, out
