@@ -26,9 +26,9 @@ static int nin_of(const cosmos_params* p) {
 }
 
 // Forward stage and reverse launchers of the matter variant.
-static cudaError_t launch_stage_for(const cosmos_params* p, const StageArgs& a, int mode, int k_cnt, cudaStream_t s) {
-  if (p->fluid) return p->scalar ? launch_stage_fluid_scalar(a, mode, k_cnt, s) : launch_stage_fluid(a, mode, k_cnt, s);
-  return p->scalar ? launch_stage_scalar(a, mode, k_cnt, s) : launch_stage_vac(a, mode, k_cnt, s);
+static cudaError_t launch_stage_for(const cosmos_params* p, const StageArgs& a, int mode, cudaStream_t s) {
+  if (p->fluid) return p->scalar ? launch_stage_fluid_scalar(a, mode, s) : launch_stage_fluid(a, mode, s);
+  return p->scalar ? launch_stage_scalar(a, mode, s) : launch_stage_vac(a, mode, s);
 }
 
 static cudaError_t launch_deriv_for(const cosmos_params* p, const StageArgs& a, cudaStream_t s) {
@@ -192,7 +192,8 @@ static cudaError_t fwd_stage(const cosmos_grid* g, const cosmos_params* p, const
   }
   const cudaError_t e = limbs_of(p, a.g, U_s, ws, L, a, ws + L.G, s);
   if (e != cudaSuccess) return e;
-  return launch_stage_for(p, a, MODE_S1, g->nz, s);
+  a.k_hi = g->nz;
+  return launch_stage_for(p, a, MODE_S1, s);
 }
 
 // Compaction: per-block partial histograms over shells k = floor(sqrt(m)) + 1,

@@ -325,7 +325,7 @@ __global__ void fp64_fma_chains(double* __restrict__ out, int iters, double a, d
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
-typedef cudaError_t (*StageLauncher)(const StageArgs&, int, int, cudaStream_t);
+typedef cudaError_t (*StageLauncher)(const StageArgs&, int, cudaStream_t);
 typedef cudaError_t (*ConstraintLauncher)(const ConstraintArgs&, cudaStream_t);
 
 static StageLauncher stage_launcher(const cosmos_params* p) {
@@ -353,6 +353,7 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
   StageArgs a;
   memset(&a, 0, sizeof(a));
   a.k_lo = k_lo;
+  a.k_hi = k_cnt > 0 ? k_lo + k_cnt : g->nz;
   a.g = make_devgrid(g);
   a.c = make_coef(g, p->ko_sigma);
   a.ap = algebra_params(p, t_stage);
@@ -401,7 +402,7 @@ int run_stage(const cosmos_grid* g, const cosmos_params* p, int mode, const doub
     a.E_next = (int*)(ws + L.enext);
     if (expo_flags & 4) CK(cudaMemsetAsync(a.E_rec, 0, sizeof(unsigned) * 32 * nslot, s));
   }
-  if (pass_mask & 4) CK(stage_launcher(p)(a, mode, k_cnt > 0 ? k_cnt : g->nz, s));
+  if (pass_mask & 4) CK(stage_launcher(p)(a, mode, s));
   return COSMOS_OK;
 }
 

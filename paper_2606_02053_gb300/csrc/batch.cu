@@ -55,10 +55,8 @@ struct BatchLayout {
 // limb slots (stage_int.cuh)
 static int nslot_of(const cosmos_params* p) { return 24 + 2 * p->scalar; }
 
-// SPLIT_TX x SPLIT_TY tiles of every plane: the work list of the stage kernel
-static long stage_tiles(const cosmos_grid& g) {
-  return (long)((g.nx + SPLIT_TX - 1) / SPLIT_TX) * ((g.ny + SPLIT_TY - 1) / SPLIT_TY) * g.nz;
-}
+// the work list of the stage kernel
+static long stage_tiles(const cosmos_grid& g) { return stage_tiles(make_devgrid(&g), g.nz); }
 
 static BatchLayout batch_layout(int n, const cosmos_grid* grids, const cosmos_params* p, int max_steps) {
   BatchLayout L;
@@ -96,6 +94,9 @@ static BatchLayout batch_layout(int n, const cosmos_grid* grids, const cosmos_pa
 
 using namespace cosmos;
 
+// Form of the stage kernel that an instance takes: + 2 unequal spacing, + 1 thin tiles.
+static int stage_kind(const StageArgs& a) { return (a.eq ? 0 : 2) + (thin_tiles(a.g) ? 1 : 0); }
+
 struct cosmos_batch_s {
   int n = 0;
   cosmos_params p;
@@ -105,11 +106,11 @@ struct cosmos_batch_s {
   int sms = 0;
   char* ws = nullptr;
   BatchLayout L;
-  long ntiles = 0, nstiles = 0, nstiles_eq = 0;  // nstiles_eq: those of the grids with equal spacing, the first
+  long ntiles = 0, stiles[5] = {};  // stiles: bounds of the four kinds' stage-kernel tiles (stage_kind)
   StageArgs* d_args = nullptr;  // [4][n]
   BatchTile* d_tiles = nullptr;
   unsigned limb_blocks = 1;       // of the limb copy and its scan (batch_limb_blocks)
-  BatchTile* d_stiles = nullptr;  // stage-kernel tiles (SPLIT_TX x SPLIT_TY of one z-plane; c = the plane)
+  BatchTile* d_stiles = nullptr;  // stage-kernel tiles (b: their rows, c: the plane, or the row of y where they are thin)
   double* d_kref = nullptr;     // [max_steps][4][n]
   cudaGraphExec_t gexec = nullptr;
   int g_first = -1, g_steps = -1;
@@ -229,6 +230,7 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
       a.out = outs[s];
       a.acc = acc;
       a.cdt = cdt[s];
+      a.k_hi = grids[i].nz;
       set_units(&a, p->ko_sigma, 2.0);
       a.L = (const long long*)(wsd + L.limbs[i]);
       a.G = wsd + L.G[i];
@@ -261,21 +263,20 @@ int cosmos_batch_plan(int n, const cosmos_grid* grids, const cosmos_params* p, c
   {
     // Tiles instance by instance, plane by plane: the blocks of the persistent
     // stage kernel then work on neighbouring planes of one grid, whose z-stencils
-    // share their planes in L2.  The grids with equal spacing come first: the stage
+    // share their planes in L2.  Grids of one kind stand together: the stage
     // kernel's forms for equal and unequal spacing round the dissipation differently,
     // and each instance takes that of cosmos_rk4_step on its own grid.
     std::vector<BatchTile> st;
-    for (int eq = 1; eq >= 0; --eq) {
+    for (int kind = 0; kind < 4; ++kind) {
       for (int i = 0; i < n; ++i) {
         const cosmos_grid& g = grids[i];
-        if (args[i].eq != eq) continue;
-        const int tx = (g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = (g.ny + SPLIT_TY - 1) / SPLIT_TY;
+        if (stage_kind(args[i]) != kind) continue;
+        const int tx = (g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = ((kind & 1 ? g.nz : g.ny) + SPLIT_TY - 1) / SPLIT_TY;
         for (long w = 0; w < stage_tiles(g); ++w)
           st.push_back(BatchTile{i, (int)(w % tx), (int)((w / tx) % ty), (int)(w / ((long)tx * ty))});
       }
-      if (eq) b->nstiles_eq = (long)st.size();
+      b->stiles[kind + 1] = (long)st.size();
     }
-    b->nstiles = (long)st.size();
     if (cudaMemcpy(b->d_stiles, st.data(), sizeof(BatchTile) * st.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
       delete b;
       return COSMOS_ECUDA;
@@ -297,14 +298,17 @@ int cosmos_batch_set_tuning(cosmos_batch b, const cosmos_batch_tuning* tuning) {
   return upload_tiles(b);
 }
 
-// The stage kernel over every instance: the tiles of the grids with equal spacing, then the others.
+// The stage kernel over every instance, kind by kind.
 static cudaError_t launch_stage(cosmos_batch b, const StageArgs* args, const double* kref, int mode, cudaStream_t s) {
   const BatchStageLauncher launch =
       b->p.fluid ? (b->p.scalar ? launch_batch_stage_fluid_scalar : launch_batch_stage_fluid)
                  : (b->p.scalar ? launch_batch_stage_scalar : launch_batch_stage_vac);
-  const cudaError_t e = launch(args, b->d_stiles, b->nstiles_eq, kref, mode, true, s);
-  if (e != cudaSuccess) return e;
-  return launch(args, b->d_stiles + b->nstiles_eq, b->nstiles - b->nstiles_eq, kref, mode, false, s);
+  for (int kind = 0; kind < 4; ++kind) {
+    const long lo = b->stiles[kind], count = b->stiles[kind + 1] - lo;
+    const cudaError_t e = launch(args, b->d_stiles + lo, count, kref, mode, kind < 2, kind & 1, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 static int batch_launch_steps(cosmos_batch b, int first_step, int steps, cudaStream_t s) {

@@ -245,10 +245,10 @@ __global__ void __launch_bounds__(BX* BY, 2) constraint_kernel(const ConstraintA
       alg_##NAME::constraints(in, out, p, k);                                                                     \
     }                                                                                                           \
   };                                                                                                            \
-  cudaError_t launch_stage_##NAME(const StageArgs& a, int mode, int k_cnt, cudaStream_t s) {                        \
+  cudaError_t launch_stage_##NAME(const StageArgs& a, int mode, cudaStream_t s) {                                   \
     if (!a.L) return cudaErrorInvalidValue; /* the differences are those of the limb copy */                        \
-    const long tiles = (long)((a.g.nx + SPLIT_TX - 1) / SPLIT_TX) * ((a.g.ny + SPLIT_TY - 1) / SPLIT_TY) * k_cnt;   \
-    return launch_split<T_##NAME, false>(a, nullptr, nullptr, tiles, nullptr, mode, a.eq, s);                             \
+    const long tiles = stage_tiles(a.g, a.k_hi - a.k_lo);                                                           \
+    return launch_split<T_##NAME, false>(a, nullptr, nullptr, tiles, nullptr, mode, a.eq, thin_tiles(a.g), s);      \
   }                                                                                                                 \
   cudaError_t launch_deriv_##NAME(const StageArgs& a, cudaStream_t s) {                                             \
     if (!a.L) return cudaErrorInvalidValue;                                                                         \
@@ -259,10 +259,10 @@ __global__ void __launch_bounds__(BX* BY, 2) constraint_kernel(const ConstraintA
     return cudaGetLastError();                                                                                      \
   }                                                                                                                 \
   cudaError_t launch_batch_stage_##NAME(const StageArgs* args, const BatchTile* tiles, long ntiles,                 \
-                                        const double* kref, int mode, bool eq, cudaStream_t s) {                             \
+                                        const double* kref, int mode, bool eq, bool thin, cudaStream_t s) {         \
     StageArgs none;                                                                                                 \
     memset(&none, 0, sizeof(none));                                                                                 \
-    return launch_split<T_##NAME, true>(none, args, tiles, ntiles, kref, mode, eq, s);                                  \
+    return launch_split<T_##NAME, true>(none, args, tiles, ntiles, kref, mode, eq, thin, s);                        \
   }                                                                                                                 \
   cudaError_t launch_constraints_##NAME(const ConstraintArgs& a, cudaStream_t s) {                              \
     constraint_kernel<T_##NAME><<<point_grid(a.g), dim3(BX, BY), 0, s>>>(a);                                    \

@@ -124,7 +124,9 @@ constexpr size_t split_smem_bytes() {
          sizeof(int) * (SPLIT_GROUPS * (48 + 32) + 32);
 }
 
-// Tile w of the plane range of one grid, or of a batch's tile list.
+// Tile w of the plane range of one grid, or of a batch's tile list: SPLIT_TX points along x from i0,
+// SPLIT_TY rows along y from j0 at plane k of z, or (THIN, thin_tiles in common.cuh) along z from j0 at
+// row k of y.
 struct SplitTile {
   int i0, j0, k, inst;
 };
@@ -166,8 +168,10 @@ __device__ __forceinline__ double ldd(const char* __restrict__ base, unsigned o)
   return __ldg(reinterpret_cast<const double*>(base + o));
 }
 
-template <class T, bool EQ>
+// Axes of a tile: 0 = x, 1 = that of its rows, 2 = the third.  Slots are by the grid's axes.
+template <class T, bool EQ, bool THIN>
 struct DiffGroup {
+  static constexpr int ROW = THIN ? 2 : 1, OUT = THIN ? 1 : 2;  // grid axes of tile axes 1 and 2, and the reverse
   const int t;     // thread of the group = point of the tile
   const int g;     // group
   double* sA;      // region A + t
@@ -187,15 +191,15 @@ struct DiffGroup {
     if (t < SPLIT_NXW)
       xw[t] = 8u * (unsigned)wrap_index(w.i0 - 3 + t, a.g.nx);
     else if (t < SPLIT_NXW + SPLIT_NYW)
-      xw[t] = row * (unsigned)wrap_index(w.j0 - 3 + t - SPLIT_NXW, a.g.ny);
+      xw[t] = (THIN ? plane : row) * (unsigned)wrap_index(w.j0 - 3 + t - SPLIT_NXW, THIN ? a.g.nz : a.g.ny);
     else if (t < SPLIT_NXW + SPLIT_NYW + SPLIT_NZW)
-      xw[t] = plane * (unsigned)wrap_index(w.k - 3 + t - SPLIT_NXW - SPLIT_NYW, a.g.nz);
+      xw[t] = (THIN ? row : plane) * (unsigned)wrap_index(w.k - 3 + t - SPLIT_NXW - SPLIT_NYW, THIN ? a.g.ny : a.g.nz);
     else if (t >= 64 && t < 64 + NSLOT)
       ex[t - 64] = max(a.E[t - 64], 1);
     sync();
     const unsigned *yw = xw + SPLIT_NXW, *zw = yw + SPLIT_NYW;
     // threads past the edge take the last column / row: their results are not stored
-    const int tx = min(t % SPLIT_TX, a.g.nx - 1 - w.i0), ty = min(t / SPLIT_TX, a.g.ny - 1 - w.j0);
+    const int tx = min(t % SPLIT_TX, a.g.nx - 1 - w.i0), ty = min(t / SPLIT_TX, (THIN ? a.g.nz : a.g.ny) - 1 - w.j0);
     const unsigned cx = xw[tx + 3], cy = yw[ty + 3], cz = zw[3];
     x.c = cx + cy + cz;
     x.o[0] = cy + cz;
@@ -215,7 +219,7 @@ struct DiffGroup {
     x.fb = 8 * a.g.fstride;
     if (!EQ) {
 #pragma unroll
-      for (int d = 0; d < 3; ++d) x.r[d] = a.ratio[d];
+      for (int d = 0; d < 3; ++d) x.r[d] = a.ratio[d == 0 ? 0 : (d == 1 ? ROW : OUT)];
     }
   }
 
@@ -254,7 +258,7 @@ struct DiffGroup {
   template <bool ODD>
   __device__ __forceinline__ void d2_slots(const DiffCtx& x, const char* __restrict__ L, int e, double kos,
                                            const double* b, double* dst) const {
-    // D_y and D_z sums of the tile with their halos; every load in flight before the first use
+    // sums along tile axes 1 and 2 with their halos; every load in flight before the first use
     long long r[4][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -304,8 +308,8 @@ struct DiffGroup {
       const int twos[3] = {2, 2, 0};
       double v[3];
       limb_values<ODD>(S, e, twos, v);
-      dst[6 * SPLIT_PTS] = v[0];
-      dst[8 * SPLIT_PTS] = v[1];
+      dst[(THIN ? 8 : 6) * SPLIT_PTS] = v[0];
+      dst[(THIN ? 6 : 8) * SPLIT_PTS] = v[1];
       ko = v[2];
     } else {
       const Limb f20 = l_mul(f0, 20);
@@ -321,9 +325,15 @@ struct DiffGroup {
     dst[SL * SPLIT_PTS] = v[1] * (x.r[AX] * x.r[AX]);                           \
     ko = fma(x.r[AX], v[2], ko);                                                \
   }
+      // in the order of the grid's axes: ko is a rounded sum
       COSMOS_SPLIT_AXIS(0, 3)
-      COSMOS_SPLIT_AXIS(1, 6)
-      COSMOS_SPLIT_AXIS(2, 8)
+      if constexpr (THIN) {
+        COSMOS_SPLIT_AXIS(2, 6)
+        COSMOS_SPLIT_AXIS(1, 8)
+      } else {
+        COSMOS_SPLIT_AXIS(1, 6)
+        COSMOS_SPLIT_AXIS(2, 8)
+      }
 #undef COSMOS_SPLIT_AXIS
     }
     sync();
@@ -343,13 +353,13 @@ struct DiffGroup {
       v[3] *= x.r[2];
       v[4] *= x.r[1] * x.r[2];
     }
-    dst[1 * SPLIT_PTS] = v[0];
-    dst[2 * SPLIT_PTS] = v[1];
-    dst[4 * SPLIT_PTS] = v[2];
-    dst[5 * SPLIT_PTS] = v[3];
+    dst[ROW * SPLIT_PTS] = v[0];
+    dst[OUT * SPLIT_PTS] = v[1];
+    dst[(3 + ROW) * SPLIT_PTS] = v[2];
+    dst[(3 + OUT) * SPLIT_PTS] = v[3];
     dst[7 * SPLIT_PTS] = v[4];
     double m = kos * ko;
-    if (b) m = fma(b[0], dx, fma(b[SPLIT_PTS], v[0], fma(b[2 * SPLIT_PTS], v[1], m)));
+    if (b) m = fma(b[0], dx, fma(b[SPLIT_PTS], v[ROW - 1], fma(b[2 * SPLIT_PTS], v[OUT - 1], m)));
     dst[9 * SPLIT_PTS] = m;
     sync();
   }
@@ -382,7 +392,7 @@ struct DiffGroup {
       P1 = l_add(P1, s1);
       P2 = l_add(P2, s2);
       P3 = l_add(P3, s3);
-      const Limb S[4] = {D[0], D[1], D[2], bracket(P1, P2, P3, l_mul(f0, 60))};
+      const Limb S[4] = {D[0], D[ROW], D[OUT], bracket(P1, P2, P3, l_mul(f0, 60))};
       const int twos[4] = {};
       limb_values<ODD>(S, e, twos, v);
     } else {
@@ -390,13 +400,14 @@ struct DiffGroup {
       const int twos[2] = {};
       v[3] = 0.0;
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        axis(n[d], D[d], s1, s2, s3);
+      for (int d = 0; d < 3; ++d) {  // grid axis, u that of the tile
+        const int u = d == 0 ? 0 : (d == 1 ? ROW : OUT);
+        axis(n[u], D[d], s1, s2, s3);
         const Limb S[2] = {D[d], bracket(s1, s2, s3, f20)};
         double w[2];
         limb_values<ODD>(S, e, twos, w);
-        v[d] = w[0] * x.r[d];
-        v[3] = fma(x.r[d], w[1], v[3]);
+        v[d] = w[0] * x.r[u];
+        v[3] = fma(x.r[u], w[1], v[3]);
       }
     }
   }
@@ -518,11 +529,11 @@ struct DiffGroup {
   template <int G>
   __device__ __forceinline__ void combine(const StageArgs& a, int mode, const SplitTile& w) const {
     using S = Slots<T>;
-    const int i = w.i0 + t % SPLIT_TX, j = w.j0 + t / SPLIT_TX;
-    const bool valid = i < a.g.nx && j < a.g.ny;
+    const int i = w.i0 + t % SPLIT_TX, j = THIN ? w.k : w.j0 + t / SPLIT_TX, k = THIN ? w.j0 + t / SPLIT_TX : w.k;
+    const bool valid = i < a.g.nx && (THIN ? k < a.k_hi : j < a.g.ny);
     const long fb = 8 * a.g.fstride;
     const unsigned row = 8u * (unsigned)a.g.pitch, plane = row * (unsigned)a.g.ny;
-    const unsigned c = valid ? plane * (unsigned)w.k + row * (unsigned)j + 8u * (unsigned)i : 0u;
+    const unsigned c = valid ? plane * (unsigned)k + row * (unsigned)j + 8u * (unsigned)i : 0u;
     const bool add = mode == MODE_S23 || mode == MODE_S4;
     const char* const u0 = mode == MODE_S4 ? reinterpret_cast<const char*>(a.U0w) : reinterpret_cast<const char*>(a.U0);
     char* const acc = reinterpret_cast<char*>(a.acc);
@@ -542,7 +553,7 @@ struct DiffGroup {
     if (T::FLUID) {
       const unsigned cx = c - 8u * (unsigned)i + 8u * (unsigned)wrap_index(i - 1, a.g.nx);
       const unsigned cy = c + row * (unsigned)(wrap_index(j - 1, a.g.ny) - j);
-      const unsigned cz = c + plane * (unsigned)(wrap_index(w.k - 1, a.g.nz) - w.k);
+      const unsigned cz = c + plane * (unsigned)(wrap_index(k - 1, a.g.nz) - k);
 #pragma unroll
       for (int q = 0; q < NFL; ++q)
 #pragma unroll
@@ -598,56 +609,28 @@ struct DiffGroup {
   }
 };
 
-// BATCH: tiles from a list, arguments per instance with K_ref in kref; else
-// the planes k_lo .. of the grid of `one`.
-template <class T, bool BATCH, bool EQ>
-__global__ void __launch_bounds__(SPLIT_THREADS, 1)
-    split_stage_kernel(const __grid_constant__ StageArgs one, const StageArgs* __restrict__ args,
-                       const BatchTile* __restrict__ tiles, long ntiles, const double* __restrict__ kref, int mode) {
-  extern __shared__ double smem[];
-  using S = Slots<T>;
-  double* const A = smem;
-  double* const B = smem + S::A * SPLIT_PTS;
-  int4* const stage = reinterpret_cast<int4*>(B + S::B * SPLIT_PTS);
-  int* const tables = reinterpret_cast<int*>(stage + SPLIT_GROUPS * (SPLIT_NDY + SPLIT_NDZ));
-  int* const rec = tables + SPLIT_GROUPS * 80;
+// The difference warps' part of the kernel below (its arguments; t: point of the tile).
+template <class T, bool BATCH, bool EQ, bool THIN>
+__device__ __forceinline__ void difference_warps(const StageArgs& one, const StageArgs* __restrict__ args,
+                                                 const BatchTile* __restrict__ tiles, long ntiles,
+                                                 const double* __restrict__ kref, int mode, int t, double* A, double* B,
+                                                 int4* stage, int* tables, int* rec) {
   constexpr int NSLOT = 24 + (T::SCALAR ? 2 : 0);
-  if (threadIdx.x < 32) rec[threadIdx.x] = 0;
-  grid_wait();
-  __syncthreads();
-  const int t = threadIdx.x % SPLIT_PTS;
-  const int tx = (one.g.nx + SPLIT_TX - 1) / SPLIT_TX, ty = (one.g.ny + SPLIT_TY - 1) / SPLIT_TY;
+  const int tx = (one.g.nx + SPLIT_TX - 1) / SPLIT_TX;
+  const int ty = ((THIN ? one.k_hi - one.k_lo : one.g.ny) + SPLIT_TY - 1) / SPLIT_TY;
   auto tile_at = [&](long w) {
     if (BATCH) {
       const BatchTile b = tiles[w];
       return SplitTile{b.a * SPLIT_TX, b.b * SPLIT_TY, b.c, b.inst};
     }
     const int q = (int)w;  // tiles of one grid: less than 2^31
-    return SplitTile{q % tx * SPLIT_TX, q / tx % ty * SPLIT_TY, q / (tx * ty) + one.k_lo, 0};
+    const int j0 = q / tx % ty * SPLIT_TY, k = q / (tx * ty);
+    return SplitTile{q % tx * SPLIT_TX, THIN ? j0 + one.k_lo : j0, THIN ? k : k + one.k_lo, 0};
   };
-  if (threadIdx.x < SPLIT_PTS) {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SPLIT_REG_ALG));
-    const Fp64Regs k = fp64_regs();
-    for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
-      const bool more = w + gridDim.x < ntiles;
-      AlgebraParams ap = one.ap;
-      if (BATCH) ap = args[tiles[w].inst].ap;
-      bar_sync(BAR_FULL_A, SPLIT_THREADS);
-      T::rhs_split(SlotIn{A + t}, SlotIn{B + t}, SlotOut<T>{B + t},
-                   [&] {
-                     if (more) bar_arrive(BAR_FREE_A, SPLIT_THREADS);
-                     bar_sync(BAR_FULL_B, SPLIT_THREADS);
-                   },
-                   ap, k);
-      bar_arrive(BAR_DONE_B, SPLIT_THREADS);
-    }
-    return;
-  }
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SPLIT_REG_DIFF));
   const int g = __shfl_sync(0xffffffffu, (int)threadIdx.x / SPLIT_PTS - 1, 0);  // uniform, and known to be
   int* const tab = tables + g * 80;
   int4* const st = stage + g * (SPLIT_NDY + SPLIT_NDZ);
-  const DiffGroup<T, EQ> d{t, g, A + t, B + t, st, reinterpret_cast<unsigned*>(tab), tab + 48, rec};
+  const DiffGroup<T, EQ, THIN> d{t, g, A + t, B + t, st, reinterpret_cast<unsigned*>(tab), tab + 48, rec};
   auto flush = [&](const StageArgs& a) {  // the record of the instance that ends here
     bar_sync(BAR_DIFF, SPLIT_THREADS - SPLIT_PTS);
     if (g == 0 && t < NSLOT && a.E_rec && mode != MODE_RHS && mode != MODE_S4) {
@@ -693,8 +676,47 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   }
 }
 
+// BATCH: tiles from a list, arguments per instance with K_ref in kref; else
+// the planes k_lo .. of the grid of `one`.  THIN: tiles along z, of every grid.
+template <class T, bool BATCH, bool EQ, bool THIN>
+__global__ void __launch_bounds__(SPLIT_THREADS, 1)
+    split_stage_kernel(const __grid_constant__ StageArgs one, const StageArgs* __restrict__ args,
+                       const BatchTile* __restrict__ tiles, long ntiles, const double* __restrict__ kref, int mode) {
+  extern __shared__ double smem[];
+  using S = Slots<T>;
+  double* const A = smem;
+  double* const B = smem + S::A * SPLIT_PTS;
+  int4* const stage = reinterpret_cast<int4*>(B + S::B * SPLIT_PTS);
+  int* const tables = reinterpret_cast<int*>(stage + SPLIT_GROUPS * (SPLIT_NDY + SPLIT_NDZ));
+  int* const rec = tables + SPLIT_GROUPS * 80;
+  if (threadIdx.x < 32) rec[threadIdx.x] = 0;
+  grid_wait();
+  __syncthreads();
+  const int t = threadIdx.x % SPLIT_PTS;
+  if (threadIdx.x < SPLIT_PTS) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SPLIT_REG_ALG));
+    const Fp64Regs k = fp64_regs();
+    for (long w = blockIdx.x; w < ntiles; w += gridDim.x) {
+      const bool more = w + gridDim.x < ntiles;
+      AlgebraParams ap = one.ap;
+      if (BATCH) ap = args[tiles[w].inst].ap;
+      bar_sync(BAR_FULL_A, SPLIT_THREADS);
+      T::rhs_split(SlotIn{A + t}, SlotIn{B + t}, SlotOut<T>{B + t},
+                   [&] {
+                     if (more) bar_arrive(BAR_FREE_A, SPLIT_THREADS);
+                     bar_sync(BAR_FULL_B, SPLIT_THREADS);
+                   },
+                   ap, k);
+      bar_arrive(BAR_DONE_B, SPLIT_THREADS);
+    }
+    return;
+  }
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SPLIT_REG_DIFF));
+  difference_warps<T, BATCH, EQ, THIN>(one, args, tiles, ntiles, kref, mode, t, A, B, stage, tables, rec);
+}
+
 // One block per SM, no more than there are tiles.
-template <class T, bool BATCH, bool EQ>
+template <class T, bool BATCH, bool EQ, bool THIN>
 cudaError_t launch_split_as(const StageArgs& one, const StageArgs* args, const BatchTile* tiles, long ntiles,
                             const double* kref, int mode, cudaStream_t s) {
   int dev = 0, sms = 0;
@@ -703,20 +725,23 @@ cudaError_t launch_split_as(const StageArgs& one, const StageArgs* args, const B
   constexpr size_t bytes = split_smem_bytes<T>();
   static_assert(bytes <= 232448, "shared memory of one block");
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(split_stage_kernel<T, BATCH, EQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    e = cudaFuncSetAttribute(split_stage_kernel<T, BATCH, EQ, THIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   const int blocks = (int)(ntiles < sms ? ntiles : sms);
-  return launch_early(split_stage_kernel<T, BATCH, EQ>, dim3(blocks), SPLIT_THREADS, bytes, s, one, args, tiles, ntiles,
+  return launch_early(split_stage_kernel<T, BATCH, EQ, THIN>, dim3(blocks), SPLIT_THREADS, bytes, s, one, args, tiles, ntiles,
                       kref, mode);
 }
 
-// eq: equal spacing (of every grid of a batch)
+// eq: equal spacing, thin: tiles along z (of every grid of a batch)
 template <class T, bool BATCH>
 cudaError_t launch_split(const StageArgs& one, const StageArgs* args, const BatchTile* tiles, long ntiles,
-                         const double* kref, int mode, bool eq, cudaStream_t s) {
+                         const double* kref, int mode, bool eq, bool thin, cudaStream_t s) {
   if (ntiles <= 0) return cudaSuccess;
-  return eq ? launch_split_as<T, BATCH, true>(one, args, tiles, ntiles, kref, mode, s)
-            : launch_split_as<T, BATCH, false>(one, args, tiles, ntiles, kref, mode, s);
+  if (thin)
+    return eq ? launch_split_as<T, BATCH, true, true>(one, args, tiles, ntiles, kref, mode, s)
+              : launch_split_as<T, BATCH, false, true>(one, args, tiles, ntiles, kref, mode, s);
+  return eq ? launch_split_as<T, BATCH, true, false>(one, args, tiles, ntiles, kref, mode, s)
+            : launch_split_as<T, BATCH, false, false>(one, args, tiles, ntiles, kref, mode, s);
 }
 
 }  // namespace cosmos
