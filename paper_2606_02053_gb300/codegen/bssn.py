@@ -29,9 +29,9 @@ grouped for few FP64 instructions (a multiply that feeds one add is free):
 factors 1/2 and 2 are folded into quantities formed once, the equal terms of
 diagonal components are formed once, terms that one tensor multiplies are
 summed before it does, and what the trace-free projection removes is not
-formed.  Vacuum: 817 FP64 instructions per point (765 products, 651 sums)
-against 973 for the textbook grouping, fluid 939 against 1148, reverse mode
-2117 against 2480, constraints 571 against 777; a 256^3 vacuum RK4 step went
+formed.  Vacuum: 803 multiply-adds per point (753 products, 633 sums)
+against 973 for the textbook grouping, fluid 925 against 1148, reverse mode
+2071 against 2480, constraints 556 against 777; a 256^3 vacuum RK4 step went
 from 169.0 to 153.3 ms and a 128^3 fluid one from 39.1 to 36.3 ms.  The stage
 kernel's form (inverse metric, 1/chi and the advection formed elsewhere) has 718
 in vacuum, 840 with the fluid.

@@ -50,7 +50,7 @@ def render() -> dict:
         g, L, out = bssn.algebra(fluid, scalar)
         c = op_counts(g, out)
         stats.append((name, c))
-        body.append(f"// variant {name}: fluid={int(fluid)} scalar={int(scalar)}; ops {dict(sorted(c.items()))}")
+        body.append(f"// variant {name}: fluid={int(fluid)} scalar={int(scalar)}; graph ops {dict(sorted(c.items()))}")
         body.append(f"namespace alg_{name} {{")
         body.append(f"constexpr int NF = {L['nf']};")
         body.append(f"constexpr int ND1 = {len(L['d1'])};")
@@ -60,10 +60,13 @@ def render() -> dict:
         body.append(_table_fn("d2_field", L["d2"]))
         body.append(_slot_fn("d1_slot", L["d1"]))
         body.append(_slot_fn("d2_slot", L["d2"]))
-        body.append(emit_function(g, "rhs", L["names"], out, ["AlgebraParams"], accessors=True))
+        if name == "vac":  # no kernel calls it
+            body.append("// the right-hand side as one function: the form that the host checks run statement by statement")
+            body.append(emit_function(g, "rhs", L["names"], out, ["AlgebraParams"], accessors=True))
         gs, S, outs = bssn.algebra(fluid, scalar, split=True)
         body.append("// the right-hand side in two phases (codegen/bssn.py, split_layout); the slots of its inputs\n"
                     "// in regions A and B, and of its outputs in B")
+        body.append(f"// variant {name}, two phases: ops {dict(sorted(op_counts(gs, outs).items()))}")
         body.append(f"constexpr int SA = {len(S['a'])}, SB = {len(S['b'])};")
         body.append(f"constexpr bool SPLIT_EARLY = {str(S['early']).lower()};  // At among the states of region A")
         body.append(_table_fn("out_slot", S["out"]))

@@ -125,15 +125,9 @@ __device__ __forceinline__ void gather(const double* __restrict__ U, const doubl
   if constexpr (T::FLUID) in[T::NIN - 1] = ldg(prim, n.c);
 }
 
-constexpr int TXH = BX + 4;  // tile width with the x halo
-
 template <class T>
 __device__ __forceinline__ int ko_slot(int f) {
   return (T::FLUID && f >= 28) ? f - 4 : f;
-}
-
-__device__ __forceinline__ long plane_off(const DevGrid& g, int x, int y, int k) {
-  return ((long)wrap_index(k, g.nz) * g.ny + wrap_index(y, g.ny)) * g.pitch + wrap_index(x, g.nx);
 }
 
 }  // namespace cosmos
