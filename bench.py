@@ -47,22 +47,23 @@ COMBINE_FLOPS = [2, 4, 4, 3]
 # Reported scaled to the bench grid by points; null when the kernel sources differ
 # from the profiled ones.
 NCU_TRAFFIC = {"sources_sha256_16": "84f7160269938728", "points": 96 ** 3, "bytes_per_launch": {"stage": 1035.1e6}}
-KERNEL_SOURCES = ["common.cuh", "stage_kernel.cuh", "stage_split.cuh", "stage_int.cuh", "limbs.cu", "stage_vac.cu",
+KERNEL_SOURCES = ["common.cuh", "fp64_regs.cuh", "stage_kernel.cuh", "stage_split.cuh", "stage_int.cuh", "limbs.cu", "stage_vac.cu",
                   "generated/bssn_algebra.cuh"]
 
 
 def generated_algebra_ops(variant="vac"):
-    """Operation count of the generated pointwise algebra of a matter variant
-    (the expression DAG after common-subexpression elimination: every named
-    intermediate and every symmetric tensor component formed once), read from
-    the comment the code generator writes into the generated header."""
+    """Operation count of the generated algebra that the stage kernel of a matter variant
+    runs (the two-phase form's expression DAG after common-subexpression elimination:
+    every named intermediate and every symmetric tensor component formed once; without
+    the inverse metric, 1/chi and the advection), read from the comment the code generator
+    writes into the generated header."""
     import ast
     import re
 
     path = os.path.join(ROOT, "paper_2606_02053_gb300", "csrc", "generated", "bssn_algebra.cuh")
     with open(path) as fh:
         for line in fh:
-            m = re.match(r"// variant (\w+): .* ops (\{.*\})", line)
+            m = re.match(r"// variant (\w+), two phases: ops (\{.*\})", line)
             if m and m.group(1) == variant:
                 return sum(ast.literal_eval(m.group(2)).values())
     raise RuntimeError("no operation count for variant " + variant)
@@ -990,10 +991,10 @@ def main():
         parts = cpu["flops_parts"]
         fl = lambda d: d["add"] + d["mul"] + d["div"] + d["sqrt"]  # noqa: E731
         combine = statistics.mean(COMBINE_FLOPS) * STATE_FIELDS
-        # stage kernel: the generated algebra's operations + the KO multiply-add (2 per field) + the RK4
+        # stage kernel: the generated algebra's operations + advection and dissipation of every field (7) + the RK4
         # combine; its finite differences are integer work.  Beside it the oracle's count (its plain
         # loops form every symmetric component twice) and its stencils as FP64 operations.
-        alg_flops = generated_algebra_ops("vac") + 2 * STATE_FIELDS + combine
+        alg_flops = generated_algebra_ops("vac") + 7 * STATE_FIELDS + combine
         oracle_flops = {"stencils": fl(parts["derivatives"]) + fl(parts["ko"]), "algebra": fl(parts["algebra"]) + combine}
         # the state read, its limb copy, inverse metric and 1/chi written; these read and the stage's states
         bytes_point = {"limbs": 8 * (2 * STATE_FIELDS + 7),
@@ -1007,7 +1008,7 @@ def main():
                 "traffic_note": "bytes per launch, ncu small-case capture scaled by points",
                 "kernel": "stage kernel (split_stage_kernel<T_vac>): differences, algebra and combine",
                 "avg_launch_ms": 1e3 * avg["stage"], "algorithmic_flops_per_point": alg_flops,
-                "flops_note": "generated algebra after CSE + KO multiply-add + RK4 combine, on the FP64 pipe",
+                "flops_note": "generated algebra after CSE + advection and dissipation + RK4 combine, on the FP64 pipe",
                 "oracle_flops_per_point": oracle_flops["algebra"],
                 "stencil_flops_per_point_fp64_equivalent": oracle_flops["stencils"],
                 "stencil_arithmetic": "exact integer (fixed point), beside the FP64 pipe",
