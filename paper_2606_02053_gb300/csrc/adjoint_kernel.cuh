@@ -66,7 +66,8 @@ struct VjpOut {
 constexpr int VJP_THREADS = 32;
 
 #ifndef COSMOS_VJP_MIN_BLOCKS
-#define COSMOS_VJP_MIN_BLOCKS 3  // reverse algebra: resident 128-thread blocks per SM the registers are sized for
+// reverse algebra: the registers are sized for 3 x 128 resident threads per SM (12 of its blocks of VJP_THREADS)
+#define COSMOS_VJP_MIN_BLOCKS 3
 #endif
 
 template <class T>
