@@ -139,6 +139,7 @@ static cudaError_t vjp_once(const cosmos_grid* g, const cosmos_params* p, const 
   d.c = a.c;
   d.U = U;
   d.D = ws + L.Dfw;
+  d.dfs = d.g.fstride;
   a.D = d.D;
   {
     cudaError_t e = limbs_of(p, d.g, U, ws, L, d, nullptr, s);

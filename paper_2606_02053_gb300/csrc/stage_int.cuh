@@ -257,9 +257,9 @@ __device__ __forceinline__ Limb id1(const long long* __restrict__ L, const NbrI&
 // First derivatives of a field that has no second ones.
 template <class T, bool ODD>
 __device__ __forceinline__ void ideriv_d1_point(const StageArgs& a, int m, const NbrI& n, int e) {
-  const long fs = a.g.fstride;
+  const long fs = a.dfs;
   const int s = ko_slot<T>(T::d1_field(m));
-  const long long* Lf = a.L + (long)s * fs;
+  const long long* Lf = a.L + (long)s * a.g.fstride;
   double* __restrict__ D = a.D + (long)(3 * m) * fs + n.c;
   D[0] = limb_value<ODD>(id1<0>(Lf, n), e) * a.c.d1b[0];
   D[fs] = limb_value<ODD>(id1<1>(Lf, n), e) * a.c.d1b[1];
@@ -272,12 +272,12 @@ template <class T, bool ODD>
 __device__ __forceinline__ void ideriv_d2_point(const StageArgs& a, int m2, const NbrI& n, int e, int tx, int ty,
                                                 const int4* __restrict__ sDy, const int4* __restrict__ sDz) {
   constexpr int TXH = BX + 4;
-  const long fs = a.g.fstride;
+  const long fs = a.dfs;
   const Coef& c = a.c;
   double* __restrict__ D = a.D;
   const int f = T::d2_field(m2);
   const int s = ko_slot<T>(f);
-  const long long* Lf = a.L + (long)s * fs;
+  const long long* Lf = a.L + (long)s * a.g.fstride;
   const int m1 = T::d1_slot(f);
   const long b = (long)(3 * T::ND1 + 6 * m2) * fs + n.c;
   const Limb f30 = l_mul(ldl(Lf, n.c), 30);
