@@ -45,9 +45,10 @@ __device__ __forceinline__ void scan_slot(const DevGrid& g, const double* __rest
   }
 }
 
+// PADDED: pitch > nx
 template <bool PADDED>
-__device__ __forceinline__ void copy_slot_of(const DevGrid& g, const double* __restrict__ F, int e_ref,
-                                             long long* __restrict__ L, long first, long stride) {
+__device__ __forceinline__ void copy_slot(const DevGrid& g, const double* __restrict__ F, int e_ref,
+                                          long long* __restrict__ L, long first, long stride) {
   for (long o = first * LIMB_RUN + threadIdx.x; o < g.fstride; o += stride * LIMB_RUN) {
     double v[LIMB_EACH];
     bool on[LIMB_EACH];
@@ -62,25 +63,17 @@ __device__ __forceinline__ void copy_slot_of(const DevGrid& g, const double* __r
   }
 }
 
-__device__ __forceinline__ void copy_slot(const DevGrid& g, const double* __restrict__ F, int e_ref,
-                                          long long* __restrict__ L, long first, long stride) {
-  if (g.pitch == g.nx)
-    copy_slot_of<false>(g, F, e_ref, L, first, stride);
-  else
-    copy_slot_of<true>(g, F, e_ref, L, first, stride);
-}
-
 // Limb copies of chi and the conformal metric (slots 0 .. 6) and, of the same loads, the inverse metric and
 // 1/chi of each point into G: blocks first, first + stride, .. of LIMB_THREADS points.  The stage's algebra
 // has one warp per scheduler, which the latency of the determinant and its reciprocal bounds; here many warps
 // are in flight and the FP64 instructions run beside the copies of the other slots, whose bound is memory.
+template <bool PADDED>
 __device__ __forceinline__ void copy_metric(const DevGrid& g, const double* __restrict__ U, const int* __restrict__ E,
                                             long long* __restrict__ L, double* __restrict__ G, long first, long stride) {
   const Fp64Regs k = fp64_regs();
   const long fs = g.fstride;
-  const bool padded = g.pitch != g.nx;
   for (long o = first * LIMB_THREADS + threadIdx.x; o < fs; o += stride * LIMB_THREADS) {
-    if (padded && !on_grid<true>(g, o)) continue;
+    if (PADDED && !on_grid<true>(g, o)) continue;
     double v[7];
 #pragma unroll
     for (int m = 0; m < 7; ++m) v[m] = __ldg(U + m * fs + o);
@@ -102,15 +95,16 @@ __device__ __forceinline__ void copy_metric(const DevGrid& g, const double* __re
 // Work of one block in a pass over all slots below s_hi (> 6) with G: of every LIMB_EACH + s_hi - 7 blocks, the
 // first LIMB_EACH take LIMB_RUN points of chi and the metric, the others LIMB_RUN points of one slot each, so
 // that the two kinds are on an SM together.
+template <bool PADDED>
 __device__ __forceinline__ void copy_all(const DevGrid& g, const double* __restrict__ U, int s_hi, int fluid,
                                          const int* __restrict__ E, long long* __restrict__ L, double* __restrict__ G) {
   const int each = LIMB_EACH + s_hi - 7, q = blockIdx.x % each;
   const long c = blockIdx.x / each, nc = gridDim.x / each;
   if (q < LIMB_EACH) {
-    copy_metric(g, U, E, L, G, c * LIMB_EACH + q, nc * LIMB_EACH);
+    copy_metric<PADDED>(g, U, E, L, G, c * LIMB_EACH + q, nc * LIMB_EACH);
   } else {
     const int s = 7 + q - LIMB_EACH;
-    copy_slot(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride, c, nc);
+    copy_slot<PADDED>(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride, c, nc);
   }
 }
 
@@ -122,27 +116,31 @@ __global__ void __launch_bounds__(LIMB_THREADS) field_exponent_kernel(const DevG
   scan_slot(g, U + (long)limb_field(s, fluid) * g.fstride, (unsigned*)E + s);
 }
 
+template <bool PADDED>
 __global__ void __launch_bounds__(LIMB_THREADS) to_limbs_kernel(const DevGrid g, const double* __restrict__ U, int s_lo,
                                                                 int fluid, const int* __restrict__ E,
                                                                 long long* __restrict__ L) {
   const int s = s_lo + blockIdx.y;
-  copy_slot(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride, blockIdx.x, gridDim.x);
+  copy_slot<PADDED>(g, U + (long)limb_field(s, fluid) * g.fstride, max(E[s], 1), L + (long)s * g.fstride, blockIdx.x,
+                    gridDim.x);
 }
 
 // all slots below s_hi (> 6) with G; keep: E is left there too (null: not)
+template <bool PADDED>
 __global__ void __launch_bounds__(LIMB_THREADS) to_limbs_all_kernel(const DevGrid g, const double* __restrict__ U,
                                                                     int s_hi, int fluid, const int* __restrict__ E,
                                                                     int* __restrict__ keep, long long* __restrict__ L,
                                                                     double* __restrict__ G) {
   grid_wait();
   if (keep && blockIdx.x == 0 && threadIdx.x < s_hi) keep[threadIdx.x] = E[threadIdx.x];
-  copy_all(g, U, s_hi, fluid, E, L, G);
+  copy_all<PADDED>(g, U, s_hi, fluid, E, L, G);
 }
 
 // G alone
+template <bool PADDED>
 __global__ void __launch_bounds__(LIMB_THREADS) metric_kernel(const DevGrid g, const double* __restrict__ U,
                                                               double* __restrict__ G) {
-  copy_metric(g, U, nullptr, nullptr, G, blockIdx.x, gridDim.x);
+  copy_metric<PADDED>(g, U, nullptr, nullptr, G, blockIdx.x, gridDim.x);
 }
 
 // The same for a batch: blockIdx.z = instance; the arguments of instance i are
@@ -158,7 +156,10 @@ __global__ void __launch_bounds__(LIMB_THREADS) batch_to_limbs_kernel(const Stag
                                                                       int fluid) {
   grid_wait();
   const StageArgs& a = args[blockIdx.y];
-  copy_all(a.g, a.U, nslot, fluid, a.E, const_cast<long long*>(a.L), const_cast<double*>(a.G));
+  if (a.g.pitch == a.g.nx)
+    copy_all<false>(a.g, a.U, nslot, fluid, a.E, const_cast<long long*>(a.L), const_cast<double*>(a.G));
+  else
+    copy_all<true>(a.g, a.U, nslot, fluid, a.E, const_cast<long long*>(a.L), const_cast<double*>(a.G));
 }
 
 // Blocks along a slot: the copy has no turn to repeat up to the largest grids;
@@ -198,20 +199,22 @@ cudaError_t launch_to_limbs(const DevGrid& g, const double* U, int fluid, int s_
                             long long* L, double* G, cudaStream_t s) {
   if (s_hi <= s_lo) return cudaSuccess;
   const unsigned blocks = copy_blocks(g);
+  const bool padded = g.pitch != g.nx;  // kernels of their own: with the test in one, the unpadded copy took 3% longer
   if (G && s_lo == 0 && s_hi > 6) {
-    return launch_early(to_limbs_all_kernel, dim3(blocks * (unsigned)(LIMB_EACH + s_hi - 7)), LIMB_THREADS, 0, s, g, U,
-                        s_hi, fluid, E, keep, L, G);
+    return launch_early(padded ? to_limbs_all_kernel<true> : to_limbs_all_kernel<false>,
+                        dim3(blocks * (unsigned)(LIMB_EACH + s_hi - 7)), LIMB_THREADS, 0, s, g, U, s_hi, fluid, E, keep, L, G);
   }
   if (keep) {
     const cudaError_t e = cudaMemcpyAsync(keep + s_lo, E + s_lo, sizeof(int) * (s_hi - s_lo), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return e;
   }
   if (G && s_lo <= 6 && s_hi > 6) {
-    metric_kernel<<<blocks * LIMB_EACH, LIMB_THREADS, 0, s>>>(g, U, G);
+    (padded ? metric_kernel<true> : metric_kernel<false>)<<<blocks * LIMB_EACH, LIMB_THREADS, 0, s>>>(g, U, G);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  to_limbs_kernel<<<dim3(blocks, (unsigned)(s_hi - s_lo)), LIMB_THREADS, 0, s>>>(g, U, s_lo, fluid, E, L);
+  (padded ? to_limbs_kernel<true> : to_limbs_kernel<false>)<<<dim3(blocks, (unsigned)(s_hi - s_lo)), LIMB_THREADS, 0, s>>>(
+      g, U, s_lo, fluid, E, L);
   return cudaGetLastError();
 }
 
