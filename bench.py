@@ -46,7 +46,7 @@ COMBINE_FLOPS = [2, 4, 4, 3]
 # capture of a small case, and the hash of the kernel sources it was taken on.
 # Reported scaled to the bench grid by points; null when the kernel sources differ
 # from the profiled ones.
-NCU_TRAFFIC = {"sources_sha256_16": "d71c26db6fffd91f", "points": 96 ** 3, "bytes_per_launch": {"stage": 910.2e6}}
+NCU_TRAFFIC = {"sources_sha256_16": "379b226a59744c27", "points": 96 ** 3, "bytes_per_launch": {"stage": 910.5e6}}
 KERNEL_SOURCES = ["common.cuh", "fp64_regs.cuh", "stage_kernel.cuh", "stage_split.cuh", "stage_int.cuh", "limbs.cu", "stage_vac.cu",
                   "generated/bssn_algebra.cuh"]
 
